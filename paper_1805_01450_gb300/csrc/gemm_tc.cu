@@ -4,8 +4,8 @@
 // (work item, b): with A = Ar + i Ai and B = Br + i Bi,
 //   [Re C[m, n], Im C[m, n]] = [Ar | Ai][m, :]  times  [[Br, Bi], [-Bi, Br]][:, (n, re/im)],
 // i.e. the left factor's real summed index is (part p, k) with part 0 = Ar and part 1 = Ai,
-// and the right factor has two real columns per complex column n: 2n = (Br; -Bi) and
-// 2n + 1 = (Bi; Br). Every real operand x is split into three bf16 parts x = h + m + l (8
+// and the right factor has two real columns per complex column n: (Br; -Bi) for Re and
+// (Bi; Br) for Im (a tile's Re columns first, then its Im columns). Every real operand x is split into three bf16 parts x = h + m + l (8
 // significant bits each: h = rn(x), m = rn(x - h), l = rn(x - h - m)), and the six products
 // h*h + h*m + m*h + h*l + l*h + m*m are accumulated in FP32; the dropped terms (m*l, l*m,
 // l*l) are below 2^-23 of the product. Two parts with three products (about 2^-16 per
@@ -14,7 +14,7 @@
 //
 // The row role goes to the operand that holds C's lowest mode, so tensor-memory lane i (row
 // m = i of a 128-row tile) holds C entries that are consecutive in memory along the lanes;
-// the real columns 2n and 2n + 1 of a lane are Re and Im of C[m, n], so the epilogue stores
+// a lane's Re column and Im column n are the two parts of C[m, n], so the epilogue stores
 // complex64 values straight from the registers tcgen05.ld fills, coalesced across the warp,
 // with no transpose. A tile is 128 complex rows by NT real (NT / 2 complex, up to 128)
 // columns of one (item, b). The kernel is persistent (one CTA per SM walks the tiles) and
@@ -50,8 +50,19 @@ constexpr uint32_t kPolls = 1u << 22;
 constexpr uint32_t kEpiThreads = 256;  // eight epilogue warps, two per tensor-memory lane quarter
 
 __host__ __device__ constexpr uint32_t region_bytes(uint32_t rows) { return rows / 8u * kPitch; }
-// One stage: A regions (part 0 h, m, l, part 1 h, m, l), then the same for B.
-__host__ __device__ constexpr uint32_t stage_bytes(uint32_t nt) { return 6u * region_bytes(kRows) + 6u * region_bytes(nt); }
+// One chunk of B: per bf16 level three consecutive blocks of NT / 2 rows, [-Bi][Br][Bi]. The
+// real columns of a tile are all its Re columns, then all its Im columns, so part 0 of the
+// right factor is the two blocks [Br][Bi] and part 1 the two blocks [-Bi][Br]: a descriptor
+// that starts one block earlier, and Br is stored once. With Re and Im interleaved column by
+// column a level took four blocks: 48 instead of 36 KB of stores per chunk of a 256-column
+// tile, whose loop is bound by shared-memory traffic. Together with one barrier arrival per
+// warp (warp_arrive) the streaming steps of a 64-qubit circuit went from 2.90 to 2.56 ms (64
+// summed entries, 190 -> 215 algorithmic TFLOP/s) and from 1.52 to 1.21 ms (32 summed, 128
+// columns).
+__host__ __device__ constexpr uint32_t b_block_bytes(uint32_t nt) { return region_bytes(nt / 2u); }
+__host__ __device__ constexpr uint32_t b_chunk_bytes(uint32_t nt) { return 9u * b_block_bytes(nt); }
+// One stage: A regions (part 0 h, m, l, part 1 h, m, l), then a chunk of B.
+__host__ __device__ constexpr uint32_t stage_bytes(uint32_t nt) { return 6u * region_bytes(kRows) + b_chunk_bytes(nt); }
 
 // Producer threads: one per operand unit of a chunk (8 summed entries of one A row or one
 // complex B column): 128 rows x 2 halves of A and NT / 2 columns x 2 halves of B (threads
@@ -60,17 +71,17 @@ template <int NT>
 __host__ __device__ constexpr uint32_t producers() { return 256u + ((uint32_t)NT < 32u ? 32u : (uint32_t)NT); }
 template <int NT>
 __host__ __device__ constexpr uint32_t block_threads() { return producers<NT>() + 32u + kEpiThreads; }
-// Operand stages of the shared-memory ring: two for 128- and 256-column tiles (52 and 77 KB),
+// Operand stages of the shared-memory ring: two for 128- and 256-column tiles (46 and 65 KB),
 // three below.
 template <int NT>
 __host__ __device__ constexpr uint32_t n_stages() { return NT >= 128 ? 2u : 3u; }
 // Raw copy slots per producer (chunks in flight): four, two for 256-column tiles (their
-// 512 producers' slots and two 77 KB stages fill the shared memory).
+// 512 producers' slots and two 65 KB stages leave no room for a third).
 template <int NT>
 __host__ __device__ constexpr uint32_t raw_depth() { return NT >= 256 ? 2u : 4u; }
-// real accumulator columns an epilogue warp reads at a time
+// complex columns an epilogue warp reads at a time (the same number of Re and Im columns)
 template <int NT>
-__host__ __device__ constexpr uint32_t epi_cols() { return NT < 32 ? (uint32_t)NT : 32u; }
+__host__ __device__ constexpr uint32_t epi_cols() { return NT >= 64 ? 16u : 8u; }
 // raw copy slot: 8 complex64 entries per producer thread, entry j of thread t at j * P + t
 template <int NT>
 __host__ __device__ constexpr uint32_t raw_slot_bytes() { return 8u * producers<NT>() * 8u; }
@@ -165,10 +176,29 @@ __device__ __forceinline__ void store_a(unsigned char *sa, const float2 *v, uint
     }
 }
 
-// Complex B column n of one summed half in the six B regions: real column 2n takes Br in
-// part 0 and -Bi in part 1, real column 2n + 1 takes Bi in part 0 and Br in part 1.
+// Complex B column n of one summed half in the nine blocks of a chunk (level q: -Bi, Br, Bi).
 template <int NT>
 __device__ __forceinline__ void store_b(unsigned char *sb, const float2 *v, uint32_t n, uint32_t h) {
+    constexpr uint32_t R = b_block_bytes(NT);
+    uint32_t re[3][4], im[3][4];
+    split8(v, re, im);
+    unsigned char *o = sb + core_offset(n, h);
+#pragma unroll
+    for (uint32_t q = 0; q < 3; q++) {
+        *reinterpret_cast<uint4 *>(o + 3u * q * R) =
+            make_uint4(im[q][0] ^ 0x80008000u, im[q][1] ^ 0x80008000u, im[q][2] ^ 0x80008000u, im[q][3] ^ 0x80008000u);
+        *reinterpret_cast<uint4 *>(o + (3u * q + 1u) * R) = make_uint4(re[q][0], re[q][1], re[q][2], re[q][3]);
+        *reinterpret_cast<uint4 *>(o + (3u * q + 2u) * R) = make_uint4(im[q][0], im[q][1], im[q][2], im[q][3]);
+    }
+}
+
+// Complex B column n of one summed half in the six B regions: real column 2n takes Br in
+// part 0 and -Bi in part 1, real column 2n + 1 takes Bi in part 0 and Br in part 1 (the
+// B-stationary form: B is stored once per column tile, and its epilogue reads the (Re, Im)
+// column pairs with one tensor-memory load; with Re and Im in two halves its largest step took
+// 7.1 instead of 6.5 ms).
+template <int NT>
+__device__ __forceinline__ void store_b_interleaved(unsigned char *sb, const float2 *v, uint32_t n, uint32_t h) {
     constexpr uint32_t R = region_bytes(NT);
     uint32_t re[3][4], im[3][4];
     split8(v, re, im);
@@ -186,6 +216,14 @@ __device__ __forceinline__ void store_b(unsigned char *sb, const float2 *v, uint
     }
 }
 
+// Arrival of a warp whose lanes have each written (and, for operand stages, fenced) their
+// share: one per warp; an arrival of every thread serialised hundreds of updates of one
+// barrier word per chunk.
+__device__ __forceinline__ void warp_arrive(uint32_t bar) {
+    __syncwarp();
+    if ((threadIdx.x & 31u) == 0u) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 __device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -193,10 +231,35 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// kW Re columns and kW Im columns of this warp's 32 tensor-memory lanes into registers (one
+// column per register), waited for.
+template <uint32_t kW>
+__device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, uint32_t (&r)[kW]) {
+    if constexpr (kW == 16) {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+            "%12, %13, %14, %15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(taddr));
+    } else {
+        static_assert(kW == 8, "8 or 16 columns");
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "r"(taddr));
+    }
+}
+template <uint32_t kW>
+__device__ __forceinline__ void tmem_ld(uint32_t re_addr, uint32_t im_addr, uint32_t (&re)[kW], uint32_t (&im)[kW]) {
+    tmem_ld_issue<kW>(re_addr, re);
+    tmem_ld_issue<kW>(im_addr, im);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 // kW accumulator columns of this warp's 32 tensor-memory lanes into registers (one column
 // per register), waited for.
 template <uint32_t kW>
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[kW]) {
+__device__ __forceinline__ void tmem_ld_pairs(uint32_t taddr, uint32_t (&r)[kW]) {
     if constexpr (kW == 32) {
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
@@ -243,6 +306,12 @@ __device__ __forceinline__ bool wait_or_fail(uint32_t bar, uint32_t parity, vola
         if ((i & 63u) == 63u && *fail) return false;
     }
     return false;
+}
+
+// The same for a whole warp, with one answer for all its lanes: the roles' loops contain
+// warp-wide operations, so their lanes must leave them together.
+__device__ __forceinline__ bool warp_wait_or_fail(uint32_t bar, uint32_t parity, volatile int *fail) {
+    return __all_sync(0xffffffffu, wait_or_fail(bar, parity, fail));
 }
 
 struct TileCoord {
@@ -314,7 +383,7 @@ struct BsCursor {
 //              tile's last chunk to the accumulator's "full" barrier;
 //   8 warps    epilogue: wait for an accumulator, read it with tcgen05.ld (warp w reads
 //              tensor-memory lanes 32 (w mod 4) ..., i.e. rows 32 (w mod 4) + lane; the two
-//              warps of a lane quarter take alternate blocks of 32 columns), store each
+//              warps of a lane quarter take alternate blocks of complex columns), store each
 //              (Re, Im) column pair as one complex64 entry of C and release the accumulator.
 //              Four warps left the epilogue about a tenth slower on output-heavy steps: each
 //              waits out its tensor-memory reads block by block.
@@ -343,12 +412,12 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
     const uint32_t sbase = smem_u32(gsm);
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < S; s++) {
-            mbar_init(smem_u32(&full_bar[s]), P);
+            mbar_init(smem_u32(&full_bar[s]), P / 32u);
             mbar_init(smem_u32(&empty_bar[s]), 1);
         }
         for (uint32_t b = 0; b < 2; b++) {
             mbar_init(smem_u32(&accf_bar[b]), 1);
-            mbar_init(smem_u32(&acce_bar[b]), kEpiThreads);
+            mbar_init(smem_u32(&acce_bar[b]), kEpiThreads / 32u);
         }
         mbar_init(smem_u32(&drain_bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -423,11 +492,11 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
         const uint64_t my_tiles = (ga.n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
         const uint64_t total = my_tiles * ga.n_chunks;
         for (uint32_t i = 0; i + 1 < kRaw; i++) issue_next(i);
-        for (uint64_t gc = 0; gc < total && !fail; gc++) {
+        for (uint64_t gc = 0; gc < total; gc++) {
             issue_next(gc + kRaw - 1);
             cp_async_wait<kRaw - 1>();   // this thread's copies of chunk gc have landed
             const uint32_t s = (uint32_t)(gc % S);
-            if (!wait_or_fail(smem_u32(&empty_bar[s]), (uint32_t)((gc / S) & 1u) ^ 1u, &fail)) {
+            if (!warp_wait_or_fail(smem_u32(&empty_bar[s]), (uint32_t)((gc / S) & 1u) ^ 1u, &fail)) {
                 fail = 1;
                 break;
             }
@@ -442,14 +511,14 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
             }
             // the generic-proxy stores must be visible to the tensor cores' reads
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_bar[s])) : "memory");
+            warp_arrive(smem_u32(&full_bar[s]));
         }
         cp_async_wait<0>();   // no copy may still be landing when the CTA leaves
     } else if (warp == kMmaWarp) {
         if (lane == 0) {   // MMA issuer
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) |
                                    ((kRows >> 4) << 24);
-            constexpr uint32_t kRegB = region_bytes(NT);
+            constexpr uint32_t kBlkB = b_block_bytes(NT);
             uint64_t gc = 0;
             uint32_t j = 0;
             for (uint64_t t = blockIdx.x; t < ga.n_tiles && !fail; t += gridDim.x, j++) {
@@ -475,7 +544,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
 #pragma unroll
                         for (uint32_t q = 0; q < 3; q++) {
                             ad[q] = smem_desc(sa + (3u * p + q) * kRegA, 128u, kPitch);
-                            bd[q] = smem_desc(sb + (3u * p + q) * kRegB, 128u, kPitch);
+                            bd[q] = smem_desc(sb + (3u * q + 1u - p) * kBlkB, 128u, kPitch);
                         }
                         // h*h, h*m, m*h, h*l, l*h, m*m
                         mma_bf16(d, ad[0], bd[0], idesc, (c | p) != 0u);
@@ -500,39 +569,39 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
         __syncwarp();
     } else {
         // epilogue: warp w reads tensor-memory lanes 32q ... 32q + 31 (q = w mod 4): row
-        // m = mt*128 + 32q + lane of the tile, whose real columns 2j and 2j + 1 are Re and Im
-        // of C[m, nt*NT/2 + j]. For each column the warp's 32 stores are 32 rows, consecutive
+        // m = mt*128 + 32q + lane of the tile, whose columns j and NT/2 + j are Re and Im of
+        // C[m, nt*NT/2 + j]. For each column the warp's 32 stores are 32 rows, consecutive
         // in C when its lowest modes are row modes (the planner gives the row role to the
         // operand that holds C's lowest mode).
         const uint32_t q = warp & 3u;
         const uint32_t share = (warp - kMmaWarp - 1u) >> 2;   // the two warps of a lane quarter split its columns
         uint32_t j = 0;
-        for (uint64_t t = blockIdx.x; t < ga.n_tiles && !fail; t += gridDim.x, j++) {
+        for (uint64_t t = blockIdx.x; t < ga.n_tiles; t += gridDim.x, j++) {
             const TileCoord tc = tile_coord(t, ga);
             const uint32_t buf = j & 1u;
             // this lane's row of C and the tile's base, while the MMAs run
             float2 *Crow = ga.arenas + (uint64_t)tc.il * ga.a.arena_elems + g.c_off + pext_runs(tc.beta, g.cb, g.n_cb) +
                            pext_runs(tc.mt * kRows + 32u * q + lane, g.cm, g.n_cm);
-            if (!wait_or_fail(smem_u32(&accf_bar[buf]), (j >> 1) & 1u, &fail)) {
+            if (!warp_wait_or_fail(smem_u32(&accf_bar[buf]), (j >> 1) & 1u, &fail)) {
                 fail = 1;
                 break;
             }
             tc_fence_after();
             const uint32_t taddr = tmem + ((q * 32u) << 16) + buf * kCols;
-            for (uint32_t j0 = share * kW; j0 < (uint32_t)NT; j0 += 2u * kW) {
-                // the column offsets of this block's kW / 2 complex columns, one per lane
-                const uint32_t my_col = pext_runs(tc.nt * kNc + j0 / 2u + (lane % (kW / 2u)), g.cn, g.n_cn);
-                uint32_t r[kW];
-                tmem_ld<kW>(taddr + j0, r);
+            for (uint32_t j0 = share * kW; j0 < kNc; j0 += 2u * kW) {
+                // the column offsets of this block's kW complex columns, one per lane
+                const uint32_t my_col = pext_runs(tc.nt * kNc + j0 + (lane % kW), g.cn, g.n_cn);
+                uint32_t re[kW], im[kW];
+                tmem_ld<kW>(taddr + j0, taddr + kNc + j0, re, im);
 #pragma unroll
-                for (uint32_t i = 0; i < kW / 2u; i++) {
+                for (uint32_t i = 0; i < kW; i++) {
                     const uint32_t coff = __shfl_sync(0xffffffffu, my_col, i);
-                    Crow[coff] = make_float2(__uint_as_float(r[2u * i]), __uint_as_float(r[2u * i + 1u]));
+                    Crow[coff] = make_float2(__uint_as_float(re[i]), __uint_as_float(im[i]));
                 }
             }
             // the accumulator's reads are done: the MMAs of the tile after next may reuse it
             tc_fence_before();
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acce_bar[buf])) : "memory");
+            warp_arrive(smem_u32(&acce_bar[buf]));
         }
     }
     tc_fence_before();
@@ -564,6 +633,9 @@ __host__ __device__ constexpr uint32_t bs_accs() { return 512u / bs_cols<NT>() <
 __host__ __device__ constexpr uint32_t bs_stage_bytes() { return 6u * region_bytes(kRows); }
 template <int NT>
 __host__ __device__ constexpr uint32_t bs_b_bytes() { return 6u * region_bytes(NT); }   // one chunk of B
+// real accumulator columns an epilogue warp reads at a time
+template <int NT>
+__host__ __device__ constexpr uint32_t bs_epi_cols() { return NT < 32 ? (uint32_t)NT : 32u; }
 template <int NT>
 __host__ __device__ constexpr uint32_t bs_b_units() { return (uint32_t)NT < 32u ? 32u : (uint32_t)NT; }
 template <int NT>
@@ -585,7 +657,7 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
     constexpr uint32_t kCols = NT < 32 ? 32u : (uint32_t)NT;
     constexpr uint32_t kRegA = region_bytes(kRows), kRegB = region_bytes(NT);
     constexpr uint32_t kStage = bs_stage_bytes(), kBChunk = bs_b_bytes<NT>();
-    constexpr uint32_t kW = epi_cols<NT>();
+    constexpr uint32_t kW = bs_epi_cols<NT>();
     constexpr uint32_t kNc = (uint32_t)NT / 2u;
     constexpr uint32_t kRaw = bs_raw_depth<NT>();
     constexpr uint32_t kRawSlotA = PA * 64u;
@@ -606,14 +678,14 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
     const uint64_t t1 = ((uint64_t)blockIdx.x + 1u) * ga.n_tiles / gridDim.x;
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < S; s++) {
-            mbar_init(smem_u32(&full_bar[s]), PA);
+            mbar_init(smem_u32(&full_bar[s]), PA / 32u);
             mbar_init(smem_u32(&empty_bar[s]), 1);
         }
         for (uint32_t b = 0; b < NA; b++) {
             mbar_init(smem_u32(&accf_bar[b]), 1);
-            mbar_init(smem_u32(&acce_bar[b]), kEpiThreads);
+            mbar_init(smem_u32(&acce_bar[b]), kEpiThreads / 32u);
         }
-        mbar_init(smem_u32(&bfull_bar), PB);
+        mbar_init(smem_u32(&bfull_bar), PB / 32u);
         mbar_init(smem_u32(&bempty_bar), 1);
         mbar_init(smem_u32(&drain_bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -676,11 +748,11 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
         if (t0 < t1) setup();
         const uint64_t total = (t1 - t0) * ga.n_chunks;
         for (uint32_t i = 0; i + 1 < kRaw; i++) issue_next(i);
-        for (uint64_t gc = 0; gc < total && !fail; gc++) {
+        for (uint64_t gc = 0; gc < total; gc++) {
             issue_next(gc + kRaw - 1);
             cp_async_wait<kRaw - 1>();
             const uint32_t s = (uint32_t)(gc % S);
-            if (!wait_or_fail(smem_u32(&empty_bar[s]), (uint32_t)((gc / S) & 1u) ^ 1u, &fail)) {
+            if (!warp_wait_or_fail(smem_u32(&empty_bar[s]), (uint32_t)((gc / S) & 1u) ^ 1u, &fail)) {
                 fail = 1;
                 break;
             }
@@ -690,7 +762,7 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
             for (uint32_t j = 0; j < 8; j++) v[j] = pad ? make_float2(0.f, 0.f) : rt[j * PA];
             store_a(gsm + s * kStage, v, row, h);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_bar[s])) : "memory");
+            warp_arrive(smem_u32(&full_bar[s]));
         }
         cp_async_wait<0>();
     } else if (warp < kMmaWarp) {
@@ -705,9 +777,9 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
         uint32_t gi = 0;
         BsCursor cur;
         cur.c = tile_coord_bs(t0, ga);
-        for (uint64_t t = t0; t < t1 && !fail; gi++) {
+        for (uint64_t t = t0; t < t1; gi++) {
             const uint64_t grp = t >> ga.mt_bits;
-            if (!wait_or_fail(smem_u32(&bempty_bar), (gi & 1u) ^ 1u, &fail)) {
+            if (!warp_wait_or_fail(smem_u32(&bempty_bar), (gi & 1u) ^ 1u, &fail)) {
                 fail = 1;
                 break;
             }
@@ -730,11 +802,11 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
                     float2 e[8];
 #pragma unroll
                     for (uint32_t j = 0; j < 8; j++) e[j] = pad ? make_float2(0.f, 0.f) : rt[j * PB];
-                    store_b<NT>(sB + c * kBChunk, e, col, h);
+                    store_b_interleaved<NT>(sB + c * kBChunk, e, col, h);
                 }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bfull_bar)) : "memory");
+            warp_arrive(smem_u32(&bfull_bar));
             t = (grp + 1u) << ga.mt_bits;   // the next column tile's first row tile
             cur.next_group(ga);
         }
@@ -804,12 +876,12 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
         uint32_t j = 0;
         BsCursor cur;
         cur.c = tile_coord_bs(t0, ga);
-        for (uint64_t t = t0; t < t1 && !fail; t++, j++, cur.next(ga)) {
+        for (uint64_t t = t0; t < t1; t++, j++, cur.next(ga)) {
             const TileCoord &tc = cur.c;
             const uint32_t buf = j % NA;
             float2 *Crow = ga.arenas + (uint64_t)tc.il * ga.a.arena_elems + g.c_off + pext_runs(tc.beta, g.cb, g.n_cb) +
                            pext_runs(tc.mt * kRows + 32u * q + lane, g.cm, g.n_cm);
-            if (!wait_or_fail(smem_u32(&accf_bar[buf]), (j / NA) & 1u, &fail)) {
+            if (!warp_wait_or_fail(smem_u32(&accf_bar[buf]), (j / NA) & 1u, &fail)) {
                 fail = 1;
                 break;
             }
@@ -818,7 +890,7 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
             for (uint32_t j0 = share * kW; j0 < (uint32_t)NT; j0 += 2u * kW) {
                 const uint32_t my_col = pext_runs(tc.nt * kNc + j0 / 2u + (lane % (kW / 2u)), g.cn, g.n_cn);
                 uint32_t r[kW];
-                tmem_ld<kW>(taddr + j0, r);
+                tmem_ld_pairs<kW>(taddr + j0, r);
 #pragma unroll
                 for (uint32_t i = 0; i < kW / 2u; i++) {
                     const uint32_t coff = __shfl_sync(0xffffffffu, my_col, i);
@@ -826,7 +898,7 @@ __global__ void __launch_bounds__(bs_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArg
                 }
             }
             tc_fence_before();
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acce_bar[buf])) : "memory");
+            warp_arrive(smem_u32(&acce_bar[buf]));
         }
     }
     tc_fence_before();
