@@ -117,12 +117,14 @@ typedef struct {
                                   amplitudes). Not with gradient plans. */
     int32_t open_qubits[16];   /* the open qubits; amplitude j of a bitstring sets open_qubits[i]
                                   to bit i of j (the bitstring's own bits there are ignored) */
-    int32_t tensor_cores;      /* stepwise engine: 1 runs the dense contractions (16 to 1024
-                                  summed entries, 64 output entries of one operand's own and 16 of
-                                  the other's, 12 or more flops per algorithmic byte) as complex
+    int32_t tensor_cores;      /* stepwise engine: 1 runs the dense contractions (8 to 1024
+                                  summed entries, 128 output entries of one operand's own and 8 of
+                                  the other's, 5 or more flops per algorithmic byte) as complex
                                   GEMMs on the tcgen05 tensor cores, each FP32 operand split into
-                                  three bf16 parts (six products, FP32 accumulation: about 2^-23
-                                  relative error per product); 0 keeps them on FP32 SIMT kernels */
+                                  two scaled fp16 parts (three products) or, for circuits whose
+                                  gate entries differ much in size, three bf16 parts (six
+                                  products), FP32 accumulation, about 2^-22 relative error per
+                                  product; 0 keeps them on FP32 SIMT kernels */
     int32_t plan_trials;       /* 1 ... 65536 independent planning trials (ordering, slice choice and
                                   re-ordering, each from its own seed; trial 0 from order_seed);
                                   the plan with the smallest bandwidth-weighted contraction

@@ -29,10 +29,10 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 uint32_t words_of(const qvx::Plan &p) { return (uint32_t)((p.model.n_qubits + 63) / 64); }
 
 // Workspace layout: [device image][status word, CTA counter][host staging: bitstrings,
-// amplitudes][item partials][stepwise arenas], and for gradient plans [derivative
-// partials][gradient arenas]
+// amplitudes][item partials][stepwise arenas][largest entries of the tensor-core steps'
+// operands], and for gradient plans [derivative partials][gradient arenas]
 struct WsLayout {
-    size_t image, status, stage_bits, stage_amps, partials, arenas, total;
+    size_t image, status, stage_bits, stage_amps, partials, arenas, maxes, total;
     int64_t items_in_flight;
     size_t grad_partials = 0, grad_arenas = 0;
     int64_t grad_slots = 0;
@@ -55,7 +55,8 @@ WsLayout layout_of(const qvx::Plan &p, int64_t batch) {
         int64_t fit = std::max<int64_t>(1, p.opts.mem_budget_bytes / arena_bytes);
         w.items_in_flight = std::min(total_items, fit);
     }
-    w.total = align256(w.arenas + (size_t)w.items_in_flight * (size_t)std::max<int64_t>(p.arena_elems, 4) * 8);
+    w.maxes = align256(w.arenas + (size_t)w.items_in_flight * (size_t)std::max<int64_t>(p.arena_elems, 4) * 8);
+    w.total = align256(w.maxes + (size_t)w.items_in_flight * (size_t)p.n_max_slots * 4);
     if (p.opts.gradient) {
         const qvx::DevProgram *h = reinterpret_cast<const qvx::DevProgram *>(p.image.data());
         const int64_t total_items = std::max<int64_t>(batch, 1) * n_outer;
@@ -231,15 +232,34 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
         *fl *= (double)n;
         *by *= (double)n;
     };
+    // largest entries: one word per work item in flight for each operand of a tensor-core step
+    uint32_t *maxes = reinterpret_cast<uint32_t *>(base + w.maxes);
+    auto max_of = [&](int t) -> uint32_t * {
+        return p.n_max_slots > 0 && p.max_slot[t] >= 0 ? maxes + (size_t)p.max_slot[t] * (size_t)w.items_in_flight : nullptr;
+    };
+    auto scale_of = [&](int s, qvx::GemmScale *sc) -> const qvx::GemmScale * {
+        if (!p.fp16_split) return nullptr;
+        const qvx::PStep &stp = p.steps[s];
+        const bool swap = p.gemm_swap[s] != 0;
+        const int ta = swap ? stp.b : stp.a, tb = swap ? stp.a : stp.b;
+        sc->max_a = max_of(ta);
+        sc->max_b = max_of(tb);
+        const qvx::GemmStep &g = p.gemm[s];
+        sc->leaf_max_a = (g.flags & qvx::kStepALeaf) ? p.leaf_max[g.a_off] : 0u;
+        sc->leaf_max_b = (g.flags & qvx::kStepBLeaf) ? p.leaf_max[g.b_off] : 0u;
+        return sc;
+    };
     // one launch of a single step s (its kind chosen as below), timed when profiling
     auto single = [&](int s, int kind, int64_t ib, int64_t n) -> cudaError_t {
         const uint32_t rc = (uint32_t)p.tensors[p.steps[s].c].modes.size();
         if (prof) prof->begin();
         cudaError_t r;
-        if (kind == QVX_KERNEL_GEMM_TC) r = qvx::launch_gemm_step(a, p.gemm[s], ib, n, arenas, st);
-        else if (kind == QVX_KERNEL_SPLITK) r = qvx::launch_splitk_step(a, (uint32_t)s, ib, n, arenas, rc, st);
-        else if (kind == QVX_KERNEL_REGTILE) r = qvx::launch_regtile_step(a, p.regtile[s], ib, n, arenas, st);
-        else r = qvx::launch_step(a, (uint32_t)s, ib, n, arenas, rc, st);
+        uint32_t *mc = max_of(p.steps[s].c);
+        qvx::GemmScale sc{};
+        if (kind == QVX_KERNEL_GEMM_TC) r = qvx::launch_gemm_step(a, p.gemm[s], scale_of(s, &sc), mc, ib, n, arenas, st);
+        else if (kind == QVX_KERNEL_SPLITK) r = qvx::launch_splitk_step(a, (uint32_t)s, ib, n, arenas, rc, mc, st);
+        else if (kind == QVX_KERNEL_REGTILE) r = qvx::launch_regtile_step(a, p.regtile[s], ib, n, arenas, mc, st);
+        else r = qvx::launch_step(a, (uint32_t)s, ib, n, arenas, rc, mc, st);
         if (prof && r == cudaSuccess) {
             double fl, by;
             cost((size_t)s, n, &fl, &by);
@@ -249,6 +269,9 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
     };
     for (int64_t ib = 0; ib < n_items; ib += w.items_in_flight) {
         const int64_t n = std::min<int64_t>(w.items_in_flight, n_items - ib);
+        if (p.n_max_slots > 0 &&
+            (e = cudaMemsetAsync(maxes, 0, (size_t)p.n_max_slots * (size_t)w.items_in_flight * 4, st)) != cudaSuccess)
+            return cuda_fail(e, "memset");
         for (const auto &ph : p.phases) {
             // the phase's small steps (under 2^18 outputs over the items in flight) share one
             // launch; the others get their own. Split-K takes the steps with many summed
@@ -266,6 +289,7 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
                 }
                 if (threads < (1u << 18) && !splitk && grp.n < (uint32_t)qvx::kMaxGroupSteps) {
                     grp.step[grp.n] = (uint32_t)s;
+                    grp.max_c[grp.n] = max_of(p.steps[s].c);
                     grp.first_block[grp.n + 1] = grp.first_block[grp.n] + (uint32_t)((threads + 255) / 256);
                     grp.n++;
                     continue;

@@ -56,6 +56,17 @@ __device__ __forceinline__ uint32_t leaf_base(const DevLeaf &L, const Bits &x, u
     return off;
 }
 
+// Largest entry of a tensor: the bits of max(|re|, |im|), which order like unsigned integers
+// (NaN above infinity above every number).
+__device__ __forceinline__ uint32_t abs_max(uint32_t m, float2 v) {
+    return max(m, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu));
+}
+// Merges the lanes' maxima into *slot (all 32 lanes of the warp, one tensor).
+__device__ __forceinline__ void note_max_warp(uint32_t *slot, uint32_t m) {
+    const uint32_t w = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31u) == 0u) atomicMax(slot, w);
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Bulk asynchronous copy (TMA engine) of `bytes` (a multiple of 16, both addresses 16-byte

@@ -556,8 +556,15 @@ __global__ void __launch_bounds__(512) fused_program_kernel(LaunchArgs a, int wa
 }
 
 // ------------------------------------------------------------------ stepwise engine
+// Merges one output entry's size into its tensor's word: by warp when the 32 lanes hold entries
+// of one item (32 or more output entries, which also makes the active lanes whole warps).
+__device__ __forceinline__ void note_entry_max(uint32_t *slot, uint32_t rc, float2 v) {
+    if (rc >= 5u) note_max_warp(slot, abs_max(0u, v));
+    else atomicMax(slot, abs_max(0u, v));
+}
+
 __global__ void step_kernel(LaunchArgs a, uint32_t s_idx, int64_t item_begin, int64_t n_items,
-                            float2 *arenas) {
+                            float2 *arenas, uint32_t *max_c) {
     const unsigned char *img = a.image;
     const DevProgram *P = reinterpret_cast<const DevProgram *>(img);
     const DevStep &st = reinterpret_cast<const DevStep *>(img + P->steps_off)[s_idx];
@@ -577,7 +584,9 @@ __global__ void step_kernel(LaunchArgs a, uint32_t s_idx, int64_t item_begin, in
     const float2 *A = (st.flags & kStepALeaf) ? ldata + leaf_base(leaves[st.a_off], x, o) : arena + st.a_off;
     const float2 *B = unary ? A
                             : ((st.flags & kStepBLeaf) ? ldata + leaf_base(leaves[st.b_off], x, o) : arena + st.b_off);
-    arena[st.c_off + c] = step_entry(st, c, A, B, unary);
+    const float2 v = step_entry(st, c, A, B, unary);
+    arena[st.c_off + c] = v;
+    if (max_c) note_entry_max(max_c + il, st.rc, v);
 }
 
 __global__ void step_group_kernel(LaunchArgs a, StepGroup g, int64_t item_begin, int64_t n_items, float2 *arenas) {
@@ -605,7 +614,9 @@ __global__ void step_group_kernel(LaunchArgs a, StepGroup g, int64_t item_begin,
     const float2 *A = (st.flags & kStepALeaf) ? ldata + leaf_base(leaves[st.a_off], x, o) : arena + st.a_off;
     const float2 *B = unary ? A
                             : ((st.flags & kStepBLeaf) ? ldata + leaf_base(leaves[st.b_off], x, o) : arena + st.b_off);
-    arena[st.c_off + c] = step_entry(st, c, A, B, unary);
+    const float2 v = step_entry(st, c, A, B, unary);
+    arena[st.c_off + c] = v;
+    if (g.max_c[j]) note_entry_max(g.max_c[j] + il, st.rc, v);
 }
 
 // ------------------------------------------------------------------ persistent engine
@@ -744,9 +755,10 @@ struct RegTileShape {
     static constexpr int kMinBlocks = kWide ? 2 : 4;
 };
 
-template <int RM, int RN>
+template <int RM, int RN, bool kMax>   // kMax: the output's largest entries are wanted (max_c)
 __global__ void __launch_bounds__(RegTileShape<RM, RN>::kThreads, RegTileShape<RM, RN>::kMinBlocks)
-    regtile_step_kernel(LaunchArgs a, RegTileStep rs, int64_t item_begin, int64_t n_items, float2 *arenas) {
+    regtile_step_kernel(LaunchArgs a, RegTileStep rs, int64_t item_begin, int64_t n_items, float2 *arenas,
+                        uint32_t *max_c) {
     constexpr int TM = 1 << RM, TN = 1 << RN;
     const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= ((uint64_t)n_items << rs.nt)) return;
@@ -806,12 +818,36 @@ __global__ void __launch_bounds__(RegTileShape<RM, RN>::kThreads, RegTileShape<R
     for (int i = 0; i < TM; i++)
 #pragma unroll
         for (int j = 0; j < TN; j++) C[rs.c_m[i] + rs.c_n[j]] = acc[i][j];
+    if constexpr (kMax) {
+        uint32_t largest = 0;
+#pragma unroll
+        for (int i = 0; i < TM; i++)
+#pragma unroll
+            for (int j = 0; j < TN; j++) largest = abs_max(largest, acc[i][j]);
+        // one merge per CTA when all of it works on one item: with one per warp the merges into
+        // one word outlasted the stores of the largest tensors
+        if ((1ull << rs.nt) >= blockDim.x) {
+            __shared__ uint32_t warp_max[RegTileShape<RM, RN>::kThreads / 32];
+            const uint32_t w = __reduce_max_sync(0xffffffffu, largest);
+            if (threadIdx.x % 32 == 0) warp_max[threadIdx.x / 32] = w;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                uint32_t m = warp_max[0];
+                for (uint32_t k = 1; k < blockDim.x / 32; k++) m = max(m, warp_max[k]);
+                atomicMax(max_c + il, m);
+            }
+        } else if (rs.nt >= 5) {
+            note_max_warp(max_c + il, largest);
+        } else {
+            atomicMax(max_c + il, largest);
+        }
+    }
 }
 
 // A contraction with many summed entries and few outputs: 32 consecutive outputs per CTA,
 // the summed index split over the 8 warps, partial sums added through shared memory.
 __global__ void __launch_bounds__(256) splitk_step_kernel(LaunchArgs a, uint32_t s_idx, int64_t item_begin,
-                                                          int64_t n_items, float2 *arenas) {
+                                                          int64_t n_items, float2 *arenas, uint32_t *max_c) {
     __shared__ float2 part[8][33];
     __shared__ __align__(16) DevStep sd;
     const unsigned char *img = a.image;
@@ -869,6 +905,7 @@ __global__ void __launch_bounds__(256) splitk_step_kernel(LaunchArgs a, uint32_t
             s.y += part[j][lane].y;
         }
         arena[sd.c_off + c] = s;
+        if (max_c) note_entry_max(max_c + (int64_t)(w >> sd.rc), sd.rc, s);
     }
 }
 
@@ -1397,11 +1434,11 @@ cudaError_t launch_fused(const LaunchArgs &a, int warps_per_item, int items_per_
 }
 
 cudaError_t launch_step(const LaunchArgs &a, uint32_t step, int64_t item_begin, int64_t n_items,
-                        float2 *arenas, uint32_t rc, cudaStream_t s) {
+                        float2 *arenas, uint32_t rc, uint32_t *max_c, cudaStream_t s) {
     const uint64_t total = (uint64_t)n_items << rc;
     const int threads = 256;
     const uint64_t blocks = (total + threads - 1) / threads;
-    step_kernel<<<(unsigned)blocks, threads, 0, s>>>(a, step, item_begin, n_items, arenas);
+    step_kernel<<<(unsigned)blocks, threads, 0, s>>>(a, step, item_begin, n_items, arenas, max_c);
     return counted(cudaGetLastError());
 }
 
@@ -1413,41 +1450,42 @@ cudaError_t launch_step_group(const LaunchArgs &a, const StepGroup &g, int64_t i
 }
 
 cudaError_t launch_splitk_step(const LaunchArgs &a, uint32_t step, int64_t item_begin, int64_t n_items,
-                               float2 *arenas, uint32_t rc, cudaStream_t s) {
+                               float2 *arenas, uint32_t rc, uint32_t *max_c, cudaStream_t s) {
     const uint64_t blocks = (((uint64_t)n_items << rc) + 31) / 32;
     if (blocks > 0x7fffffffull) return cudaErrorInvalidConfiguration;
-    splitk_step_kernel<<<(unsigned)blocks, 256, 0, s>>>(a, step, item_begin, n_items, arenas);
+    splitk_step_kernel<<<(unsigned)blocks, 256, 0, s>>>(a, step, item_begin, n_items, arenas, max_c);
     return counted(cudaGetLastError());
 }
 
 template <int RM, int RN>
 static void launch_regtile_t(const LaunchArgs &a, const RegTileStep &rs, int64_t item_begin, int64_t n_items,
-                             float2 *arenas, cudaStream_t s) {
+                             float2 *arenas, uint32_t *max_c, cudaStream_t s) {
     constexpr int kThreads = RegTileShape<RM, RN>::kThreads;
     const uint64_t blocks = (((uint64_t)n_items << rs.nt) + kThreads - 1) / kThreads;
-    regtile_step_kernel<RM, RN><<<(unsigned)blocks, kThreads, 0, s>>>(a, rs, item_begin, n_items, arenas);
+    if (max_c) regtile_step_kernel<RM, RN, true><<<(unsigned)blocks, kThreads, 0, s>>>(a, rs, item_begin, n_items, arenas, max_c);
+    else regtile_step_kernel<RM, RN, false><<<(unsigned)blocks, kThreads, 0, s>>>(a, rs, item_begin, n_items, arenas, nullptr);
 }
 
 cudaError_t launch_regtile_step(const LaunchArgs &a, const RegTileStep &rs, int64_t item_begin, int64_t n_items,
-                                float2 *arenas, cudaStream_t s) {
+                                float2 *arenas, uint32_t *max_c, cudaStream_t s) {
     const uint64_t blocks = (((uint64_t)n_items << rs.nt) + 127) / 128;
     if (blocks > 0x7fffffffull || rs.rm > 3 || rs.rn > 3 || rs.rm + rs.rn == 0) return cudaErrorInvalidConfiguration;
     switch (rs.rm * 4 + rs.rn) {
-        case 1: launch_regtile_t<0, 1>(a, rs, item_begin, n_items, arenas, s); break;
-        case 2: launch_regtile_t<0, 2>(a, rs, item_begin, n_items, arenas, s); break;
-        case 3: launch_regtile_t<0, 3>(a, rs, item_begin, n_items, arenas, s); break;
-        case 4: launch_regtile_t<1, 0>(a, rs, item_begin, n_items, arenas, s); break;
-        case 5: launch_regtile_t<1, 1>(a, rs, item_begin, n_items, arenas, s); break;
-        case 6: launch_regtile_t<1, 2>(a, rs, item_begin, n_items, arenas, s); break;
-        case 7: launch_regtile_t<1, 3>(a, rs, item_begin, n_items, arenas, s); break;
-        case 8: launch_regtile_t<2, 0>(a, rs, item_begin, n_items, arenas, s); break;
-        case 9: launch_regtile_t<2, 1>(a, rs, item_begin, n_items, arenas, s); break;
-        case 10: launch_regtile_t<2, 2>(a, rs, item_begin, n_items, arenas, s); break;
-        case 11: launch_regtile_t<2, 3>(a, rs, item_begin, n_items, arenas, s); break;
-        case 12: launch_regtile_t<3, 0>(a, rs, item_begin, n_items, arenas, s); break;
-        case 13: launch_regtile_t<3, 1>(a, rs, item_begin, n_items, arenas, s); break;
-        case 14: launch_regtile_t<3, 2>(a, rs, item_begin, n_items, arenas, s); break;
-        default: launch_regtile_t<3, 3>(a, rs, item_begin, n_items, arenas, s); break;
+        case 1: launch_regtile_t<0, 1>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 2: launch_regtile_t<0, 2>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 3: launch_regtile_t<0, 3>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 4: launch_regtile_t<1, 0>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 5: launch_regtile_t<1, 1>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 6: launch_regtile_t<1, 2>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 7: launch_regtile_t<1, 3>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 8: launch_regtile_t<2, 0>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 9: launch_regtile_t<2, 1>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 10: launch_regtile_t<2, 2>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 11: launch_regtile_t<2, 3>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 12: launch_regtile_t<3, 0>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 13: launch_regtile_t<3, 1>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        case 14: launch_regtile_t<3, 2>(a, rs, item_begin, n_items, arenas, max_c, s); break;
+        default: launch_regtile_t<3, 3>(a, rs, item_begin, n_items, arenas, max_c, s); break;
     }
     return counted(cudaGetLastError());
 }

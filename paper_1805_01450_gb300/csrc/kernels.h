@@ -56,10 +56,14 @@ cudaError_t fused_prepare(size_t smem_bytes);
 bool fused_shape(const DevProgram *h, uint64_t arena_elems, int warps_per_item, LaunchArgs *a, size_t *shared,
                  size_t *group, int *max_ipc);
 
+// The step launchers take `max_c`: null, or one word per work item of the launch (zero before
+// the launch) that receives the bits of the output tensor's largest entry, for the operands of
+// tensor-core steps (GemmScale).
+
 // Stepwise engine: one launch per program step over `n_items` work items, tensors in a
 // global-memory arena per item.
 cudaError_t launch_step(const LaunchArgs &a, uint32_t step, int64_t item_begin, int64_t n_items,
-                        float2 *arenas, uint32_t rc, cudaStream_t s);
+                        float2 *arenas, uint32_t rc, uint32_t *max_c, cudaStream_t s);
 // Several independent small steps (of one level phase) in one launch: step j takes the CTAs
 // [first_block[j], first_block[j + 1]), one thread per output entry of each work item.
 constexpr int kMaxGroupSteps = 24;
@@ -67,15 +71,16 @@ struct StepGroup {
     uint32_t n;
     uint32_t step[kMaxGroupSteps];
     uint32_t first_block[kMaxGroupSteps + 1];
+    uint32_t *max_c[kMaxGroupSteps];
 };
 cudaError_t launch_step_group(const LaunchArgs &a, const StepGroup &g, int64_t item_begin, int64_t n_items,
                               float2 *arenas, cudaStream_t s);
 // Contraction with many summed entries: 32 outputs per CTA, the summed index split over warps.
 cudaError_t launch_splitk_step(const LaunchArgs &a, uint32_t step, int64_t item_begin, int64_t n_items,
-                               float2 *arenas, uint32_t rc, cudaStream_t s);
+                               float2 *arenas, uint32_t rc, uint32_t *max_c, cudaStream_t s);
 // Register-tiled form of a two-operand step (2^rm x 2^rn outputs per thread, rm, rn <= 2).
 cudaError_t launch_regtile_step(const LaunchArgs &a, const RegTileStep &rs, int64_t item_begin, int64_t n_items,
-                                float2 *arenas, cudaStream_t s);
+                                float2 *arenas, uint32_t *max_c, cudaStream_t s);
 // Persistent engine: one cooperative launch per chunk of work items (grid <= co-resident CTAs).
 int persistent_blocks_per_sm();
 cudaError_t launch_persistent(const LaunchArgs &a, int64_t item_begin, int64_t n_items, float2 *arenas,
@@ -123,10 +128,15 @@ uint64_t launches_issued();
 cudaError_t launch_counted(cudaError_t e);
 // Tensor-core form of a dense step (gemm_tc.cu): the column tile size, and the launch for
 // items [item0, item0 + n_items) whose arenas start at `arenas` (operands are read from the
-// arenas as complex64 and split into bf16 parts inside the kernel).
+// arenas as complex64 and split into 16-bit parts inside the kernel): two fp16 parts scaled by
+// the operands' largest entries (`scale`), or three bf16 parts (null).
+struct GemmScale {
+    const uint32_t *max_a, *max_b;       // per work item of the launch (max_c of the operand's step); null: a leaf
+    uint32_t leaf_max_a, leaf_max_b;     // the same bits of a leaf operand
+};
 uint32_t gemm_nt(const GemmStep &g);
-cudaError_t launch_gemm_step(const LaunchArgs &a, const GemmStep &g, int64_t item0, int64_t n_items, float2 *arenas,
-                             cudaStream_t s);
+cudaError_t launch_gemm_step(const LaunchArgs &a, const GemmStep &g, const GemmScale *scale, uint32_t *max_c, int64_t item0,
+                             int64_t n_items, float2 *arenas, cudaStream_t s);
 // Self-test of the bounded waits (grid barrier and mbarrier that can never complete).
 cudaError_t launch_wait_selftest(unsigned *words, unsigned *status, uint32_t polls, unsigned *out, cudaStream_t s);
 

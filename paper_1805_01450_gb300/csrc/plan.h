@@ -73,6 +73,14 @@ struct Plan {
     int warps_per_item = 1;
     std::vector<unsigned char> image;          // device image (DevProgram first)
     std::vector<RegTileStep> regtile;          // per step, global-arena engines: register-tiled form (rm + rn > 0)
+    // two-part fp16 operands of tensor-core steps (else three-part bf16): per tensor the word
+    // that receives its largest entry (-1: not an operand of such a step), their count, and per
+    // device leaf the bits of its largest entry
+    bool fp16_split = false;
+    std::vector<int> max_slot;
+    int n_max_slots = 0;
+    std::vector<uint32_t> leaf_max;
+    std::vector<char> gemm_swap;               // per step: the GEMM's row operand is the step's B
     std::vector<GemmStep> gemm;                // per step, stepwise engine with tensor cores: GEMM form (nk > 0)
     // gradient program
     int n_params = 0;

@@ -1408,6 +1408,7 @@ bool serialize(Plan &p, std::string *err) {
     // whose lowest output mode is held by both operands (a batch mode) keeps its SIMT form.
     // Complex products commute, so the step's B may take the row role.
     std::vector<GemmStep> gms;
+    p.gemm_swap.assign(ds.size(), 0);
     if (p.engine == QVX_ENGINE_STEPWISE && p.opts.tensor_cores) {
         gms.assign(ds.size(), GemmStep{});
         for (size_t s = 0; s < p.steps.size(); s++) {
@@ -1451,6 +1452,7 @@ bool serialize(Plan &p, std::string *err) {
             gmap(gb, LB, g.bb, &g.n_bb); gmap(gn, LB, g.bn, &g.n_bn); gmap(st.k_ab, LB, g.bk, &g.n_bk);
             gmap(gb, LC, g.cb, &g.n_cb); gmap(gm, LC, g.cm, &g.n_cm); gmap(gn, LC, g.cn, &g.n_cn);
             if (!ok) { std::memset(&g, 0, sizeof(g)); continue; }
+            p.gemm_swap[s] = swap ? 1 : 0;
             g.a_off = swap ? ds[s].b_off : ds[s].a_off;
             g.b_off = swap ? ds[s].a_off : ds[s].b_off;
             g.c_off = ds[s].c_off;
@@ -1461,6 +1463,26 @@ bool serialize(Plan &p, std::string *err) {
             g.nm = (uint8_t)gm.size();
             g.nn = (uint8_t)gn.size();
             g.nk = (uint8_t)st.k_ab.size();
+        }
+    }
+    // the operands of tensor-core steps whose largest entry the two-part split needs
+    p.max_slot.assign(p.tensors.size(), -1);
+    p.n_max_slots = 0;
+    p.leaf_max.clear();
+    if (p.fp16_split) {
+        for (size_t s = 0; s < gms.size(); s++) {
+            if (gms[s].nk == 0) continue;
+            for (int t : {p.steps[s].a, p.steps[s].b})
+                if (p.tensors[t].leaf < 0 && p.max_slot[t] < 0) p.max_slot[t] = p.n_max_slots++;
+        }
+        for (const DevLeaf &d : dl) {   // stored entries of a leaf: its modes and its fixed modes
+            uint32_t m = 0;
+            for (uint64_t e = 0; e < 2 * ((uint64_t)d.n_elem << d.n_fixed); e++) {
+                uint32_t w;
+                std::memcpy(&w, &ldata[2 * d.data_off + e], 4);
+                m = std::max(m, w & 0x7fffffffu);
+            }
+            p.leaf_max.push_back(m);
         }
     }
     // fused form: per-step tables of pext(c) for both operands (16-bit offsets), and per
@@ -1840,10 +1862,30 @@ qvx_status make_plan(const qvx_circuit *c, const int32_t *order, int32_t n_order
 
 namespace {
 
+// Whether the entries of every gate are zero or of magnitude 2^-4 ... 2: the tensors' entries
+// then stay within the range that two fp16 parts hold after scaling (gates with very unequal
+// entries, U1 matrices or rotations by tiny angles, would lose the small ones).
+bool gates_alike(const qvx_circuit *c) {
+    if (!c || c->n_gates < 0 || (c->n_gates > 0 && !c->gates)) return false;
+    for (int64_t i = 0; i < c->n_gates; i++) {
+        cplx m[2][2];
+        if (c->gates[i].kind == QVX_GATE_CZ) continue;
+        if (c->gates[i].kind == QVX_GATE_T) continue;
+        if (!gate_matrix(c->gates[i], m)) return false;
+        for (int r = 0; r < 2; r++)
+            for (int k = 0; k < 2; k++) {
+                const double v = std::abs(m[r][k]);
+                if (!(v < 1e-16 || (v >= 1.0 / 16.0 && v <= 2.0))) return false;
+            }
+    }
+    return true;
+}
+
 qvx_status plan_once(const qvx_circuit *c, const int32_t *order, int32_t n_order,
                      const int32_t *slices, int32_t n_slices, const qvx_plan_opts &opts,
                      Plan *p, std::string *err) {
     p->opts = opts;
+    p->fp16_split = gates_alike(c);
     if (!build_model(c, &p->model, err, opts.gradient != 0)) return QVX_EINVAL;
     if (opts.n_open_qubits < 0 || opts.n_open_qubits > 16) { *err = "opts: n_open_qubits must be in [0, 16]"; return QVX_EINVAL; }
     if (opts.n_open_qubits > 0 && opts.gradient) { *err = "open qubits are not supported with gradients"; return QVX_EUNSUPPORTED; }
