@@ -320,7 +320,9 @@ typedef struct {
     int64_t items;         /* work items the launch processed (sums: partials added) */
     double flops;          /* algorithmic real flops of the launch (8 per complex MAC) */
     double bytes;          /* algorithmic bytes of the launch: each operand read and each
-                              output written once (complex64; 32-byte exact partials) */
+                              output written once (complex64; 32-byte exact partials), summed
+                              over the contractions it runs, also where a tensor between two of
+                              them stays on the chip */
     float ms;              /* device time between CUDA events recorded on the call's stream
                               just before and just after the launch */
     int32_t pad;

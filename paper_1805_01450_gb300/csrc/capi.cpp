@@ -227,8 +227,15 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
         }
         return QVX_OK;
     }
+    auto paired = [&](int s) { return !p.pairs.empty() && p.pairs[s].consumer >= 0; };
     auto cost = [&](size_t s, int64_t n, double *fl, double *by) {
         qvx::step_cost(p, s, fl, by);
+        if (paired((int)s)) {   // one launch for both steps' work
+            double f2, b2;
+            qvx::step_cost(p, (size_t)p.pairs[s].consumer, &f2, &b2);
+            *fl += f2;
+            *by += b2;
+        }
         *fl *= (double)n;
         *by *= (double)n;
     };
@@ -240,13 +247,15 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
     auto scale_of = [&](int s, qvx::GemmScale *sc) -> const qvx::GemmScale * {
         if (!p.fp16_split) return nullptr;
         const qvx::PStep &stp = p.steps[s];
-        const bool swap = p.gemm_swap[s] != 0;
+        const bool pair = paired(s);
+        const bool swap = pair ? p.pairs[s].swap : p.gemm_swap[s] != 0;
         const int ta = swap ? stp.b : stp.a, tb = swap ? stp.a : stp.b;
         sc->max_a = max_of(ta);
         sc->max_b = max_of(tb);
-        const qvx::GemmStep &g = p.gemm[s];
+        const qvx::GemmStep &g = pair ? p.pairs[s].g : p.gemm[s];
         sc->leaf_max_a = (g.flags & qvx::kStepALeaf) ? p.leaf_max[g.a_off] : 0u;
         sc->leaf_max_b = (g.flags & qvx::kStepBLeaf) ? p.leaf_max[g.b_off] : 0u;
+        sc->leaf_max_d = pair ? p.leaf_max[p.pairs[s].leaf.leaf] : 0u;
         return sc;
     };
     // one launch of a single step s (its kind chosen as below), timed when profiling
@@ -254,9 +263,11 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
         const uint32_t rc = (uint32_t)p.tensors[p.steps[s].c].modes.size();
         if (prof) prof->begin();
         cudaError_t r;
-        uint32_t *mc = max_of(p.steps[s].c);
+        uint32_t *mc = max_of(p.steps[paired(s) ? p.pairs[s].consumer : s].c);
         qvx::GemmScale sc{};
-        if (kind == QVX_KERNEL_GEMM_TC) r = qvx::launch_gemm_step(a, p.gemm[s], scale_of(s, &sc), mc, ib, n, arenas, st);
+        if (paired(s)) r = qvx::launch_gemm_step(a, p.pairs[s].g, &p.pairs[s].leaf, scale_of(s, &sc), mc, ib, n, arenas, st);
+        else if (kind == QVX_KERNEL_GEMM_TC)
+            r = qvx::launch_gemm_step(a, p.gemm[s], nullptr, scale_of(s, &sc), mc, ib, n, arenas, st);
         else if (kind == QVX_KERNEL_SPLITK) r = qvx::launch_splitk_step(a, (uint32_t)s, ib, n, arenas, rc, mc, st);
         else if (kind == QVX_KERNEL_REGTILE) r = qvx::launch_regtile_step(a, p.regtile[s], ib, n, arenas, mc, st);
         else r = qvx::launch_step(a, (uint32_t)s, ib, n, arenas, rc, mc, st);
@@ -282,7 +293,8 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
                 const PStepShape sh = shape_of(p, s);
                 const uint64_t threads = (uint64_t)n << rc;
                 const bool splitk = sh.nk >= 5 && rc <= 12;
-                if (!p.gemm.empty() && p.gemm[s].nk > 0) {   // tensor cores
+                if (!p.pairs.empty() && p.pairs[s].absorbed) continue;   // its operand's producer runs it
+                if (paired(s) || (!p.gemm.empty() && p.gemm[s].nk > 0)) {   // tensor cores
                     if ((e = single(s, QVX_KERNEL_GEMM_TC, ib, n)) != cudaSuccess)
                         return cuda_fail(e, "tensor-core step launch");
                     continue;

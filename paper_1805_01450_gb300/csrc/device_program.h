@@ -132,6 +132,24 @@ struct GemmStep {
     DevRun cb[kGroupRuns], cm[kGroupRuns], cn[kGroupRuns];   // C: b, m, n
 };
 
+// A leaf multiplied into one operand of a tensor-core step while the operand is staged:
+//   C[b, m, n] = sum_k A[b, m, k] D[b, k, n] B[b, k, n]   (on_rows: D[b, m, k] with A instead).
+// It runs a contraction X = A B and the contraction of X with a leaf D as one GEMM whose
+// summed index holds the modes of both.
+struct GemmLeaf {
+    uint32_t leaf;                 // leaf index
+    uint8_t on_rows, n_b, n_r, n_k;
+    DevRun b[kGroupRuns], r[kGroupRuns], k[kGroupRuns];   // D: b, m or n, k
+};
+// Two steps run as one (stepwise engine with tensor cores): step `producer` (X = A B) and step
+// `consumer` (X D). The kernels take these as launch parameters; the image holds them for
+// inspection.
+struct StepPair {
+    uint32_t producer, consumer;
+    GemmStep g;
+    GemmLeaf leaf;
+};
+
 struct DevProgram {
     uint32_t magic;
     uint32_t n_steps, n_leaves, pad0;
@@ -168,6 +186,8 @@ struct DevProgram {
     uint64_t gemm_off;             // byte offset of n_steps GemmStep (0 if absent)
     uint64_t image_bytes;
     uint64_t zero_mask_hi;         // qubits 64..127 of the zero mask
+    uint64_t pairs_off;            // byte offset of n_pairs StepPair (0 if none)
+    uint32_t n_pairs, pad1;
 };
 
 constexpr uint32_t kProgramMagic = 0x51565831u;  // "QVX1"
@@ -177,7 +197,8 @@ constexpr uint32_t kProgramMagic = 0x51565831u;  // "QVX1"
 namespace qvx {
 static_assert(sizeof(DevStep) == 136, "DevStep layout");
 static_assert(sizeof(DevLeaf) == 40, "DevLeaf layout");
-static_assert(sizeof(DevProgram) == 328, "DevProgram layout");
+static_assert(sizeof(DevProgram) == 344, "DevProgram layout");
+static_assert(sizeof(GemmLeaf) == 104 && sizeof(StepPair) == 448, "StepPair layout");
 static_assert(sizeof(GemmStep) == 336, "GemmStep layout");
 static_assert(sizeof(GradEntry) == 16, "GradEntry layout");
 static_assert(sizeof(RegTileStep) == 288, "RegTileStep layout");

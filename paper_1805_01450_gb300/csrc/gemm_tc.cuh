@@ -121,8 +121,8 @@ __host__ __device__ constexpr uint32_t n_stages() { return 3u; }
 template <int NT>
 __host__ __device__ constexpr uint32_t epi_cols() { return NT >= 64 ? 16u : 8u; }
 template <int NT, int kParts>
-__host__ __device__ constexpr size_t smem_bytes(uint32_t K) {
-    return (size_t)n_stages<NT, kParts>() * stage_bytes<NT, kParts>() + 8u * (size_t)K;
+__host__ __device__ constexpr size_t smem_bytes(uint32_t K) {   // three offset tables (A, B, the leaf)
+    return (size_t)n_stages<NT, kParts>() * stage_bytes<NT, kParts>() + 12u * (size_t)K;
 }
 
 __device__ __forceinline__ uint32_t core_offset(uint32_t r, uint32_t g) {
@@ -211,17 +211,30 @@ __device__ __forceinline__ uint32_t scale_field(uint32_t m) {
 }
 __device__ __forceinline__ float pow2_field(uint32_t f) { return __uint_as_float(f << 23); }
 
+// The tensor cores truncate the FP32 accumulator at every MMA, which on average takes a part
+// kTrunc off its value. A sum of n_chunks chunks is built of M = 2 n_chunks increments (Ar, Ai
+// parts), each followed by three truncations (three products), and after increment j the partial
+// sum is, in the mean, j / M of the result, for terms of random signs as for terms of one sign:
+// the result is 3 kTrunc (M + 1) / 2 too small. That systematic part was nine tenths of the
+// error of the slice terms (64-qubit circuits, coefficient of a fit to the FP64 values: -1.8 to
+// -4.0e-6, rest 0.7 to 1.4e-6), so the epilogue's scale takes it back. kTrunc is the value that
+// these fits give over four programs with sums of 8 to 512 entries: 3.2e-8 +- 10 %.
+constexpr float kTrunc = 3.2e-8f;
+__device__ __forceinline__ float truncation_gain(uint32_t n_chunks) {
+    return 1.f + 1.5f * kTrunc * (float)(2u * n_chunks + 1u);
+}
+
 // What the epilogue multiplies an accumulator by to take out both operands' scales: 2^t with
-// t = 254 - fa - fb, in two exact factors when t is outside the float exponents.
+// t = 254 - fa - fb, in two factors when t is outside the float exponents.
 struct Unscale {
     float f1, f2;
     bool two;
 };
-__device__ __forceinline__ Unscale unscale_of(uint32_t ma, uint32_t mb) {
+__device__ __forceinline__ Unscale unscale_of(uint32_t ma, uint32_t mb, uint32_t n_chunks) {
     const int t = 254 - (int)scale_field(ma) - (int)scale_field(mb);
     const int t1 = max(-126, min(126, t)), t2 = max(-126, min(126, t - t1));
     Unscale u;
-    u.f1 = pow2_field((uint32_t)(t1 + 127));
+    u.f1 = pow2_field((uint32_t)(t1 + 127)) * truncation_gain(n_chunks);
     u.f2 = pow2_field((uint32_t)(t2 + 127));
     u.two = t2 != 0;
     return u;
@@ -350,6 +363,8 @@ __device__ __forceinline__ void store_b_interleaved(unsigned char *sb, const Uni
 struct Fetch {
     float2 v[8];
     uint32_t max;
+    uint32_t chunk;                // with a leaf: the chunk, and the leaf's entries for the
+    const float2 *factor;          // tile and the thread's row or column
 };
 template <bool kL2>   // read through L2 only: rows that the SM does not read again
 __device__ __forceinline__ void fetch8(Fetch &f, const float2 *src, const uint32_t *off) {
@@ -362,6 +377,8 @@ __device__ __forceinline__ void fetch_zero(Fetch &f) {
 #pragma unroll
     for (uint32_t j = 0; j < 8; j++) f.v[j] = make_float2(0.f, 0.f);
     f.max = 0u;
+    f.chunk = 0u;
+    f.factor = nullptr;
 }
 template <int kParts>
 __device__ __forceinline__ void split_fetch(Fetch &f, Unit<kParts> &x) {
@@ -449,6 +466,7 @@ __device__ __forceinline__ void tmem_ld_pairs(uint32_t taddr, uint32_t (&r)[kW])
 struct GemmArgs {
     LaunchArgs a;
     GemmStep g;
+    GemmLeaf leaf;                 // kernels with a leaf only
     GemmScale sc;                  // the operands' largest entries (fp16 split)
     uint32_t *max_c;               // per item: bits of C's largest entry, or null (not needed)
     int64_t item0, n_items;
@@ -460,13 +478,37 @@ struct GemmArgs {
 };
 // The launchers of the two splits (fp16: two parts, gemm_tc.cu; bf16: three, gemm_tc_bf16.cu).
 cudaError_t launch_gemm_f16(const GemmArgs &ga, uint32_t nt_cols, cudaStream_t s);
+cudaError_t launch_gemm_leaf(const GemmArgs &ga, uint32_t nt_cols, cudaStream_t s);   // fp16, with a leaf (gemm_tc_leaf.cu)
 cudaError_t launch_gemm_bf16(const GemmArgs &ga, uint32_t nt_cols, cudaStream_t s);
 
 namespace {
 
-// Bits of an operand's largest entry for item il of the launch.
+// Bits of an operand's largest entry for item il of the launch; with the leaf multiplied in, of
+// a bound on it (a component of a product is at most twice the product of the components).
 __device__ __forceinline__ uint32_t operand_max(const uint32_t *max, uint32_t leaf_max, int64_t il) {
     return max ? __ldg(max + il) : leaf_max;
+}
+template <bool kLeaf>
+__device__ __forceinline__ uint32_t side_max(const GemmArgs &ga, bool rows, int64_t il) {
+    uint32_t m = rows ? operand_max(ga.sc.max_a, ga.sc.leaf_max_a, il) : operand_max(ga.sc.max_b, ga.sc.leaf_max_b, il);
+    if (kLeaf && rows == (ga.leaf.on_rows != 0))
+        m = __float_as_uint(2.f * __uint_as_float(m) * __uint_as_float(ga.sc.leaf_max_d)) & 0x7fffffffu;
+    return m;
+}
+
+// The leaf's entries for one item; the caller adds the offsets of b and of the row or column.
+__device__ __forceinline__ const float2 *leaf_entries(const GemmArgs &ga, int64_t item) {
+    return gemm_operand(ga.a, nullptr, ga.leaf.leaf, true, item);
+}
+// 8 summed entries of an operand times the leaf's (off: their offsets in the leaf).
+__device__ __forceinline__ void times_leaf(Fetch &f, const float2 *d, const uint32_t *off) {
+    const uint4 o0 = *reinterpret_cast<const uint4 *>(off), o1 = *reinterpret_cast<const uint4 *>(off + 4);
+    const uint32_t o[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+#pragma unroll
+    for (uint32_t j = 0; j < 8; j++) {
+        const float2 y = __ldg(d + o[j]), x = f.v[j];
+        f.v[j] = make_float2(x.x * y.x - x.y * y.y, x.x * y.y + x.y * y.x);
+    }
 }
 
 // Bounded mbarrier wait that also gives up once another role has set the CTA's fail flag.
@@ -569,7 +611,10 @@ struct BsCursor {
 // Every wait is bounded; a wait that runs out sets the CTA's fail flag, the other roles
 // leave their loops, the MMA thread waits (bounded) for its issued MMAs before the tensor
 // memory is freed, and QVX_ETIMEOUT goes to the status word.
-template <int NT, int kParts>
+// kLeaf: one operand is multiplied by a leaf between its load and its split, so that a
+// contraction and the leaf contraction of its result are one pass with a longer summed index
+// (find_pairs in planner.cpp).
+template <int NT, int kParts, bool kLeaf>
 __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArgs ga) {
     constexpr uint32_t kMmaWarp = mma_warp<NT>(), kEpiWarp = epi_warp<NT>();
     constexpr uint32_t S = n_stages<NT, kParts>();
@@ -606,10 +651,11 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
     // the summed index's offsets in A and B (bit-run maps evaluated once per CTA)
     const uint32_t K = ga.n_chunks * kKq;
     uint32_t *tka = reinterpret_cast<uint32_t *>(gsm + S * kStage);
-    uint32_t *tkb = tka + K;
+    uint32_t *tkb = tka + K, *tkd = tkb + K;
     for (uint32_t i = threadIdx.x; i < K; i += block_threads<NT>()) {
         tka[i] = pext_runs(i, g.ak, g.n_ak);
         tkb[i] = pext_runs(i, g.bk, g.n_bk);
+        if (kLeaf) tkd[i] = pext_runs(i, ga.leaf.k, ga.leaf.n_k);
     }
     tc_fence_before();
     __syncthreads();
@@ -632,12 +678,12 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
         // the part of the operand's offset that is the thread's own; the tile's part is the
         // same for the whole block
         const uint32_t own = is_a ? pext_runs(row, g.am, g.n_am) : pext_runs(row, g.bn, g.n_bn);
-        const uint32_t *max_base = is_a ? ga.sc.max_a : ga.sc.max_b;
-        const uint32_t leaf_max = is_a ? ga.sc.leaf_max_a : ga.sc.leaf_max_b;
+        const bool scaled = kLeaf && loads && is_a == (ga.leaf.on_rows != 0);   // the leaf's side
+        const uint32_t own_d = kLeaf ? pext_runs(row, ga.leaf.r, ga.leaf.n_r) : 0u;
         // load cursor: the tile and chunk that are loaded next
         uint64_t lt = blockIdx.x;
         uint32_t lc = 0, tile_max = 0;
-        const float2 *src = nullptr;
+        const float2 *src = nullptr, *factor = nullptr;
         auto setup = [&]() {
             const TileCoord tc = tile_coord(lt, ga);
             const float2 *arena = ga.arenas + (uint64_t)tc.il * ga.a.arena_elems;
@@ -645,11 +691,18 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
             const uint32_t tb = pext_runs(tc.beta, g.bb, g.n_bb) + pext_runs(tc.nt * kNc, g.bn, g.n_bn);
             src = (is_a ? gemm_operand(ga.a, arena, g.a_off, g.flags & kStepALeaf, ga.item0 + tc.il) + ta
                         : gemm_operand(ga.a, arena, g.b_off, g.flags & kStepBLeaf, ga.item0 + tc.il) + tb) + own;
-            if (kParts == 2) tile_max = operand_max(max_base, leaf_max, tc.il);
+            if (kParts == 2) tile_max = side_max<kLeaf>(ga, is_a, tc.il);
+            if (kLeaf && scaled)
+                factor = leaf_entries(ga, ga.item0 + tc.il) + pext_runs(tc.beta, ga.leaf.b, ga.leaf.n_b) + own_d +
+                         pext_runs(is_a ? tc.mt * kRows : tc.nt * kNc, ga.leaf.r, ga.leaf.n_r);
         };
         auto fetch = [&](Fetch &f) {
             if (lt >= ga.n_tiles) return;
             if (loads) fetch8<true>(f, src, koff + lc * kKq);
+            if (kLeaf) {
+                f.factor = factor;
+                f.chunk = lc;
+            }
             f.max = tile_max;
             if (++lc == ga.n_chunks) {
                 lc = 0;
@@ -665,6 +718,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
         // and stores the parts once the stage is free
         auto produce = [&](Fetch &f) -> bool {
             Unit<kParts> x;
+            if (kLeaf && scaled) times_leaf(f, f.factor, tkd + f.chunk * kKq + 8u * h);
             split_fetch<kParts>(f, x);
             fetch(f);
             if (!warp_wait_or_fail(smem_u32(&empty_bar[ring.s]), ring.phase ^ 1u, &fail)) {
@@ -696,15 +750,15 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
             constexpr uint32_t kBlkB = b_block_bytes(NT);
             RingPos ring;
             uint32_t j = 0;
-            for (uint64_t t = blockIdx.x; t < ga.n_tiles && !fail; t += gridDim.x, j++) {
+            bool ok = true;
+            for (uint64_t t = blockIdx.x; t < ga.n_tiles && ok; t += gridDim.x, j++) {
                 const uint32_t buf = j & 1u;
                 if (!wait_or_fail(smem_u32(&acce_bar[buf]), ((j >> 1) & 1u) ^ 1u, &fail)) {
-                    fail = 1;
+                    ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t d = tmem + buf * kCols;
-                bool ok = true;
                 for (uint32_t c = 0; c < ga.n_chunks; c++, ring.next(S)) {
                     const uint32_t s = ring.s;
                     if (!wait_or_fail(smem_u32(&full_bar[s]), ring.phase, &fail)) {
@@ -722,12 +776,9 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
                     mma_chunk<kParts>(d, sa, kRegA, bs, idesc, c == 0u);
                     mma_commit(smem_u32(&empty_bar[s]));
                 }
-                if (!ok) {
-                    fail = 1;
-                    break;
-                }
-                mma_commit(smem_u32(&accf_bar[buf]));
+                if (ok) mma_commit(smem_u32(&accf_bar[buf]));
             }
+            if (!ok) fail = 1;
             // every MMA issued so far completes before the tensor memory is freed
             mma_commit(smem_u32(&drain_bar));
             if (!mbar_wait(smem_u32(&drain_bar), 0, kPolls)) fail = 1;
@@ -754,8 +805,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
             float2 *Crow = ga.arenas + (uint64_t)tc.il * ga.a.arena_elems + g.c_off + pext_runs(tc.beta, g.cb, g.n_cb) +
                            pext_runs(tc.mt * kRows, g.cm, g.n_cm) + own;
             Unscale un{1.f, 1.f, false};
-            if (kParts == 2)
-                un = unscale_of(operand_max(ga.sc.max_a, ga.sc.leaf_max_a, tc.il), operand_max(ga.sc.max_b, ga.sc.leaf_max_b, tc.il));
+            if (kParts == 2) un = unscale_of(side_max<kLeaf>(ga, true, tc.il), side_max<kLeaf>(ga, false, tc.il), ga.n_chunks);
             uint32_t largest = 0;
             if (!warp_wait_or_fail(smem_u32(&accf_bar[buf]), (j >> 1) & 1u, &fail)) {
                 fail = 1;
@@ -818,15 +868,15 @@ constexpr uint32_t kBsBytes = 222u << 10;
 template <int NT, int kParts>
 __host__ __device__ constexpr uint32_t bs_chunks() {
     uint32_t c = 2u;
-    while (2u * c * kKq <= 1024u && 2u * c * bs_b_bytes<NT, kParts>() + 3u * a_bytes<kParts>() + 8u * 2u * c * kKq <= kBsBytes) c *= 2u;
+    while (2u * c * kKq <= 1024u && 2u * c * bs_b_bytes<NT, kParts>() + 3u * a_bytes<kParts>() + 12u * 2u * c * kKq <= kBsBytes) c *= 2u;
     return c;
 }
 template <int NT, int kParts>
 uint32_t bs_stages(uint32_t n_chunks) {
-    return std::min(kBsStages, (kBsBytes - n_chunks * (bs_b_bytes<NT, kParts>() + 8u * kKq)) / a_bytes<kParts>());
+    return std::min(kBsStages, (kBsBytes - n_chunks * (bs_b_bytes<NT, kParts>() + 12u * kKq)) / a_bytes<kParts>());
 }
 
-template <int NT, int kParts>
+template <int NT, int kParts, bool kLeaf>   // kLeaf: one operand is multiplied by a leaf as it is split
 __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArgs ga) {
     const uint32_t S = ga.stages;
     constexpr uint32_t NA = bs_accs<NT>();
@@ -847,7 +897,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
     unsigned char *sB = gsm + S * kStage;                          // resident B, one region set per chunk
     const uint32_t K = ga.n_chunks * kKq;
     uint32_t *tka = reinterpret_cast<uint32_t *>(sB + ga.n_chunks * kBChunk);
-    uint32_t *tkb = tka + K;
+    uint32_t *tkb = tka + K, *tkd = tkb + K;
     // this CTA's contiguous range of tiles
     const uint64_t t0 = (uint64_t)blockIdx.x * ga.n_tiles / gridDim.x;
     const uint64_t t1 = ((uint64_t)blockIdx.x + 1u) * ga.n_tiles / gridDim.x;
@@ -875,6 +925,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
     for (uint32_t i = threadIdx.x; i < K; i += block_threads<NT>()) {
         tka[i] = pext_runs(i, g.ak, g.n_ak);
         tkb[i] = pext_runs(i, g.bk, g.n_bk);
+        if (kLeaf) tkd[i] = pext_runs(i, ga.leaf.k, ga.leaf.n_k);
     }
     tc_fence_before();
     __syncthreads();
@@ -890,22 +941,31 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
         const uint32_t *koff = tka + 8u * h;
         uint64_t lt = t0;
         uint32_t lc = 0;
-        const float2 *src = nullptr;
-        const uint32_t *max_src = nullptr;
+        const float2 *src = nullptr, *factor = nullptr;
+        uint32_t tile_max = 0;
+        const bool scaled = kLeaf && !pad && ga.leaf.on_rows != 0;   // the leaf goes with the rows
+        const uint32_t own_d = kLeaf && scaled ? pext_runs(row, ga.leaf.r, ga.leaf.n_r) : 0u;
         BsCursor cur;
         cur.c = tile_coord_bs(t0, ga);
         const uint32_t own = pext_runs(row, g.am, g.n_am);
         auto setup = [&]() {
             const TileCoord &tc = cur.c;
             const float2 *arena = ga.arenas + (uint64_t)tc.il * ga.a.arena_elems;
-            if (kParts == 2) max_src = ga.sc.max_a + tc.il;
+            if (kParts == 2) tile_max = side_max<kLeaf>(ga, true, tc.il);
+            if (kLeaf && scaled)
+                factor = leaf_entries(ga, ga.item0 + tc.il) + pext_runs(tc.beta, ga.leaf.b, ga.leaf.n_b) + own_d +
+                         pext_runs(tc.mt * kRows, ga.leaf.r, ga.leaf.n_r);
             src = gemm_operand(ga.a, arena, g.a_off, g.flags & kStepALeaf, ga.item0 + tc.il) +
                   pext_runs(tc.beta, g.ab, g.n_ab) + pext_runs(tc.mt * kRows, g.am, g.n_am) + own;
         };
         auto fetch = [&](Fetch &f) {
             if (lt >= t1) return;
             if (!pad) fetch8<false>(f, src, koff + lc * kKq);
-            if (kParts == 2) f.max = ga.sc.max_a ? __ldg(max_src) : ga.sc.leaf_max_a;
+            if (kLeaf) {
+                f.factor = factor;
+                f.chunk = lc;
+            }
+            f.max = tile_max;
             if (++lc == ga.n_chunks) {
                 lc = 0;
                 if (++lt < t1) {
@@ -919,6 +979,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
         RingPos ring;
         auto produce = [&](Fetch &f) -> bool {   // as in the streaming form
             Unit<kParts> x;
+            if (kLeaf && scaled) times_leaf(f, f.factor, tkd + f.chunk * kKq + 8u * h);
             split_fetch<kParts>(f, x);
             fetch(f);
             if (!warp_wait_or_fail(smem_u32(&empty_bar[ring.s]), ring.phase ^ 1u, &fail)) {
@@ -963,13 +1024,19 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
                                 pext_runs(tc.beta, g.bb, g.n_bb) + pext_runs(tc.nt * kNc + (active ? col : 0u), g.bn, g.n_bn);
             // the first chunk is loaded while the old column tile's last MMAs run
             if (loads) fetch8<false>(f, src, koff);
-            f.max = operand_max(ga.sc.max_b, ga.sc.leaf_max_b, tc.il);
+            f.max = side_max<kLeaf>(ga, false, tc.il);
+            const float2 *factor = nullptr;
+            const bool scaled = kLeaf && loads && ga.leaf.on_rows == 0;   // the leaf goes with the columns
+            if (scaled)
+                factor = leaf_entries(ga, ga.item0 + tc.il) + pext_runs(tc.beta, ga.leaf.b, ga.leaf.n_b) +
+                         pext_runs(tc.nt * kNc + (active ? col : 0u), ga.leaf.r, ga.leaf.n_r);
             if (!warp_wait_or_fail(smem_u32(&bempty_bar), (gi & 1u) ^ 1u, &fail)) {
                 fail = 1;
                 break;
             }
             for (uint32_t c = 0; c < ga.n_chunks; c++) {
                 Unit<kParts> x;
+                if (kLeaf && scaled) times_leaf(f, factor, tkd + c * kKq + 8u * h);
                 split_fetch<kParts>(f, x);
                 if (loads && c + 1u < ga.n_chunks) fetch8<false>(f, src, koff + (c + 1u) * kKq);
                 if (active) store_b_interleaved<NT, kParts>(sB + c * kBChunk, x, col, h);
@@ -1049,7 +1116,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
                            pext_runs(tc.mt * kRows, g.cm, g.n_cm) + own;
             Unscale un{1.f, 1.f, false};
             if (kParts == 2)
-                un = unscale_of(operand_max(ga.sc.max_a, ga.sc.leaf_max_a, tc.il), operand_max(ga.sc.max_b, ga.sc.leaf_max_b, tc.il));
+                un = unscale_of(side_max<kLeaf>(ga, true, tc.il), side_max<kLeaf>(ga, false, tc.il), ga.n_chunks);
             uint32_t largest = 0;
             if (!warp_wait_or_fail(smem_u32(&accf_bar[buf]), (j / NA) & 1u, &fail)) {
                 fail = 1;
@@ -1089,7 +1156,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
 // its 512 tensor-memory columns, so that no allocation ever waits for another CTA's
 // columns), queried once per device and kernel (under a lock: host threads may launch on
 // several streams at once).
-template <int NT, int kParts, bool kBs>
+template <int NT, int kParts, bool kBs, bool kLeaf>
 static cudaError_t gemm_grid(uint64_t n_tiles, uint64_t *grid) {
     static int per_sm[64] = {0}, sms[64] = {0};
     static std::mutex mu;
@@ -1099,8 +1166,8 @@ static cudaError_t gemm_grid(uint64_t n_tiles, uint64_t *grid) {
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (!per_sm[dev]) {
-        const void *fn = kBs ? reinterpret_cast<const void *>(gemm_tc_bs_kernel<NT, kParts>)
-                             : reinterpret_cast<const void *>(gemm_tc_kernel<NT, kParts>);
+        const void *fn = kBs ? reinterpret_cast<const void *>(gemm_tc_bs_kernel<NT, kParts, kLeaf>)
+                             : reinterpret_cast<const void *>(gemm_tc_kernel<NT, kParts, kLeaf>);
         const size_t smem = kBs ? (size_t)kBsBytes : smem_bytes<NT, kParts>(1024);
         const int threads = kBs ? (int)block_threads<NT>() : (int)(int)block_threads<NT>();
         if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
@@ -1120,7 +1187,7 @@ static cudaError_t gemm_grid(uint64_t n_tiles, uint64_t *grid) {
     return cudaSuccess;
 }
 
-template <int NT, int kParts>
+template <int NT, int kParts, bool kLeaf>
 static cudaError_t launch_gemm_nt(GemmArgs ga, cudaStream_t s) {
     ga.n_tiles = ((uint64_t)ga.n_items << ga.g.nb) * ga.n_mt * ga.n_nt;
     if (ga.n_tiles == 0) return cudaErrorInvalidConfiguration;
@@ -1131,7 +1198,7 @@ static cudaError_t launch_gemm_nt(GemmArgs ga, cudaStream_t s) {
     // tile's MMAs, cost more than the reuse saved; tile coordinates above the row tiles within
     // 32 bits)
     if (ga.n_chunks <= bs_chunks<NT, kParts>() && ga.n_mt >= 4u && (uint64_t)ga.n_items * ga.n_nt < (1ull << 32)) {
-        if ((e = gemm_grid<NT, kParts, true>(ga.n_tiles, &grid)) != cudaSuccess) return e;
+        if ((e = gemm_grid<NT, kParts, true, kLeaf>(ga.n_tiles, &grid)) != cudaSuccess) return e;
         ga.stages = bs_stages<NT, kParts>(ga.n_chunks);
         // Shared memory asked for leaves the rest of the SM's 256 KB as L1 cache. At 256 columns
         // and up to 32 summed entries the step is bound by C's stores, and the smallest cache
@@ -1142,25 +1209,25 @@ static cudaError_t launch_gemm_nt(GemmArgs ga, cudaStream_t s) {
         size_t bytes = kBsBytes;
         if (NT < 256 || ga.n_chunks > 2u) {
             if (NT >= 256) ga.stages = 3u;
-            bytes = ga.stages * a_bytes<kParts>() + ga.n_chunks * (bs_b_bytes<NT, kParts>() + 8u * kKq);
+            bytes = ga.stages * a_bytes<kParts>() + ga.n_chunks * (bs_b_bytes<NT, kParts>() + 12u * kKq);
         }
-        gemm_tc_bs_kernel<NT, kParts><<<(unsigned)grid, block_threads<NT>(), bytes, s>>>(ga);
+        gemm_tc_bs_kernel<NT, kParts, kLeaf><<<(unsigned)grid, block_threads<NT>(), bytes, s>>>(ga);
         return cudaGetLastError();
     }
     // dynamic shared memory: the operand stage ring and the summed index tables, sized for the largest summed index (1024 entries)
-    if ((e = gemm_grid<NT, kParts, false>(ga.n_tiles, &grid)) != cudaSuccess) return e;
-    gemm_tc_kernel<NT, kParts><<<(unsigned)grid, (int)block_threads<NT>(), smem_bytes<NT, kParts>(1024), s>>>(ga);
+    if ((e = gemm_grid<NT, kParts, false, kLeaf>(ga.n_tiles, &grid)) != cudaSuccess) return e;
+    gemm_tc_kernel<NT, kParts, kLeaf><<<(unsigned)grid, (int)block_threads<NT>(), smem_bytes<NT, kParts>(1024), s>>>(ga);
     return cudaGetLastError();
 }
 
-template <int kParts>
+template <int kParts, bool kLeaf>
 static cudaError_t launch_gemm_split(const GemmArgs &ga, uint32_t nt_cols, cudaStream_t s) {
     switch (nt_cols) {
-        case 16: return launch_gemm_nt<16, kParts>(ga, s);
-        case 32: return launch_gemm_nt<32, kParts>(ga, s);
-        case 64: return launch_gemm_nt<64, kParts>(ga, s);
-        case 128: return launch_gemm_nt<128, kParts>(ga, s);
-        default: return launch_gemm_nt<256, kParts>(ga, s);
+        case 16: return launch_gemm_nt<16, kParts, kLeaf>(ga, s);
+        case 32: return launch_gemm_nt<32, kParts, kLeaf>(ga, s);
+        case 64: return launch_gemm_nt<64, kParts, kLeaf>(ga, s);
+        case 128: return launch_gemm_nt<128, kParts, kLeaf>(ga, s);
+        default: return launch_gemm_nt<256, kParts, kLeaf>(ga, s);
     }
 }
 

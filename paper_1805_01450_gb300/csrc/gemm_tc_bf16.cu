@@ -4,7 +4,7 @@
 namespace qvx {
 
 cudaError_t launch_gemm_bf16(const GemmArgs &ga, uint32_t nt_cols, cudaStream_t s) {
-    return launch_gemm_split<3>(ga, nt_cols, s);
+    return launch_gemm_split<3, false>(ga, nt_cols, s);
 }
 
 }  // namespace qvx

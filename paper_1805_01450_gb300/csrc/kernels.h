@@ -133,10 +133,12 @@ cudaError_t launch_counted(cudaError_t e);
 struct GemmScale {
     const uint32_t *max_a, *max_b;       // per work item of the launch (max_c of the operand's step); null: a leaf
     uint32_t leaf_max_a, leaf_max_b;     // the same bits of a leaf operand
+    uint32_t leaf_max_d;                 // and of the leaf multiplied in (GemmLeaf)
 };
 uint32_t gemm_nt(const GemmStep &g);
-cudaError_t launch_gemm_step(const LaunchArgs &a, const GemmStep &g, const GemmScale *scale, uint32_t *max_c, int64_t item0,
-                             int64_t n_items, float2 *arenas, cudaStream_t s);
+// With `leaf` (fp16 parts only) the step is two contractions in one (GemmLeaf).
+cudaError_t launch_gemm_step(const LaunchArgs &a, const GemmStep &g, const GemmLeaf *leaf, const GemmScale *scale,
+                             uint32_t *max_c, int64_t item0, int64_t n_items, float2 *arenas, cudaStream_t s);
 // Self-test of the bounded waits (grid barrier and mbarrier that can never complete).
 cudaError_t launch_wait_selftest(unsigned *words, unsigned *status, uint32_t polls, unsigned *out, cudaStream_t s);
 

@@ -50,6 +50,16 @@ struct PTensor {
     int64_t offset = 0;                         // arena offset (complex64 entries)
 };
 
+// A step that runs as one tensor-core GEMM with its consumer, the contraction of its output
+// with a leaf (consumer >= 0), or is run by its operand's producer (absorbed).
+struct GemmPair {
+    int consumer = -1;
+    bool absorbed = false;
+    bool swap = false;               // the row operand is the step's B
+    GemmStep g{};
+    GemmLeaf leaf{};
+};
+
 struct Plan {
     qvx_plan_opts opts{};
     Model model;
@@ -81,6 +91,7 @@ struct Plan {
     int n_max_slots = 0;
     std::vector<uint32_t> leaf_max;
     std::vector<char> gemm_swap;               // per step: the GEMM's row operand is the step's B
+    std::vector<GemmPair> pairs;               // per step (stepwise engine with tensor cores, else empty)
     std::vector<GemmStep> gemm;                // per step, stepwise engine with tensor cores: GEMM form (nk > 0)
     // gradient program
     int n_params = 0;

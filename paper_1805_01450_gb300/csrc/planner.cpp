@@ -801,8 +801,14 @@ int64_t allocate_arena(Plan &p) {
     };
     // steps of one phase run concurrently: their outputs are placed while every operand of
     // the phase is still live, and the operands are released after the phase
+    auto absorbed = [&](int s) { return !p.pairs.empty() && p.pairs[s].absorbed; };
     for (const auto &ph : p.phases) {
-        for (int s = ph.first; s < ph.second; s++) alloc(p.steps[s].c);
+        for (int s = ph.first; s < ph.second; s++) {
+            if (!absorbed(s)) alloc(p.steps[s].c);
+            // a pair writes its consumer's output: live from here, so that the program may run
+            // step by step or with its pairs
+            if (!p.pairs.empty() && p.pairs[s].consumer >= 0) alloc(p.steps[p.pairs[s].consumer].c);
+        }
         for (int s = ph.first; s < ph.second; s++) {
             const PStep &st = p.steps[s];
             if (p.tensors[st.a].leaf < 0) release(st.a);
@@ -1238,6 +1244,97 @@ bool build_grad_tables(const Plan &p, std::vector<GradEntry> *ent, std::vector<u
     return true;
 }
 
+// The groups of a tensor-core step with output modes LC, row operand LA, column operand LB and
+// summed modes K (bit-run maps of each group in each tensor); false if a map needs too many
+// runs. Modes that an operand lacks contribute nothing to its address.
+bool gemm_groups(const std::vector<int> &gb, const std::vector<int> &gm, const std::vector<int> &gn,
+                 const std::vector<int> &K, const std::vector<int> &LA, const std::vector<int> &LB,
+                 const std::vector<int> &LC, GemmStep *g) {
+    auto gmap = [&](const std::vector<int> &grp, const std::vector<int> &L, DevRun *runs, uint8_t *n) {
+        DevRun r[kMaxRuns];
+        uint8_t nr = 0;
+        if (!map_runs(grp, L, r, &nr) || nr > kGroupRuns) return false;
+        for (int i = 0; i < nr; i++) runs[i] = r[i];
+        *n = nr;
+        return true;
+    };
+    g->nb = (uint8_t)gb.size();
+    g->nm = (uint8_t)gm.size();
+    g->nn = (uint8_t)gn.size();
+    g->nk = (uint8_t)K.size();
+    return gmap(gb, LA, g->ab, &g->n_ab) && gmap(gm, LA, g->am, &g->n_am) && gmap(K, LA, g->ak, &g->n_ak) &&
+           gmap(gb, LB, g->bb, &g->n_bb) && gmap(gn, LB, g->bn, &g->n_bn) && gmap(K, LB, g->bk, &g->n_bk) &&
+           gmap(gb, LC, g->cb, &g->n_cb) && gmap(gm, LC, g->cm, &g->n_cm) && gmap(gn, LC, g->cn, &g->n_cn);
+}
+
+// Pairs of steps that run as one tensor-core GEMM (stepwise engine, opts.tensor_cores, fp16
+// parts): X = sum_k A B, and E = sum_J X D with a leaf D over modes of X, where both A and B
+// hold the modes J (batch modes of the first step). Then E = sum_{k, J} A (D B): D is multiplied
+// into one operand while it is staged, J joins the summed index, and X, which is 2^|J| times E
+// and only exists to be summed, is neither written nor read. The result must have the
+// tensor-core form (row role at E's lowest mode, 128 rows, 8 columns, 8 to 512 summed entries,
+// 5 flops per byte of A, B and E). D goes with the operand that leaves the fewest batch modes
+// (its modes held by the other operand alone become batch modes); if equal, with the columns,
+// whose staged operand the row tiles may share. Slice terms of 8x8x40 circuits: 5001 27.4 -> 23.4
+// ms, 5002 42.1 -> 27.4, 5003 17.0 -> 9.1 (X alone moved 34, 94 and 48 GB).
+void find_pairs(Plan &p) {
+    p.pairs.assign(p.steps.size(), GemmPair{});
+    for (size_t t = 0; t < p.steps.size(); t++) {
+        const PStep &q = p.steps[t];
+        if (q.b < 0 || !q.k_a.empty() || !q.k_b.empty() || q.k_ab.empty()) continue;
+        const bool a_leaf = p.tensors[q.a].leaf >= 0, b_leaf = p.tensors[q.b].leaf >= 0;
+        if (a_leaf == b_leaf) continue;
+        const PTensor &X = p.tensors[a_leaf ? q.b : q.a], &D = p.tensors[a_leaf ? q.a : q.b];
+        const int s = X.producer;
+        if (s < 0) continue;
+        const PStep &st = p.steps[s];
+        if (st.b < 0 || !st.k_a.empty() || !st.k_b.empty() || p.pairs[s].absorbed) continue;
+        const std::vector<int> &MA = p.tensors[st.a].modes, &MB = p.tensors[st.b].modes, &E = p.tensors[q.c].modes;
+        if (!is_subset(D.modes, X.modes) || !is_subset(q.k_ab, MA) || !is_subset(q.k_ab, MB) || E.empty()) continue;
+        std::vector<int> K = st.k_ab;
+        K.insert(K.end(), q.k_ab.begin(), q.k_ab.end());
+        if (K.size() < 3 || K.size() > 9) continue;
+        const double flops = 8.0 * std::ldexp(1.0, (int)(E.size() + K.size()));
+        const double bytes = 8.0 * (std::ldexp(1.0, (int)MA.size()) + std::ldexp(1.0, (int)MB.size()) +
+                                    std::ldexp(1.0, (int)E.size()));
+        if (flops < 5.0 * bytes) continue;
+        GemmPair best;
+        for (int d_on_b = 0; d_on_b < 2; d_on_b++) {   // D with A, then with B
+            auto in_d = [&](int v) { return find_pos(D.modes, v) >= 0; };
+            auto in_a = [&](int v) { return find_pos(MA, v) >= 0 || (!d_on_b && in_d(v)); };
+            auto in_b = [&](int v) { return find_pos(MB, v) >= 0 || (d_on_b && in_d(v)); };
+            if (in_a(E[0]) == in_b(E[0])) continue;
+            const bool swap = in_b(E[0]);   // the step's B takes the row role
+            std::vector<int> gb, gm, gn;
+            for (int v : E) {
+                const bool row = swap ? in_b(v) : in_a(v), col = swap ? in_a(v) : in_b(v);
+                (row && col ? gb : (row ? gm : gn)).push_back(v);
+            }
+            if (gm.size() < 7 || gn.size() < 3) continue;
+            GemmPair c;
+            c.consumer = (int)t;
+            c.swap = swap;
+            if (!gemm_groups(gb, gm, gn, K, swap ? MB : MA, swap ? MA : MB, E, &c.g)) continue;
+            c.leaf.on_rows = (d_on_b != 0) == swap;
+            auto dmap = [&](const std::vector<int> &grp, DevRun *runs, uint8_t *n) {
+                DevRun r[kMaxRuns];
+                uint8_t nr = 0;
+                if (!map_runs(grp, D.modes, r, &nr) || nr > kGroupRuns) return false;
+                for (int i = 0; i < nr; i++) runs[i] = r[i];
+                *n = nr;
+                return true;
+            };
+            if (!dmap(gb, c.leaf.b, &c.leaf.n_b) || !dmap(c.leaf.on_rows ? gm : gn, c.leaf.r, &c.leaf.n_r) ||
+                !dmap(K, c.leaf.k, &c.leaf.n_k))
+                continue;
+            if (best.consumer < 0 || c.g.nb < best.g.nb || (c.g.nb == best.g.nb && best.leaf.on_rows)) best = c;
+        }
+        if (best.consumer < 0) continue;
+        p.pairs[s] = best;
+        p.pairs[t].absorbed = true;
+    }
+}
+
 bool serialize(Plan &p, std::string *err) {
     const Model &m = p.model;
     // leaf element maps and stored data
@@ -1440,18 +1537,7 @@ bool serialize(Plan &p, std::string *err) {
             const double bytes = 8.0 * (std::ldexp(1.0, (int)LA.size()) + std::ldexp(1.0, (int)LB.size()) +
                                         std::ldexp(1.0, (int)LC.size()));
             if (flops < 5.0 * bytes) continue;
-            bool ok = true;
-            auto gmap = [&](const std::vector<int> &grp, const std::vector<int> &L, DevRun *runs, uint8_t *n) {
-                DevRun r[kMaxRuns];
-                uint8_t nr = 0;
-                if (!map_runs(grp, L, r, &nr) || nr > kGroupRuns) { ok = false; return; }
-                for (int i = 0; i < nr; i++) runs[i] = r[i];
-                *n = nr;
-            };
-            gmap(gb, LA, g.ab, &g.n_ab); gmap(gm, LA, g.am, &g.n_am); gmap(st.k_ab, LA, g.ak, &g.n_ak);
-            gmap(gb, LB, g.bb, &g.n_bb); gmap(gn, LB, g.bn, &g.n_bn); gmap(st.k_ab, LB, g.bk, &g.n_bk);
-            gmap(gb, LC, g.cb, &g.n_cb); gmap(gm, LC, g.cm, &g.n_cm); gmap(gn, LC, g.cn, &g.n_cn);
-            if (!ok) { std::memset(&g, 0, sizeof(g)); continue; }
+            if (!gemm_groups(gb, gm, gn, st.k_ab, LA, LB, LC, &g)) { std::memset(&g, 0, sizeof(g)); continue; }
             p.gemm_swap[s] = swap ? 1 : 0;
             g.a_off = swap ? ds[s].b_off : ds[s].a_off;
             g.b_off = swap ? ds[s].a_off : ds[s].b_off;
@@ -1459,11 +1545,29 @@ bool serialize(Plan &p, std::string *err) {
             g.flags = ds[s].flags & ~(kStepALeaf | kStepBLeaf);
             if (ds[s].flags & (swap ? kStepBLeaf : kStepALeaf)) g.flags |= kStepALeaf;
             if (ds[s].flags & (swap ? kStepALeaf : kStepBLeaf)) g.flags |= kStepBLeaf;
-            g.nb = (uint8_t)gb.size();
-            g.nm = (uint8_t)gm.size();
-            g.nn = (uint8_t)gn.size();
-            g.nk = (uint8_t)st.k_ab.size();
         }
+    }
+    // the pairs' operands, now that leaves and offsets are numbered
+    std::vector<StepPair> prs;
+    for (size_t s = 0; s < p.pairs.size(); s++) {
+        GemmPair &pr = p.pairs[s];
+        if (pr.consumer < 0) continue;
+        const PStep &q = p.steps[pr.consumer];
+        GemmStep &g = pr.g;
+        g.a_off = pr.swap ? ds[s].b_off : ds[s].a_off;
+        g.b_off = pr.swap ? ds[s].a_off : ds[s].b_off;
+        g.c_off = ds[pr.consumer].c_off;
+        g.flags = 0;
+        if (ds[s].flags & (pr.swap ? kStepBLeaf : kStepALeaf)) g.flags |= kStepALeaf;
+        if (ds[s].flags & (pr.swap ? kStepALeaf : kStepBLeaf)) g.flags |= kStepBLeaf;
+        pr.leaf.leaf = (uint32_t)dev_leaf[p.tensors[p.tensors[q.a].leaf >= 0 ? q.a : q.b].leaf];
+        StepPair rec;
+        std::memset(&rec, 0, sizeof(rec));
+        rec.producer = (uint32_t)s;
+        rec.consumer = (uint32_t)pr.consumer;
+        rec.g = g;
+        rec.leaf = pr.leaf;
+        prs.push_back(rec);
     }
     // the operands of tensor-core steps whose largest entry the two-part split needs
     p.max_slot.assign(p.tensors.size(), -1);
@@ -1471,7 +1575,7 @@ bool serialize(Plan &p, std::string *err) {
     p.leaf_max.clear();
     if (p.fp16_split) {
         for (size_t s = 0; s < gms.size(); s++) {
-            if (gms[s].nk == 0) continue;
+            if (p.pairs[s].absorbed || (gms[s].nk == 0 && p.pairs[s].consumer < 0)) continue;
             for (int t : {p.steps[s].a, p.steps[s].b})
                 if (p.tensors[t].leaf < 0 && p.max_slot[t] < 0) p.max_slot[t] = p.n_max_slots++;
         }
@@ -1608,6 +1712,11 @@ bool serialize(Plan &p, std::string *err) {
         h.gemm_off = off;
         off = align256(off + gms.size() * sizeof(GemmStep));
     }
+    if (!prs.empty()) {
+        h.pairs_off = off;
+        h.n_pairs = (uint32_t)prs.size();
+        off = align256(off + prs.size() * sizeof(StepPair));
+    }
     // level phases (first step of each phase, then the step count)
     std::vector<uint32_t> level_first;
     for (const auto &ph : p.phases) level_first.push_back((uint32_t)ph.first);
@@ -1702,6 +1811,7 @@ bool serialize(Plan &p, std::string *err) {
     p.regtile = rts;
     if (!gms.empty()) std::memcpy(p.image.data() + h.gemm_off, gms.data(), gms.size() * sizeof(GemmStep));
     p.gemm = gms;
+    if (!prs.empty()) std::memcpy(p.image.data() + h.pairs_off, prs.data(), prs.size() * sizeof(StepPair));
     if (p.opts.gradient) {
         unsigned char *img = p.image.data();
         if (!p.grad_steps.empty()) std::memcpy(img + h.grad_steps_off, p.grad_steps.data(), p.grad_steps.size() * sizeof(GenStep));
@@ -1736,6 +1846,7 @@ bool build_program(Plan &p, std::string *err) {
     p.leaves.clear();
     p.tensors.clear();
     p.steps.clear();
+    p.pairs.clear();
     p.final_tensor = -1;
     ProgramBuilder b(p, p.model);
     if (!b.run()) { *err = b.err; return false; }
@@ -2018,6 +2129,11 @@ qvx_status plan_once(const qvx_circuit *c, const int32_t *order, int32_t n_order
         return QVX_EUNSUPPORTED;
     }
     if (p->engine == QVX_ENGINE_PERSISTENT) p->arena_elems = allocate_arena_unique(*p);
+    if (p->engine == QVX_ENGINE_STEPWISE && opts.tensor_cores) {
+        if (p->fp16_split) find_pairs(*p);
+        else p->pairs.assign(p->steps.size(), GemmPair{});
+        p->arena_elems = allocate_arena(*p);
+    }
     if (!serialize(*p, err)) return QVX_EUNSUPPORTED;
     if (p->engine == QVX_ENGINE_FUSED &&
         reinterpret_cast<const DevProgram *>(p->image.data())->fused_steps_off == 0 && !p->steps.empty()) {
