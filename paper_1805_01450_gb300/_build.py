@@ -11,7 +11,7 @@ OUT = os.path.join(HERE, "libqvx.so")
 BUILD = os.path.join(ROOT, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 HOST_SOURCES = ["planner.cpp", "capi.cpp"]
-CUDA_SOURCES = ["kernels.cu", "noalloc.cu", "gemm_tc.cu", "gemm_tc_leaf.cu", "gemm_tc_bf16.cu"]
+CUDA_SOURCES = ["kernels.cu", "noalloc.cu", "gemm_tc.cu", "gemm_tc_leaf.cu", "gemm_tc_reduce.cu", "gemm_tc_bf16.cu"]
 HEADERS = ["plan.h", "device_program.h", "kernels.h", "plan_handle.h", "device_util.cuh", "gemm_tc.cuh"]
 
 

@@ -228,11 +228,13 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
         return QVX_OK;
     }
     auto paired = [&](int s) { return !p.pairs.empty() && p.pairs[s].consumer >= 0; };
+    auto reduced = [&](int s) { return !p.reduces.empty() && p.reduces[s].producer >= 0; };
     auto cost = [&](size_t s, int64_t n, double *fl, double *by) {
         qvx::step_cost(p, s, fl, by);
-        if (paired((int)s)) {   // one launch for both steps' work
+        const int with = paired((int)s) ? p.pairs[s].consumer : (reduced((int)s) ? p.reduces[s].producer : -1);
+        if (with >= 0) {   // one launch for both steps' work
             double f2, b2;
-            qvx::step_cost(p, (size_t)p.pairs[s].consumer, &f2, &b2);
+            qvx::step_cost(p, (size_t)with, &f2, &b2);
             *fl += f2;
             *by += b2;
         }
@@ -265,7 +267,15 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
         cudaError_t r;
         uint32_t *mc = max_of(p.steps[paired(s) ? p.pairs[s].consumer : s].c);
         qvx::GemmScale sc{};
-        if (paired(s)) r = qvx::launch_gemm_step(a, p.pairs[s].g, &p.pairs[s].leaf, scale_of(s, &sc), mc, ib, n, arenas, st);
+        if (reduced(s)) {
+            const qvx::GemmReduce &rd = p.reduces[s];
+            const qvx::PStep &ps = p.steps[rd.producer];
+            sc.max_a = max_of(rd.swap ? ps.b : ps.a);
+            sc.max_b = max_of(rd.swap ? ps.a : ps.b);
+            sc.leaf_max_a = (rd.r.flags & qvx::kStepALeaf) ? p.leaf_max[rd.r.a_off] : 0u;
+            sc.leaf_max_b = (rd.r.flags & qvx::kStepBLeaf) ? p.leaf_max[rd.r.b_off] : 0u;
+            r = qvx::launch_reduce_step(a, rd.r, sc, max_of(p.steps[s].c), ib, n, arenas, st);
+        } else if (paired(s)) r = qvx::launch_gemm_step(a, p.pairs[s].g, &p.pairs[s].leaf, scale_of(s, &sc), mc, ib, n, arenas, st);
         else if (kind == QVX_KERNEL_GEMM_TC)
             r = qvx::launch_gemm_step(a, p.gemm[s], nullptr, scale_of(s, &sc), mc, ib, n, arenas, st);
         else if (kind == QVX_KERNEL_SPLITK) r = qvx::launch_splitk_step(a, (uint32_t)s, ib, n, arenas, rc, mc, st);
@@ -294,7 +304,8 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
                 const uint64_t threads = (uint64_t)n << rc;
                 const bool splitk = sh.nk >= 5 && rc <= 12;
                 if (!p.pairs.empty() && p.pairs[s].absorbed) continue;   // its operand's producer runs it
-                if (paired(s) || (!p.gemm.empty() && p.gemm[s].nk > 0)) {   // tensor cores
+                if (!p.reduces.empty() && p.reduces[s].merged) continue;    // its consumer runs it
+                if (paired(s) || reduced(s) || (!p.gemm.empty() && p.gemm[s].nk > 0)) {   // tensor cores
                     if ((e = single(s, QVX_KERNEL_GEMM_TC, ib, n)) != cudaSuccess)
                         return cuda_fail(e, "tensor-core step launch");
                     continue;

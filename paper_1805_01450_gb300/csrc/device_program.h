@@ -150,6 +150,29 @@ struct StepPair {
     GemmLeaf leaf;
 };
 
+// A tensor-core step whose result X = sum_k A B is multiplied by a tensor D and summed over the
+// modes J at once (E = sum_J X D; stepwise engine): where each mode of X goes in the tiles of
+// gemm_tc_reduce_kernel. Index groups: row (7 bits), col (7: jc of J lowest), unit (nu), mo
+// (row modes walked inside a unit), jo (J outside the tile, the jb bits that B holds highest),
+// k (nk). A map moves a group's compact index into a tensor's entry index.
+constexpr uint32_t kReduceDLeaf = 8;   // flags: D is a leaf (A and B as kStepALeaf, kStepBLeaf)
+struct ModeMap {
+    uint8_t n, pad[3];
+    DevRun runs[kGroupRuns];
+};
+struct ReduceStep {
+    uint64_t a_off, b_off, d_off, e_off;   // arena offsets or leaf indices
+    uint32_t flags;
+    uint8_t nk, nu, mo, jo, jb, jc, pad[2];
+    ModeMap row_a, row_d, row_e, col_b, col_d, col_e, unit_a, unit_b, unit_d, unit_e, mo_a, mo_d, mo_e, jo_a, jo_b, jo_d,
+        k_a, k_b;                          // col_e: of the kept columns (col >> jc)
+};
+// In the image: step `producer` (X) and step `consumer` (E) run as one.
+struct StepReduce {
+    uint32_t producer, consumer;
+    ReduceStep r;
+};
+
 struct DevProgram {
     uint32_t magic;
     uint32_t n_steps, n_leaves, pad0;
@@ -187,7 +210,8 @@ struct DevProgram {
     uint64_t image_bytes;
     uint64_t zero_mask_hi;         // qubits 64..127 of the zero mask
     uint64_t pairs_off;            // byte offset of n_pairs StepPair (0 if none)
-    uint32_t n_pairs, pad1;
+    uint32_t n_pairs, n_reduces;
+    uint64_t reduces_off;          // byte offset of n_reduces StepReduce (0 if none)
 };
 
 constexpr uint32_t kProgramMagic = 0x51565831u;  // "QVX1"
@@ -197,8 +221,9 @@ constexpr uint32_t kProgramMagic = 0x51565831u;  // "QVX1"
 namespace qvx {
 static_assert(sizeof(DevStep) == 136, "DevStep layout");
 static_assert(sizeof(DevLeaf) == 40, "DevLeaf layout");
-static_assert(sizeof(DevProgram) == 344, "DevProgram layout");
+static_assert(sizeof(DevProgram) == 352, "DevProgram layout");
 static_assert(sizeof(GemmLeaf) == 104 && sizeof(StepPair) == 448, "StepPair layout");
+static_assert(sizeof(ReduceStep) == 696 && sizeof(StepReduce) == 704, "StepReduce layout");
 static_assert(sizeof(GemmStep) == 336, "GemmStep layout");
 static_assert(sizeof(GradEntry) == 16, "GradEntry layout");
 static_assert(sizeof(RegTileStep) == 288, "RegTileStep layout");

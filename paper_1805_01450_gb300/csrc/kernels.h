@@ -139,6 +139,10 @@ uint32_t gemm_nt(const GemmStep &g);
 // With `leaf` (fp16 parts only) the step is two contractions in one (GemmLeaf).
 cudaError_t launch_gemm_step(const LaunchArgs &a, const GemmStep &g, const GemmLeaf *leaf, const GemmScale *scale,
                              uint32_t *max_c, int64_t item0, int64_t n_items, float2 *arenas, cudaStream_t s);
+// A contraction and the sum of its result times another tensor in one launch (gemm_tc_reduce.cu);
+// scale.max_a and max_b as for launch_gemm_step, max_c of the second step's output.
+cudaError_t launch_reduce_step(const LaunchArgs &a, const ReduceStep &r, const GemmScale &scale, uint32_t *max_c,
+                               int64_t item0, int64_t n_items, float2 *arenas, cudaStream_t s);
 // Self-test of the bounded waits (grid barrier and mbarrier that can never complete).
 cudaError_t launch_wait_selftest(unsigned *words, unsigned *status, uint32_t polls, unsigned *out, cudaStream_t s);
 

@@ -60,6 +60,16 @@ struct GemmPair {
     GemmLeaf leaf{};
 };
 
+// A step that runs together with the producer of its operand X (producer >= 0: X is not
+// stored), or whose result is only made inside its consumer (merged).
+struct GemmReduce {
+    int producer = -1;
+    bool merged = false;
+    bool swap = false;               // the row operand is the producer's B
+    int d = -1;                      // the other operand's tensor
+    ReduceStep r{};
+};
+
 struct Plan {
     qvx_plan_opts opts{};
     Model model;
@@ -92,6 +102,7 @@ struct Plan {
     std::vector<uint32_t> leaf_max;
     std::vector<char> gemm_swap;               // per step: the GEMM's row operand is the step's B
     std::vector<GemmPair> pairs;               // per step (stepwise engine with tensor cores, else empty)
+    std::vector<GemmReduce> reduces;           // per step (stepwise engine with tensor cores, else empty)
     std::vector<GemmStep> gemm;                // per step, stepwise engine with tensor cores: GEMM form (nk > 0)
     // gradient program
     int n_params = 0;

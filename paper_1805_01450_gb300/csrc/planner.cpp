@@ -810,9 +810,15 @@ int64_t allocate_arena(Plan &p) {
             if (!p.pairs.empty() && p.pairs[s].consumer >= 0) alloc(p.steps[p.pairs[s].consumer].c);
         }
         for (int s = ph.first; s < ph.second; s++) {
+            if (!p.reduces.empty() && p.reduces[s].merged) continue;   // its operands are read in its consumer's phase
             const PStep &st = p.steps[s];
             if (p.tensors[st.a].leaf < 0) release(st.a);
             if (st.b >= 0 && p.tensors[st.b].leaf < 0) release(st.b);
+            if (!p.reduces.empty() && p.reduces[s].producer >= 0) {
+                const PStep &ps = p.steps[p.reduces[s].producer];
+                if (p.tensors[ps.a].leaf < 0) release(ps.a);
+                if (p.tensors[ps.b].leaf < 0) release(ps.b);
+            }
         }
     }
     return peak;
@@ -1335,6 +1341,97 @@ void find_pairs(Plan &p) {
     }
 }
 
+// Steps that run as one gemm_tc_reduce_kernel (stepwise engine, opts.tensor_cores, fp16 parts):
+// E = sum_J X D with X = sum_k A B, where X has the largest part of both steps' memory traffic
+// (at least twice A, B and E together, and 2^18 entries: below, X stays in L2). Needed for the
+// kernel's tiles: seven row modes that E keeps, seven column modes of which two to four are in J,
+// and B's chunks for all its values of J within shared memory. Modes that D lacks come first
+// in the units, so that units reading the same entries of D run together.
+void find_reduces(Plan &p) {
+    p.reduces.assign(p.steps.size(), GemmReduce{});
+    for (size_t t = 0; t < p.steps.size(); t++) {
+        const PStep &q = p.steps[t];
+        if (q.b < 0 || !q.k_a.empty() || !q.k_b.empty() || q.k_ab.empty() || p.pairs[t].absorbed || p.pairs[t].consumer >= 0)
+            continue;
+        GemmReduce best;
+        double best_size = 0;
+        for (int side = 0; side < 2; side++) {   // X as the step's A, as its B
+            const PTensor &X = p.tensors[side ? q.b : q.a];
+            const int dt = side ? q.a : q.b;
+            const std::vector<int> &D = p.tensors[dt].modes, &E = p.tensors[q.c].modes;
+            const int s = X.producer;
+            if (s < 0 || E.empty() || X.modes.size() < 18 || !is_subset(D, X.modes)) continue;
+            const PStep &st = p.steps[s];
+            if (st.b < 0 || !st.k_a.empty() || !st.k_b.empty() || st.k_ab.size() < 3 || st.k_ab.size() > 6) continue;
+            if (p.pairs[s].absorbed || p.pairs[s].consumer >= 0 || p.reduces[s].merged || p.reduces[s].producer >= 0) continue;
+            const std::vector<int> &MA = p.tensors[st.a].modes, &MB = p.tensors[st.b].modes;
+            const double size = std::ldexp(1.0, (int)X.modes.size());
+            const double rest = std::ldexp(1.0, (int)MA.size()) + std::ldexp(1.0, (int)MB.size()) + std::ldexp(1.0, (int)E.size());
+            if (size < 2.0 * rest) continue;
+            auto in = [](const std::vector<int> &v, int x) { return find_pos(v, x) >= 0; };
+            if (in(MA, E[0]) == in(MB, E[0])) continue;
+            GemmReduce c;
+            c.producer = s;
+            c.d = dt;
+            c.swap = in(MB, E[0]);
+            const std::vector<int> &R = c.swap ? MB : MA, &C = c.swap ? MA : MB;   // row and column operands
+            std::vector<int> row, col, unit, mo, jo, jn, jb, kn, ub, un;
+            for (int v : E) {
+                if (in(R, v) && !in(C, v)) (row.size() < 7 ? row : mo).push_back(v);
+                else if (!in(R, v)) kn.push_back(v);
+                else (in(D, v) ? un : ub).push_back(v);   // a batch mode: those that D lacks first
+            }
+            for (int v : q.k_ab) {
+                if (in(R, v) && !in(C, v)) jo.push_back(v);
+                else if (!in(R, v)) jn.push_back(v);
+                else jb.push_back(v);
+            }
+            const size_t jc = std::min<size_t>(4, jn.size());
+            if (row.size() < 7 || jc < 2 || kn.size() < 7 - jc) continue;
+            col.assign(jn.begin(), jn.begin() + jc);
+            jb.insert(jb.end(), jn.begin() + jc, jn.end());
+            std::vector<int> kept(kn.begin(), kn.begin() + (7 - jc));
+            col.insert(col.end(), kept.begin(), kept.end());
+            for (size_t i = 7 - jc; i < kn.size(); i++) (in(D, kn[i]) ? un : ub).push_back(kn[i]);
+            unit = ub;
+            unit.insert(unit.end(), un.begin(), un.end());
+            // enough units for every SM several times over
+            while (unit.size() < 7 && !mo.empty()) { unit.push_back(mo.back()); mo.pop_back(); }
+            if (((std::max<size_t>(16, size_t(1) << st.k_ab.size()) / 16) << jb.size()) > 4) continue;
+            if (unit.size() > 28 || jo.size() + jb.size() + mo.size() > 20) continue;
+            c.r.jb = (uint8_t)jb.size();
+            jo.insert(jo.end(), jb.begin(), jb.end());
+            c.r.nk = (uint8_t)st.k_ab.size();
+            c.r.nu = (uint8_t)unit.size();
+            c.r.mo = (uint8_t)mo.size();
+            c.r.jo = (uint8_t)jo.size();
+            c.r.jc = (uint8_t)jc;
+            auto map = [&](const std::vector<int> &grp, const std::vector<int> &L, ModeMap *m) {
+                DevRun r[kMaxRuns];
+                uint8_t nr = 0;
+                if (!map_runs(grp, L, r, &nr) || nr > kGroupRuns) return false;
+                for (int i = 0; i < nr; i++) m->runs[i] = r[i];
+                m->n = nr;
+                return true;
+            };
+            ReduceStep &r = c.r;
+            if (!map(row, R, &r.row_a) || !map(row, D, &r.row_d) || !map(row, E, &r.row_e) || !map(col, C, &r.col_b) ||
+                !map(col, D, &r.col_d) || !map(kept, E, &r.col_e) || !map(unit, R, &r.unit_a) || !map(unit, C, &r.unit_b) ||
+                !map(unit, D, &r.unit_d) || !map(unit, E, &r.unit_e) || !map(mo, R, &r.mo_a) || !map(mo, D, &r.mo_d) ||
+                !map(mo, E, &r.mo_e) || !map(jo, R, &r.jo_a) || !map(jo, C, &r.jo_b) || !map(jo, D, &r.jo_d) ||
+                !map(st.k_ab, R, &r.k_a) || !map(st.k_ab, C, &r.k_b))
+                continue;
+            if (size > best_size) {
+                best = c;
+                best_size = size;
+            }
+        }
+        if (best.producer < 0) continue;
+        p.reduces[t] = best;
+        p.reduces[best.producer].merged = true;
+    }
+}
+
 bool serialize(Plan &p, std::string *err) {
     const Model &m = p.model;
     // leaf element maps and stored data
@@ -1569,13 +1666,36 @@ bool serialize(Plan &p, std::string *err) {
         rec.leaf = pr.leaf;
         prs.push_back(rec);
     }
+    std::vector<StepReduce> reds;
+    for (size_t t = 0; t < p.reduces.size(); t++) {
+        GemmReduce &rd = p.reduces[t];
+        if (rd.producer < 0) continue;
+        const DevStep &x = ds[rd.producer];
+        ReduceStep &r = rd.r;
+        r.a_off = rd.swap ? x.b_off : x.a_off;
+        r.b_off = rd.swap ? x.a_off : x.b_off;
+        r.e_off = ds[t].c_off;
+        const bool d_is_a = rd.d == p.steps[t].a;
+        r.d_off = d_is_a ? ds[t].a_off : ds[t].b_off;
+        r.flags = 0;
+        if (x.flags & (rd.swap ? kStepBLeaf : kStepALeaf)) r.flags |= kStepALeaf;
+        if (x.flags & (rd.swap ? kStepALeaf : kStepBLeaf)) r.flags |= kStepBLeaf;
+        if (ds[t].flags & (d_is_a ? kStepALeaf : kStepBLeaf)) r.flags |= kReduceDLeaf;
+        StepReduce rec;
+        std::memset(&rec, 0, sizeof(rec));
+        rec.producer = (uint32_t)rd.producer;
+        rec.consumer = (uint32_t)t;
+        rec.r = r;
+        reds.push_back(rec);
+    }
     // the operands of tensor-core steps whose largest entry the two-part split needs
     p.max_slot.assign(p.tensors.size(), -1);
     p.n_max_slots = 0;
     p.leaf_max.clear();
     if (p.fp16_split) {
         for (size_t s = 0; s < gms.size(); s++) {
-            if (p.pairs[s].absorbed || (gms[s].nk == 0 && p.pairs[s].consumer < 0)) continue;
+            if (p.pairs[s].absorbed || (gms[s].nk == 0 && p.pairs[s].consumer < 0 && !p.reduces[s].merged)) continue;
+            if (p.reduces[s].producer >= 0) continue;
             for (int t : {p.steps[s].a, p.steps[s].b})
                 if (p.tensors[t].leaf < 0 && p.max_slot[t] < 0) p.max_slot[t] = p.n_max_slots++;
         }
@@ -1717,6 +1837,11 @@ bool serialize(Plan &p, std::string *err) {
         h.n_pairs = (uint32_t)prs.size();
         off = align256(off + prs.size() * sizeof(StepPair));
     }
+    if (!reds.empty()) {
+        h.reduces_off = off;
+        h.n_reduces = (uint32_t)reds.size();
+        off = align256(off + reds.size() * sizeof(StepReduce));
+    }
     // level phases (first step of each phase, then the step count)
     std::vector<uint32_t> level_first;
     for (const auto &ph : p.phases) level_first.push_back((uint32_t)ph.first);
@@ -1811,6 +1936,7 @@ bool serialize(Plan &p, std::string *err) {
     p.regtile = rts;
     if (!gms.empty()) std::memcpy(p.image.data() + h.gemm_off, gms.data(), gms.size() * sizeof(GemmStep));
     p.gemm = gms;
+    if (!reds.empty()) std::memcpy(p.image.data() + h.reduces_off, reds.data(), reds.size() * sizeof(StepReduce));
     if (!prs.empty()) std::memcpy(p.image.data() + h.pairs_off, prs.data(), prs.size() * sizeof(StepPair));
     if (p.opts.gradient) {
         unsigned char *img = p.image.data();
@@ -1847,6 +1973,7 @@ bool build_program(Plan &p, std::string *err) {
     p.tensors.clear();
     p.steps.clear();
     p.pairs.clear();
+    p.reduces.clear();
     p.final_tensor = -1;
     ProgramBuilder b(p, p.model);
     if (!b.run()) { *err = b.err; return false; }
@@ -2130,8 +2257,12 @@ qvx_status plan_once(const qvx_circuit *c, const int32_t *order, int32_t n_order
     }
     if (p->engine == QVX_ENGINE_PERSISTENT) p->arena_elems = allocate_arena_unique(*p);
     if (p->engine == QVX_ENGINE_STEPWISE && opts.tensor_cores) {
-        if (p->fp16_split) find_pairs(*p);
-        else p->pairs.assign(p->steps.size(), GemmPair{});
+        p->pairs.assign(p->steps.size(), GemmPair{});
+        p->reduces.assign(p->steps.size(), GemmReduce{});
+        if (p->fp16_split) {
+            find_pairs(*p);
+            find_reduces(*p);
+        }
         p->arena_elems = allocate_arena(*p);
     }
     if (!serialize(*p, err)) return QVX_EUNSUPPORTED;
