@@ -14,7 +14,10 @@
 // on different SMs and read D's entries through L2 together.
 //
 // Roles are those of the B-stationary form (gemm_tc.cuh). The epilogue holds its accumulators,
-// a block's columns and their D entries in registers, so it takes most of the register file.
+// a block's columns and two blocks' D entries in registers, so it takes most of the register
+// file. What bounds it is the latency of D's entries: 128 KB per tile with 32 to 64 KB in
+// flight per SM (DRAM 19 %, tensor pipe 18 %, LSU data pipe 19 % busy). Circuit 5001: 7.02 ms,
+// the two steps before 6.22 + 5.84; circuit 5002: 4.6 ms, before 3.64 + 3.12.
 #include "gemm_tc.cuh"
 
 namespace qvx {
@@ -251,16 +254,42 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_tc_reduce_kernel(ReduceArgs
         uint32_t doff[16];
 #pragma unroll
         for (uint32_t i = 0; i < 16u; i++) doff[i] = mv(i, r.col_d);
+        // tile cursor of D: a block's entries are loaded while the block before is summed (without
+        // that the merged step of circuit 5001 took 7.33 instead of 7.02 ms; with prefetches of
+        // D into L2 a tile ahead 8.6 ms by line, 16.6 ms by bulk prefetch of row runs)
+        uint64_t pu = blockIdx.x;
+        uint32_t pmo = 0, pjo = 0;
+        const float2 *pbase = nullptr;
+        auto d_unit = [&]() {
+            const int64_t il = (int64_t)(pu >> r.nu);
+            pbase = gemm_operand(ra.a, ra.arenas + (uint64_t)il * ra.a.arena_elems, r.d_off, r.flags & kReduceDLeaf, ra.item0 + il) +
+                    mv((uint32_t)pu & unit_mask, r.unit_d);
+        };
+        auto d_tile = [&]() { return pbase + mv(pmo, r.mo_d) + mv(pjo, r.jo_d); };
+        auto d_next = [&]() {   // past the last tile the cursor stays on it
+            if (++pjo < n_jb * n_jm) return;
+            pjo = 0;
+            if (++pmo < n_mo) return;
+            pmo = 0;
+            if (pu + gridDim.x < ra.n_units) {
+                pu += gridDim.x;
+                d_unit();
+            }
+        };
+        auto load_block = [&](float2 (&dv)[16], const float2 *dt, uint32_t b) {
+            const float2 *db = dt + mv((share + 2u * b) * 16u, r.col_d) + own_d;
+#pragma unroll
+            for (uint32_t i = 0; i < 16u; i++) dv[i] = db[doff[i]];
+        };
+        d_unit();
+        const float2 *dt = d_tile();   // the tile that is summed
+        float2 dv[2][16];
+        load_block(dv[0], dt, 0);
         uint32_t j = 0;
         bool ok = true;
         for (uint64_t u = blockIdx.x; u < ra.n_units && ok; u += gridDim.x) {
             const int64_t il = (int64_t)(u >> r.nu);
-            const uint32_t ui = (uint32_t)u & unit_mask;
-            float2 *arena = ra.arenas + (uint64_t)il * ra.a.arena_elems;
-            const float2 *dbase = gemm_operand(ra.a, arena, r.d_off, r.flags & kReduceDLeaf, ra.item0 + il) + mv(ui, r.unit_d) + own_d;
-            float2 *ebase = arena + r.e_off + mv(ui, r.unit_e) + own_e;
-            const Unscale un = unscale_of(operand_max(ra.sc.max_a, ra.sc.leaf_max_a, il),
-                                          operand_max(ra.sc.max_b, ra.sc.leaf_max_b, il), ra.n_chunks);
+            float2 *ebase = ra.arenas + (uint64_t)il * ra.a.arena_elems + r.e_off + mv((uint32_t)u & unit_mask, r.unit_e) + own_e;
             uint32_t largest = 0;
             for (uint32_t mo = 0; mo < n_mo && ok; mo++) {
                 float2 acc[4][kE];
@@ -268,43 +297,43 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_tc_reduce_kernel(ReduceArgs
                 for (uint32_t b = 0; b < 4u; b++)
 #pragma unroll
                     for (uint32_t e = 0; e < kE; e++) acc[b][e] = make_float2(0.f, 0.f);
-                const float2 *dmo = dbase + mv(mo, r.mo_d);
                 for (uint32_t jo = 0; jo < n_jb * n_jm; jo++, j++) {
                     const uint32_t buf = j & 1u;
-                    const float2 *dt = dmo + mv(jo, r.jo_d);
                     const uint32_t taddr = tmem + ((q * 32u) << 16) + buf * kNt;
+                    d_next();
+                    const float2 *dn = d_tile();
+                    if (!warp_wait_or_fail(smem_u32(&accf_bar[buf]), (j >> 1) & 1u, &fail)) {
+                        fail = 1;
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
 #pragma unroll
                     for (uint32_t b = 0; b < 4u; b++) {
-                        const uint32_t j0 = (share + 2u * b) * 16u;
-                        const float2 *db = dt + mv(j0, r.col_d);
-                        float2 dv[16];
+                        load_block(dv[(b + 1u) & 1u], b < 3u ? dt : dn, (b + 1u) & 3u);
 #pragma unroll
-                        for (uint32_t i = 0; i < 16u; i++) dv[i] = db[doff[i]];
-                        if (b == 0u) {
-                            if (!warp_wait_or_fail(smem_u32(&accf_bar[buf]), (j >> 1) & 1u, &fail)) {
-                                fail = 1;
-                                ok = false;
-                                break;
+                        for (uint32_t half = 0; half < 2u; half++) {
+                            uint32_t x[16];
+                            tmem_ld_pairs<16>(taddr + 2u * ((share + 2u * b) * 16u + 8u * half), x);
+#pragma unroll
+                            for (uint32_t i = 0; i < 8u; i++) {
+                                const float xr = __uint_as_float(x[2u * i]), xi = __uint_as_float(x[2u * i + 1u]);
+                                const float2 d = dv[b & 1u][8u * half + i];
+                                float2 &s = acc[b][(8u * half + i) >> JC];
+                                s.x = fmaf(xr, d.x, s.x);
+                                s.x = fmaf(-xi, d.y, s.x);
+                                s.y = fmaf(xr, d.y, s.y);
+                                s.y = fmaf(xi, d.x, s.y);
                             }
-                            tc_fence_after();
-                        }
-                        uint32_t x[32];
-                        tmem_ld_pairs<32>(taddr + 2u * j0, x);
-#pragma unroll
-                        for (uint32_t i = 0; i < 16u; i++) {
-                            const float xr = __uint_as_float(x[2u * i]), xi = __uint_as_float(x[2u * i + 1u]);
-                            float2 &s = acc[b][i >> JC];
-                            s.x = fmaf(xr, dv[i].x, s.x);
-                            s.x = fmaf(-xi, dv[i].y, s.x);
-                            s.y = fmaf(xr, dv[i].y, s.y);
-                            s.y = fmaf(xi, dv[i].x, s.y);
                         }
                     }
-                    if (!ok) break;
                     tc_fence_before();
                     warp_arrive(smem_u32(&acce_bar[buf]));
+                    dt = dn;
                 }
                 if (!ok) break;
+                const Unscale un = unscale_of(operand_max(ra.sc.max_a, ra.sc.leaf_max_a, il),
+                                              operand_max(ra.sc.max_b, ra.sc.leaf_max_b, il), ra.n_chunks);
                 float2 *emo = ebase + mv(mo, r.mo_e);
 #pragma unroll
                 for (uint32_t b = 0; b < 4u; b++)
