@@ -222,6 +222,17 @@ qvx_status qvx_amplitude(qvx_plan *plan, const uint64_t *bitstrings_dev, int64_t
 qvx_status qvx_amplitude_host(qvx_plan *plan, const uint64_t *bitstrings_host, int64_t batch, double *amps_host,
                               void *workspace_dev, size_t workspace_bytes, void *stream);
 
+/* Checks device bitstrings without waiting for the work already in the stream: qvx_bits_check
+ * enqueues one small kernel that looks for bits at or above n_qubits and returns a ticket;
+ * qvx_bits_result waits for that kernel only (not for anything enqueued after it), gives the
+ * ticket back and returns QVX_EINVAL if a bitstring had such bits. A program enqueues its calls
+ * between the two, so the stream does not run dry while the host waits: the calls read no bit
+ * at or above n_qubits, and their results are discarded if the check fails. Tickets come from a
+ * process-wide pool (at most 64 kept; safe from several threads and streams). Not during
+ * stream capture (QVX_ECUDA). */
+qvx_status qvx_bits_check(const qvx_plan *plan, const uint64_t *bitstrings_dev, int64_t batch, void *stream, int64_t *ticket);
+qvx_status qvx_bits_result(int64_t ticket);
+
 /* Sum of the slice terms s in [slice_begin, slice_begin + slice_count) only: the share of
  * one rank when the slices are split over several processes (Section 3.B.2). */
 qvx_status qvx_amplitude_slices(qvx_plan *plan, const uint64_t *bitstrings_dev, int64_t batch,

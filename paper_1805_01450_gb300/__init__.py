@@ -77,7 +77,7 @@ EXPORTED = ("qvx_plan_opts_default", "qvx_graph_export", "qvx_plan_create", "qvx
             "qvx_amplitude", "qvx_amplitude_slices", "qvx_slice_terms", "qvx_workspace_status",
             "qvx_last_error", "qvx_amplitude_noalloc", "qvx_amplitude_grad", "qvx_amplitude_host",
             "qvx_selftest_wait_timeout", "qvx_kernel_launches", "qvx_noalloc_status", "qvx_amplitude_profiled",
-            "qvx_profile_read", "qvx_kernel_name", "qvx_selftest_fused_timeout")
+            "qvx_profile_read", "qvx_kernel_name", "qvx_selftest_fused_timeout", "qvx_bits_check", "qvx_bits_result")
 
 
 def lib():
@@ -115,6 +115,8 @@ def lib():
         "qvx_profile_read": (ctypes.c_int, [P, ctypes.POINTER(LaunchRecord), i64, ctypes.POINTER(ctypes.c_int64)]),
         "qvx_kernel_name": (ctypes.c_char_p, [i32]),
         "qvx_selftest_fused_timeout": (ctypes.c_int, [P, P, i64, P, P, ctypes.c_size_t, P]),
+        "qvx_bits_check": (ctypes.c_int, [P, P, i64, P, ctypes.POINTER(i64)]),
+        "qvx_bits_result": (ctypes.c_int, [i64]),
     }
     for name, (res, args) in sig.items():
         f = getattr(L, name)
@@ -189,10 +191,27 @@ def bits_tensor(bitstrings, words, device=None):
     return t.contiguous().view(-1)
 
 
-def _stream_ptr(stream):
+def _current_stream():
+    """The current CUDA stream's handle as an integer (0: the default stream). torch's Stream
+    objects cost 3 us each to make, a third of the smallest call's launch, so the raw handle is
+    asked for where torch has it."""
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
+
+
+def _stream_ptr(stream):
+    return ctypes.c_void_p(_current_stream() if stream is None else stream.cuda_stream)
+
+
+def _as_complex(out, rows):
+    """The complex128 view of `rows` (re, im) pairs in a float64 tensor."""
+    import torch
+    if out.dtype == torch.float64 and out.dim() == 1 and out.is_contiguous() and out.numel() == 2 * rows and out.storage_offset() % 2 == 0:
+        return out.view(torch.complex128)
+    return torch.view_as_complex(out.view(rows, 2))
 
 
 class Plan:
@@ -293,33 +312,80 @@ class Plan:
     def _bits(self, bitstrings, device=None):
         return bits_tensor(bitstrings, self.words, device)
 
-    def _check_bits(self, bits):
+    def _check_host_bits(self, bitstrings):
+        """Refuses host bitstrings (Python ints, or a CPU tensor of words) with bits at or above
+        n_qubits; looks at the words that are uploaded."""
         import torch
-        w = bits.view(-1, self.words)
-        for j in range(self.words):
-            valid = self.n_qubits - 64 * j
-            if valid < 64 and bool(torch.any((w[:, j] >> valid) != 0)):
-                raise QvxError(QVX_EINVAL, "bitstring has bits at or above n_qubits")
+        bad = False
+        if isinstance(bitstrings, torch.Tensor):
+            w = bitstrings.reshape(-1, self.words)
+            for j in range(self.words):
+                valid = self.n_qubits - 64 * j
+                if valid < 64:
+                    bad = bad or bool(torch.any((w[:, j] >> valid) != 0))
+        else:
+            n, mask = self.n_qubits, (1 << (64 * self.words)) - 1
+            bad = any((int(b) & mask) >> n for b in bitstrings)
+        if bad:
+            raise QvxError(QVX_EINVAL, "bitstring has bits at or above n_qubits")
+
+    def _checked_bits(self, bitstrings, stream, first, validate=True):
+        """(device words, ticket). Host bitstrings are checked here; device ones by a kernel on
+        the current stream, whose result the caller asks for (qvx_bits_result) after it has
+        enqueued its own work. `first`: that work must not start on bitstrings that fail (it
+        writes into the caller's memory), or runs on another stream than the current one: the
+        result is waited for here."""
+        import torch
+        if isinstance(bitstrings, torch.Tensor) and bitstrings.is_cuda:
+            bits = self._bits(bitstrings)
+            if not validate:
+                return bits, -1
+            cur = _current_stream()
+            first = first or stream.value != (cur or None)
+            ticket = ctypes.c_int64(-1)
+            _check(lib().qvx_bits_check(self._h, bits.data_ptr(), bits.numel() // self.words, cur, ctypes.byref(ticket)))
+            if first:
+                _check(lib().qvx_bits_result(ticket))
+                return bits, -1
+            return bits, ticket.value
+        if not isinstance(bitstrings, torch.Tensor):
+            bitstrings = list(bitstrings)
+            if validate:
+                self._check_host_bits(bitstrings)
+            if bitstrings and stream.value == (_current_stream() or None):
+                # pageable words are staged by the driver before the call returns: no need to
+                # wait for the stream as well
+                words = torch.tensor(bitstring_words(bitstrings, self.words), dtype=torch.int64)
+                return words.to("cuda", non_blocking=True), -1
+            return self._bits(bitstrings), -1
+        bits = self._bits(bitstrings)
+        if validate:
+            self._check_host_bits(bitstrings)
+        return bits, -1
 
     def amplitude(self, bitstrings, workspace=None, out=None, stream=None, slice_begin=0,
                   slice_count=None, validate=True):
         """<x|C|0> for each bitstring: complex128 torch tensor on the bitstrings' device.
         slice_begin/slice_count restrict the sum to a range of slice numbers."""
         import torch
-        bits = self._bits(bitstrings)
-        if validate:
-            self._check_bits(bits)
-        n = bits.numel() // self.words
-        ws = workspace if workspace is not None else self._ws_for(n, bits.device)
-        m = 1 << self.n_open
-        if out is None:
-            out = torch.empty(2 * n * m, dtype=torch.float64, device=bits.device)
-        if slice_count is None:
-            slice_count = self.n_slice_terms - slice_begin
-        _check(lib().qvx_amplitude_slices(self._h, ctypes.c_void_p(bits.data_ptr()), n, slice_begin,
-                                          slice_count, ctypes.c_void_p(out.data_ptr()),
-                                          ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream_ptr(stream)))
-        a = torch.view_as_complex(out.view(n * m, 2))
+        sp = _stream_ptr(stream)
+        bits, ticket = self._checked_bits(bitstrings, sp, out is not None, validate)
+        try:
+            n = bits.numel() // self.words
+            ws = workspace if workspace is not None else self._ws_for(n, bits.device)
+            m = 1 << self.n_open
+            a = None
+            if out is None:
+                out = a = torch.empty(n * m, dtype=torch.complex128, device=bits.device)
+            if slice_count is None:
+                slice_count = self.n_slice_terms - slice_begin
+            _check(lib().qvx_amplitude_slices(self._h, bits.data_ptr(), n, slice_begin, slice_count, out.data_ptr(),
+                                              ws.data_ptr(), ws.numel(), sp))
+        finally:
+            if ticket >= 0:
+                _check(lib().qvx_bits_result(ticket))
+        if a is None:
+            a = _as_complex(out, n * m)
         return a.view(n, m) if self.n_open else a
 
     def amplitude_grad(self, bitstrings, thetas=None, workspace=None, stream=None):
@@ -327,25 +393,25 @@ class Plan:
         device, for a plan created with gradient=True. thetas: float64 tensor of n_params
         angles (any device) replacing the circuit's, or None."""
         import torch
-        bits = self._bits(bitstrings)
-        self._check_bits(bits)
+        sp = _stream_ptr(stream)
+        # the call rewrites the workspace's gate entries for these angles: only after the check
+        bits, _ = self._checked_bits(bitstrings, sp, True)
         n = bits.numel() // self.words
         npar = self.info["n_params"]
         ws = workspace if workspace is not None else self._ws_for(n, bits.device)
-        amps = torch.empty(2 * n, dtype=torch.float64, device=bits.device)
-        grad = torch.empty(2 * n * max(npar, 1), dtype=torch.float64, device=bits.device)
+        a = torch.empty(n, dtype=torch.complex128, device=bits.device)
+        g = torch.empty((n, npar), dtype=torch.complex128, device=bits.device)
         th = None
         if thetas is not None:
-            th = torch.as_tensor(thetas, dtype=torch.float64).to(bits.device).contiguous()
+            th = thetas
+            if not (isinstance(th, torch.Tensor) and th.dtype == torch.float64 and th.device == bits.device
+                    and th.is_contiguous()):
+                th = torch.as_tensor(thetas, dtype=torch.float64).to(bits.device).contiguous()
             if th.numel() != npar:
                 raise QvxError(QVX_EINVAL, f"expected {npar} angles, got {th.numel()}")
-        _check(lib().qvx_amplitude_grad(self._h, ctypes.c_void_p(bits.data_ptr()), n,
-                                        None if th is None else ctypes.c_void_p(th.data_ptr()),
-                                        0 if th is None else npar, ctypes.c_void_p(amps.data_ptr()),
-                                        ctypes.c_void_p(grad.data_ptr()), ctypes.c_void_p(ws.data_ptr()),
-                                        ws.numel(), _stream_ptr(stream)))
-        a = torch.view_as_complex(amps.view(n, 2))
-        g = torch.view_as_complex(grad.view(n, max(npar, 1), 2))[:, :npar]
+        _check(lib().qvx_amplitude_grad(self._h, bits.data_ptr(), n, None if th is None else th.data_ptr(),
+                                        0 if th is None else npar, a.data_ptr(), g.data_ptr(), ws.data_ptr(),
+                                        ws.numel(), sp))
         return a, g
 
     def graphed(self, bitstrings, workspace=None):
@@ -388,29 +454,30 @@ class Plan:
         n = h.numel() // self.words
         if out is None:
             out = torch.empty(2 * n * (1 << self.n_open), dtype=torch.float64)
-        dev = torch.device("cuda", torch.cuda.current_device())
-        ws = workspace if workspace is not None else self._ws_for(n, dev)
+        ws = workspace if workspace is not None else self._ws_for(n, torch.device("cuda", torch.cuda.current_device()))
         _check(lib().qvx_amplitude_host(self._h, ctypes.c_void_p(h.data_ptr()), n, ctypes.c_void_p(out.data_ptr()),
                                         ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream_ptr(stream)))
-        a = out[0::2].numpy() + 1j * out[1::2].numpy()
+        a = out.numpy().view("complex128").copy()
         return a.reshape(n, 1 << self.n_open) if self.n_open else a
 
     def slice_terms(self, bitstrings, slice_begin=0, slice_count=None, workspace=None, stream=None):
         """The slice terms beta_s (complex64, [batch, slice_count]) of Section 3.B.2."""
         import torch
-        bits = self._bits(bitstrings)
-        self._check_bits(bits)
-        n = bits.numel() // self.words
-        if slice_count is None:
-            slice_count = self.n_slice_terms - slice_begin
-        ws = workspace if workspace is not None else self._ws_for(n, bits.device)
-        m = 1 << self.n_open
-        out = torch.empty(2 * n * m * slice_count, dtype=torch.float32, device=bits.device)
-        _check(lib().qvx_slice_terms(self._h, ctypes.c_void_p(bits.data_ptr()), n, slice_begin, slice_count,
-                                     ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(ws.data_ptr()),
-                                     ws.numel(), _stream_ptr(stream)))
-        t = torch.view_as_complex(out.view(n * m, slice_count, 2))
-        return t.view(n, m, slice_count) if self.n_open else t.view(n, slice_count)
+        sp = _stream_ptr(stream)
+        bits, ticket = self._checked_bits(bitstrings, sp, False)
+        try:
+            n = bits.numel() // self.words
+            if slice_count is None:
+                slice_count = self.n_slice_terms - slice_begin
+            ws = workspace if workspace is not None else self._ws_for(n, bits.device)
+            m = 1 << self.n_open
+            t = torch.empty((n * m, slice_count), dtype=torch.complex64, device=bits.device)
+            _check(lib().qvx_slice_terms(self._h, bits.data_ptr(), n, slice_begin, slice_count, t.data_ptr(),
+                                         ws.data_ptr(), ws.numel(), sp))
+        finally:
+            if ticket >= 0:
+                _check(lib().qvx_bits_result(ticket))
+        return t.view(n, m, slice_count) if self.n_open else t
 
     def amplitude_profiled(self, bits, workspace, out, stream=None, slice_begin=0, slice_count=None):
         """plan.amplitude (device int64 bitstring words, caller's workspace and float64

@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 
@@ -754,6 +755,102 @@ qvx_status qvx_amplitude_grad(qvx_plan *plan, const uint64_t *bitstrings_dev, in
                                   grad_dev, g.status, st)) != cudaSuccess)
         return cuda_fail(e, "gradient sum launch");
     return QVX_OK;
+}
+
+}  // extern "C"
+
+namespace {
+// One bitstring check in flight: a page-locked flag that the kernel sets, and the event after it.
+struct BitsTicket {
+    unsigned *flag = nullptr;
+    cudaEvent_t done = nullptr;
+    int device = -1;
+    bool busy = false;
+};
+constexpr size_t kKeptTickets = 64;
+std::mutex g_ticket_mutex;
+std::vector<BitsTicket> g_tickets;
+
+void free_ticket(BitsTicket &t) {
+    if (t.done) cudaEventDestroy(t.done);
+    if (t.flag) cudaFreeHost(t.flag);
+    t = BitsTicket{};
+}
+
+// A free ticket of the device (a new one if there is none): its index, or -1 with *e set.
+int64_t take_ticket(int device, BitsTicket *out, cudaError_t *e) {
+    std::lock_guard<std::mutex> lock(g_ticket_mutex);
+    size_t at = g_tickets.size();
+    for (size_t i = 0; i < g_tickets.size(); i++) {
+        if (g_tickets[i].busy) continue;
+        if (g_tickets[i].device == device) { at = i; break; }
+        if (g_tickets[i].device < 0) at = i;
+    }
+    if (at == g_tickets.size()) g_tickets.push_back(BitsTicket{});
+    BitsTicket &t = g_tickets[at];
+    if (t.device != device) {
+        t = BitsTicket{};
+        if ((*e = cudaHostAlloc(reinterpret_cast<void **>(&t.flag), 64, cudaHostAllocPortable)) != cudaSuccess ||
+            (*e = cudaEventCreateWithFlags(&t.done, cudaEventDisableTiming)) != cudaSuccess) {
+            free_ticket(t);
+            return -1;
+        }
+        t.device = device;
+    }
+    t.busy = true;
+    *out = t;
+    return (int64_t)at;
+}
+
+void give_ticket(int64_t i) {
+    std::lock_guard<std::mutex> lock(g_ticket_mutex);
+    g_tickets[(size_t)i].busy = false;
+    if ((size_t)i >= kKeptTickets) free_ticket(g_tickets[(size_t)i]);   // a peak of concurrent calls is not kept
+}
+}  // namespace
+
+extern "C" {
+
+qvx_status qvx_bits_check(const qvx_plan *plan, const uint64_t *bitstrings_dev, int64_t batch, void *stream, int64_t *ticket) {
+    if (!plan || !ticket || batch < 0 || (batch > 0 && !bitstrings_dev)) return fail(QVX_EINVAL, "bad argument");
+    *ticket = -1;
+    const int n = plan->p.model.n_qubits;
+    if (batch == 0 || n % 64 == 0) return QVX_OK;   // nothing to find
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(st, &cap)) != cudaSuccess) return cuda_fail(e, "capture query");
+    if (cap != cudaStreamCaptureStatusNone) return fail(QVX_ECUDA, "bitstrings cannot be checked during stream capture");
+    int dev = -1;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+    BitsTicket t;
+    const int64_t i = take_ticket(dev, &t, &e);
+    if (i < 0) return cuda_fail(e, "bitstring check");
+    *t.flag = 0u;
+    const uint64_t lo = n >= 64 ? ~0ull : (1ull << n) - 1ull, hi = n > 64 ? (1ull << (n - 64)) - 1ull : 0ull;
+    if ((e = qvx::launch_check_bits(bitstrings_dev, batch, words_of(plan->p), lo, hi, t.flag, st)) != cudaSuccess ||
+        (e = cudaEventRecord(t.done, st)) != cudaSuccess) {
+        cudaStreamSynchronize(st);   // the kernel may be running: the flag is its until then
+        give_ticket(i);
+        return cuda_fail(e, "bitstring check launch");
+    }
+    *ticket = i;
+    return QVX_OK;
+}
+
+qvx_status qvx_bits_result(int64_t ticket) {
+    if (ticket < 0) return QVX_OK;
+    BitsTicket t;
+    {
+        std::lock_guard<std::mutex> lock(g_ticket_mutex);
+        if ((size_t)ticket >= g_tickets.size() || !g_tickets[(size_t)ticket].busy) return fail(QVX_EINVAL, "unknown ticket");
+        t = g_tickets[(size_t)ticket];
+    }
+    const cudaError_t e = cudaEventSynchronize(t.done);
+    const bool bad = e == cudaSuccess && *reinterpret_cast<volatile unsigned *>(t.flag) != 0u;
+    give_ticket(ticket);
+    if (e != cudaSuccess) return cuda_fail(e, "bitstring check");
+    return bad ? fail(QVX_EINVAL, "bitstring has bits at or above n_qubits") : QVX_OK;
 }
 
 qvx_status qvx_selftest_wait_timeout(const qvx_plan *plan, void *ws, size_t ws_bytes, uint32_t polls, void *stream) {

@@ -1257,6 +1257,14 @@ __global__ void grad_sum_kernel(const unsigned char *img, const ExactPair *gpart
     }
 }
 
+__global__ void check_bits_kernel(const uint64_t *bitstrings, int64_t n, uint32_t words, uint64_t valid_lo,
+                                  uint64_t valid_hi, unsigned *flag) {
+    bool bad = false;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        bad |= (bitstrings[i] & ~(words > 1 && (i & 1) ? valid_hi : valid_lo)) != 0ull;
+    if (bad) *reinterpret_cast<volatile unsigned *>(flag) = 1u;
+}
+
 // Self-test of the bounded waits: a grid barrier for two CTAs run by one, and an mbarrier
 // whose phase never completes. Each wait must give up after `polls` polls; the kernel
 // records which did in out[0] (barrier) and out[1] (mbarrier) and sets the status word.
@@ -1295,6 +1303,14 @@ cudaError_t counted(cudaError_t e) {
 uint64_t launches_issued() { return t_launches; }
 
 cudaError_t launch_counted(cudaError_t e) { return counted(e); }
+
+cudaError_t launch_check_bits(const uint64_t *bitstrings, int64_t batch, uint32_t words, uint64_t valid_lo,
+                              uint64_t valid_hi, unsigned *flag, cudaStream_t s) {
+    const int64_t n = batch * words;
+    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 64));
+    check_bits_kernel<<<blocks, 256, 0, s>>>(bitstrings, n, words, valid_lo, valid_hi, flag);
+    return counted(cudaGetLastError());
+}
 
 cudaError_t launch_wait_selftest(unsigned *words, unsigned *status, uint32_t polls, unsigned *out, cudaStream_t s) {
     wait_selftest_kernel<<<1, 32, 0, s>>>(words, status, polls, out);

@@ -143,6 +143,10 @@ cudaError_t launch_gemm_step(const LaunchArgs &a, const GemmStep &g, const GemmL
 // scale.max_a and max_b as for launch_gemm_step, max_c of the second step's output.
 cudaError_t launch_reduce_step(const LaunchArgs &a, const ReduceStep &r, const GemmScale &scale, uint32_t *max_c,
                                int64_t item0, int64_t n_items, float2 *arenas, cudaStream_t s);
+// Sets *flag (device-accessible) to 1 if a bitstring has bits outside valid_lo (word 0) or
+// valid_hi (word 1).
+cudaError_t launch_check_bits(const uint64_t *bitstrings, int64_t batch, uint32_t words, uint64_t valid_lo,
+                              uint64_t valid_hi, unsigned *flag, cudaStream_t s);
 // Self-test of the bounded waits (grid barrier and mbarrier that can never complete).
 cudaError_t launch_wait_selftest(unsigned *words, unsigned *status, uint32_t polls, unsigned *out, cudaStream_t s);
 
