@@ -679,50 +679,196 @@ __device__ __forceinline__ float2 persistent_entry(const DevStep &st, uint32_t c
     return acc;
 }
 
+// The bitstring and outer slice number of a work item (32-bit division where both sides allow
+// it: the 64-bit one is a called routine).
+__device__ __forceinline__ Bits item_bits(const LaunchArgs &a, int64_t item, uint64_t *o) {
+    int64_t b, r;
+    if (((uint64_t)item | (uint64_t)a.o_count) < (1ull << 32)) {
+        b = (int64_t)((uint32_t)item / (uint32_t)a.o_count);
+        r = (int64_t)((uint32_t)item % (uint32_t)a.o_count);
+    } else {
+        b = item / a.o_count;
+        r = item % a.o_count;
+    }
+    *o = (uint64_t)(a.o_begin + r);
+    return load_bits(a.bitstrings, b, a.words);
+}
+
+// First stored entry of a leaf for one work item, its fixed modes one by one (a step's leaf is
+// the same for the whole block, so the loop is uniform; the predicated form of leaf_base costs
+// its twelve rounds for every leaf).
+__device__ __forceinline__ uint32_t leaf_base_loop(const DevLeaf &L, const Bits &x, uint64_t o) {
+    uint32_t off = L.data_off;
+    const uint32_t n = L.n_fixed;
+    for (uint32_t f = 0; f < n; f++) {
+        const uint32_t src = L.fixed_src[f];
+        const uint64_t v = src < 64u ? x.w0 : (src < 128u ? x.w1 : o);
+        off += (uint32_t)((v >> (src & 63u)) & 1ull) << L.fixed_pos[f];
+    }
+    return off;
+}
+
+// 2^RM x 2^RN output entries of a register-tiled step (RegTileStep) from the operands' bases at
+// the tile's first entry: every entry is the same sequence of multiply-adds as step_entry's.
+template <int RM, int RN>
+__device__ __forceinline__ void tile_entries(const RegTileStep &rs, const float2 *A, const float2 *B, float2 *C) {
+    constexpr int TM = 1 << RM, TN = 1 << RN;
+    const uint32_t nab = rs.nk_ab, na = rs.nk_a;
+    const uint32_t nk = nab + na + rs.nk_b;
+    const uint32_t mask_ka = (1u << (nab + na)) - 1u, mask_ab = (1u << nab) - 1u;
+    uint32_t am[TM], bn[TN];
+#pragma unroll
+    for (int i = 0; i < TM; i++) am[i] = rs.a_m[i];
+#pragma unroll
+    for (int j = 0; j < TN; j++) bn[j] = rs.b_n[j];
+    float2 acc[TM][TN];
+#pragma unroll
+    for (int i = 0; i < TM; i++)
+#pragma unroll
+        for (int j = 0; j < TN; j++) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (uint32_t k = 0; k < (1u << nk); k++) {
+        const float2 *Ak = A + ((k & mask_ka) << rs.a_cb);
+        const float2 *Bk = B + (((k & mask_ab) | ((k >> (nab + na)) << nab)) << rs.b_cb);
+        float2 av[TM], bv[TN];
+#pragma unroll
+        for (int i = 0; i < TM; i++) av[i] = Ak[am[i]];
+#pragma unroll
+        for (int j = 0; j < TN; j++) bv[j] = Bk[bn[j]];
+#pragma unroll
+        for (int i = 0; i < TM; i++)
+#pragma unroll
+            for (int j = 0; j < TN; j++) cmac(acc[i][j], av[i], bv[j]);
+    }
+#pragma unroll
+    for (int i = 0; i < TM; i++)
+#pragma unroll
+        for (int j = 0; j < TN; j++) C[rs.c_m[i] + rs.c_n[j]] = acc[i][j];
+}
+
 // All contractions of a chunk of work items in one cooperative launch: phase by phase;
-// within a phase the CTAs sweep each step's (item, entry) space with a grid-stride loop
-// (the step's descriptor staged once in shared memory), a grid barrier separates phases,
-// then each item's final tensor is summed into its partial.
-__global__ void __launch_bounds__(256) persistent_program_kernel(LaunchArgs a, int64_t item_begin, int64_t n_items,
-                                                                 float2 *arenas, unsigned *bar_count, unsigned *bar_gen) {
-    __shared__ __align__(16) DevStep sd;
+// within a phase the CTAs sweep each step's (item, tile) space with a grid-stride loop, a grid
+// barrier separates phases, then each item's final tensor is summed into its partial.
+// A step's descriptor is staged in shared memory, and for register-tiled steps the bit-run
+// maps of the tile index are tabulated there for its low and next eight bits (output, A and B
+// offset), so a tile costs two table reads instead of some fifteen run moves. What bounds the
+// kernel is instruction issue. 16 amplitudes of a 49-qubit circuit (8 sliced variables, 4096
+// work items): 8.84 ms with one thread per entry, 2.57 ms; three CTAs per SM (80 registers) ran
+// 4 % faster than four (64, spilled).
+constexpr uint32_t kStepBits = 1024;
+struct PersistentSmem {
+    RegTileStep rt;
+    DevStep sd;
+    uint32_t lc[256], la[256], lb[256];   // tile index bits 0-7
+    uint32_t hc[256], ha[256], hb[256];   // bits 8-15
+    uint8_t bits[kStepBits];              // of the first steps: work unit bits, 128 added when tiled
+};
+__global__ void __launch_bounds__(256, 3) persistent_program_kernel(LaunchArgs a, int64_t item_begin, int64_t n_items,
+                                                                    float2 *arenas, unsigned *bar_count, unsigned *bar_gen) {
+    __shared__ __align__(16) PersistentSmem sm;
     const unsigned char *img = a.image;
     const DevProgram *P = reinterpret_cast<const DevProgram *>(img);
     const DevStep *steps = reinterpret_cast<const DevStep *>(img + P->steps_off);
+    const RegTileStep *tiles = P->regtile_off ? reinterpret_cast<const RegTileStep *>(img + P->regtile_off) : nullptr;
     const DevLeaf *leaves = reinterpret_cast<const DevLeaf *>(img + P->leaves_off);
     const float2 *ldata = reinterpret_cast<const float2 *>(img + P->leaf_data_off);
     const uint32_t *phase_first = reinterpret_cast<const uint32_t *>(img + P->level_phases_off);
     const uint32_t n_phases = P->n_level_phases;
     const uint64_t arena_elems = a.arena_elems;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    const DevStep &sd = sm.sd;
+    const RegTileStep &rt = sm.rt;
+    // unit bits of step s, 128 added when it is register-tiled
+    auto unit_bits = [&](uint32_t s) -> uint32_t {
+        return tiles && tiles[s].rm + tiles[s].rn > 0 ? 128u + tiles[s].nt : steps[s].rc;
+    };
+    for (uint32_t s = threadIdx.x; s < min(a.n_steps, kStepBits); s += blockDim.x) sm.bits[s] = (uint8_t)unit_bits(s);
+    __syncthreads();
     for (uint32_t ph = 0; ph < n_phases; ph++) {
         const uint32_t s0 = phase_first[ph], s1 = phase_first[ph + 1];
         for (uint32_t s = s0; s < s1; s++) {
-            __syncthreads();   // the previous step's readers are done with sd
-            if (threadIdx.x < sizeof(DevStep) / 8)
-                reinterpret_cast<uint64_t *>(&sd)[threadIdx.x] = reinterpret_cast<const uint64_t *>(steps + s)[threadIdx.x];
+            // the step's work units (tiles, or single entries) start at another CTA for every step
+            // of the phase, so that small steps land on different CTAs; a CTA without a unit
+            // skips the step
+            const uint32_t ub = s < kStepBits ? sm.bits[s] : unit_bits(s);
+            const bool tiled = ub >= 128u;
+            const uint32_t bits = ub & 127u;
+            const uint64_t total = (uint64_t)n_items << bits;
+            const uint64_t first_block = ((uint64_t)blockIdx.x + (uint64_t)(s - s0) * 37u) % gridDim.x;
+            if (first_block * blockDim.x >= total) continue;
+            const uint64_t first = first_block * blockDim.x + threadIdx.x;
+            __syncthreads();   // the previous step's readers are done with the shared descriptors
+            if (tiled) {
+                if (threadIdx.x < sizeof(RegTileStep) / 8)
+                    reinterpret_cast<uint64_t *>(&sm.rt)[threadIdx.x] = reinterpret_cast<const uint64_t *>(tiles + s)[threadIdx.x];
+            } else if (threadIdx.x < sizeof(DevStep) / 8) {
+                reinterpret_cast<uint64_t *>(&sm.sd)[threadIdx.x] = reinterpret_cast<const uint64_t *>(steps + s)[threadIdx.x];
+            }
             __syncthreads();
+            if (tiled) {
+                const uint32_t mask = bits >= 32u ? ~0u : (1u << bits) - 1u;
+                const uint32_t lo = pext_runs(threadIdx.x & mask, rt.free_runs, rt.n_free);
+                sm.lc[threadIdx.x] = lo;
+                sm.la[threadIdx.x] = pext_runs(lo, rt.runs_a, rt.na_runs);
+                sm.lb[threadIdx.x] = pext_runs(lo, rt.runs_b, rt.nb_runs);
+                if (bits > 8u) {
+                    const uint32_t hi = pext_runs((threadIdx.x << 8) & mask, rt.free_runs, rt.n_free);
+                    sm.hc[threadIdx.x] = hi;
+                    sm.ha[threadIdx.x] = pext_runs(hi, rt.runs_a, rt.na_runs);
+                    sm.hb[threadIdx.x] = pext_runs(hi, rt.runs_b, rt.nb_runs);
+                } else if (threadIdx.x == 0) {
+                    sm.hc[0] = sm.ha[0] = sm.hb[0] = 0u;
+                }
+                __syncthreads();
+                const bool a_leaf = rt.flags & kStepALeaf, b_leaf = rt.flags & kStepBLeaf;
+                for (uint64_t w = first; w < total; w += stride) {
+                    const int64_t il = (int64_t)(w >> bits);
+                    const uint32_t t = (uint32_t)w & mask;
+                    float2 *arena = arenas + (uint64_t)il * arena_elems;
+                    const float2 *A = arena + rt.a_off, *B = arena + rt.b_off;
+                    if (a_leaf || b_leaf) {
+                        uint64_t o;
+                        const Bits x = item_bits(a, item_begin + il, &o);
+                        if (a_leaf) A = ldata + leaf_base_loop(leaves[rt.a_off], x, o);
+                        if (b_leaf) B = ldata + leaf_base_loop(leaves[rt.b_off], x, o);
+                    }
+                    const uint32_t lo_t = t & 255u, hi_t = (t >> 8) & 255u;
+                    uint32_t c0 = sm.lc[lo_t] | sm.hc[hi_t];
+                    uint32_t ia = sm.la[lo_t] | sm.ha[hi_t], ib = sm.lb[lo_t] | sm.hb[hi_t];
+                    if (bits > 16u) {   // the bits above the tables
+                        const uint32_t top = pext_runs(t & ~0xffffu, rt.free_runs, rt.n_free);
+                        c0 |= top;
+                        ia |= pext_runs(top, rt.runs_a, rt.na_runs);
+                        ib |= pext_runs(top, rt.runs_b, rt.nb_runs);
+                    }
+                    float2 *C = arena + rt.c_off + c0;
+                    switch (rt.rm * 3 + rt.rn) {
+                        case 1: tile_entries<0, 1>(rt, A + ia, B + ib, C); break;
+                        case 2: tile_entries<0, 2>(rt, A + ia, B + ib, C); break;
+                        case 3: tile_entries<1, 0>(rt, A + ia, B + ib, C); break;
+                        case 4: tile_entries<1, 1>(rt, A + ia, B + ib, C); break;
+                        case 5: tile_entries<1, 2>(rt, A + ia, B + ib, C); break;
+                        case 6: tile_entries<2, 0>(rt, A + ia, B + ib, C); break;
+                        case 7: tile_entries<2, 1>(rt, A + ia, B + ib, C); break;
+                        default: tile_entries<2, 2>(rt, A + ia, B + ib, C); break;
+                    }
+                }
+                continue;
+            }
             const uint32_t rc = sd.rc, flags = sd.flags;
             const bool unary = flags & kStepUnary;
             const bool a_leaf = flags & kStepALeaf, b_leaf = flags & kStepBLeaf;
-            const uint64_t total = (uint64_t)n_items << rc;
-            // rotate the start so that small steps of one phase land on different CTAs
-            const uint64_t first = (((uint64_t)blockIdx.x + (uint64_t)(s - s0) * 37u) % gridDim.x) * blockDim.x + threadIdx.x;
             for (uint64_t w = first; w < total; w += stride) {
                 const int64_t il = (int64_t)(w >> rc);
                 const uint32_t c = (uint32_t)(w & ((1ull << rc) - 1));
-                const int64_t item = item_begin + il;
-                const int64_t b = item / a.o_count;
-                const uint64_t o = (uint64_t)(a.o_begin + item % a.o_count);
                 float2 *arena = arenas + (uint64_t)il * arena_elems;
-                const float2 *A, *B;
+                const float2 *A = arena + sd.a_off, *B = unary ? A : arena + sd.b_off;
                 if (a_leaf || (!unary && b_leaf)) {
-                    const Bits x = load_bits(a.bitstrings, b, a.words);
-                    A = a_leaf ? ldata + leaf_base(leaves[sd.a_off], x, o) : arena + sd.a_off;
-                    B = unary ? A : (b_leaf ? ldata + leaf_base(leaves[sd.b_off], x, o) : arena + sd.b_off);
-                } else {
-                    A = arena + sd.a_off;
-                    B = unary ? A : arena + sd.b_off;
+                    uint64_t o;
+                    const Bits x = item_bits(a, item_begin + il, &o);
+                    if (a_leaf) A = ldata + leaf_base_loop(leaves[sd.a_off], x, o);
+                    if (!unary && b_leaf) B = ldata + leaf_base_loop(leaves[sd.b_off], x, o);
+                    if (unary) B = A;
                 }
                 arena[sd.c_off + c] = persistent_entry(sd, c, A, !a_leaf, B, !b_leaf, unary);
             }

@@ -1537,7 +1537,8 @@ bool serialize(Plan &p, std::string *err) {
             const std::vector<int> &LA = p.tensors[st.a].modes, &LB = p.tensors[st.b].modes, &LC = p.tensors[st.c].modes;
             double fl = 0, by = 0;
             step_work(p, st, &fl, &by);
-            const size_t max_bits = fl >= 16.0 * by && LC.size() >= 18 ? 3 : 2;
+            // (the persistent kernel has the tiles of up to 4 x 4)
+            const size_t max_bits = p.engine == QVX_ENGINE_STEPWISE && fl >= 16.0 * by && LC.size() >= 18 ? 3 : 2;
             std::vector<int> tm, tn;   // tile bits: positions in C
             for (int j = 5; j < (int)LC.size(); j++) {
                 const bool ia = find_pos(LA, LC[j]) >= 0, ib = find_pos(LB, LC[j]) >= 0;
