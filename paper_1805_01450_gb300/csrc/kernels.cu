@@ -890,46 +890,90 @@ __global__ void __launch_bounds__(256, 3) persistent_program_kernel(LaunchArgs a
 // ------------------------------------------------------------------ register-tiled contraction
 // One thread per 2^RM x 2^RN output entries of a two-operand step (RegTileStep): per summed
 // index it loads 2^RM entries of A and 2^RN of B and forms all their products, so each
-// loaded entry serves several outputs from registers. Tiles of up to 4 x 4 run 256 threads
-// per CTA with the summed-index loop unrolled four deep (more loads in flight per thread);
-// the 8-wide tiles of compute-heavy steps hold 2 x 64 accumulator registers and run 128
-// threads per CTA, two CTAs per SM, with the loop unrolled twice.
+// loaded entry serves several outputs from registers. 256 threads per CTA; the 8 x 4 tiles
+// hold 2 x 32 accumulator registers and run two CTAs per SM, the 8 x 8 tiles 2 x 64 and two CTAs
+// of 128 threads.
+//
+// Steps of few summed entries are bound by DRAM (5.1 to 6.8 of 6.9 TB/s); the compute-heavy ones
+// by load latency and instructions, at 45 % of the issue slots. What was taken from that, on the
+// 1,024 amplitudes of a 7 x 7 grid at depth 30 (9.93 ms at first, 8.46 now):
+//  - the item, its leaves and the tile index's high bits are found once per CTA, and a CTA walks
+//    up to 8 blocks of tiles: 9.2 ms (with one block per CTA 10.4);
+//  - 4 x 4 tiles of a small and a large operand address these by a block-uniform base and a
+//    32-bit offset per thread, which leaves registers for loads: a 32-entry sum goes from 1.80
+//    to 1.56 ms. Smaller tiles lose 10 % by it and keep their own pointers;
+//  - in that form, with 64 registers, the compiler loads a tile's B entries together and its A
+//    entries one by one, so B has to be the operand that comes from DRAM: they are swapped where
+//    A is the larger (a 16-entry sum over a 2^25-entry A: 1.85 to 0.94 ms). At 72 and 80
+//    registers it does so for none (2.28 ms for 1.56);
+//  - 8 x 4 tiles from 4 flops per byte up (RegTileStep's rule): 8.73 to 8.58 ms.
+constexpr uint32_t kMaxTileBlocks = 8;          // blocks of tiles per CTA (16: 3 % slower)
+constexpr uint64_t kMinTileCtas = 2048;         // while this many CTAs remain (3.4 waves of 4 per SM)
 template <int RM, int RN>
 struct RegTileShape {
     static constexpr bool kWide = RM + RN >= 5;
-    static constexpr int kThreads = kWide ? 128 : 256;
+    static constexpr int kThreads = RM + RN == 6 ? 128 : 256;
+    static constexpr int kThreadBits = RM + RN == 6 ? 7 : 8;
     static constexpr int kMinBlocks = kWide ? 2 : 4;
 };
 
-template <int RM, int RN, bool kMax>   // kMax: the output's largest entries are wanted (max_c)
+// What a thread adds to an item's tensors: the output entry of its tile and both operands'
+// entries for it.
+struct TileOffsets {
+    uint32_t c, a, b;
+};
+__device__ __forceinline__ TileOffsets tile_offsets(const RegTileStep &rs, uint32_t t) {
+    TileOffsets o;
+    o.c = pext_runs(t, rs.free_runs, rs.n_free);
+    o.a = pext_runs(o.c, rs.runs_a, rs.na_runs);
+    o.b = pext_runs(o.c, rs.runs_b, rs.nb_runs);
+    return o;
+}
+
+__device__ __forceinline__ float2 at_bytes(const float2 *base, uint32_t bytes) {
+    return *reinterpret_cast<const float2 *>(reinterpret_cast<const char *>(base) + bytes);
+}
+// How a CTA goes over a step's tiles (tile_form picks one).
+enum TileForm {
+    kTilesFlat,      // one tile per thread, any item and tile per thread
+    kTilesBlocks,    // several blocks of tiles of one item
+    kTilesBase,      // the same; block-uniform bases and a 32-bit offset per thread
+    kTilesSwapped    // the same; A and B are the step's second and first operand. A product's
+};                   // two terms are added in the step's own order, so the bits are the same
+// kMax: the output's largest entries are wanted (max_c).
+template <int RM, int RN, bool kMax, TileForm kForm>
 __global__ void __launch_bounds__(RegTileShape<RM, RN>::kThreads, RegTileShape<RM, RN>::kMinBlocks)
     regtile_step_kernel(LaunchArgs a, RegTileStep rs, int64_t item_begin, int64_t n_items, float2 *arenas,
-                        uint32_t *max_c) {
+                        uint32_t *max_c, uint32_t per_cta) {
     constexpr int TM = 1 << RM, TN = 1 << RN;
-    const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= ((uint64_t)n_items << rs.nt)) return;
-    const int64_t il = (int64_t)(g >> rs.nt);
-    const uint32_t t = (uint32_t)(g & ((1ull << rs.nt) - 1ull));
+    constexpr int kThreadBits = RegTileShape<RM, RN>::kThreadBits;
+    constexpr bool kWhole = kForm != kTilesFlat, kUniform = kForm == kTilesBase || kForm == kTilesSwapped;
+    int64_t il;
+    uint32_t blk = 0;              // kWhole: first block of tiles of this CTA
+    TileOffsets own;
+    if constexpr (kWhole) {
+        const uint64_t first = (uint64_t)blockIdx.x * per_cta;   // per_cta divides an item's blocks
+        il = (int64_t)(first >> (rs.nt - kThreadBits));
+        blk = (uint32_t)(first & ((1ull << (rs.nt - kThreadBits)) - 1ull));
+        own = tile_offsets(rs, threadIdx.x);
+    } else {
+        const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+        if (g >= ((uint64_t)n_items << rs.nt)) return;
+        il = (int64_t)(g >> rs.nt);
+        own = tile_offsets(rs, (uint32_t)(g & ((1ull << rs.nt) - 1ull)));
+    }
     float2 *arena = arenas + (uint64_t)il * a.arena_elems;
-    const float2 *A, *B;
-    {
+    const float2 *A0 = arena + rs.a_off, *B0 = arena + rs.b_off;
+    if (rs.flags & (kStepALeaf | kStepBLeaf)) {
         const unsigned char *img = a.image;
         const DevProgram *P = reinterpret_cast<const DevProgram *>(img);
         const DevLeaf *leaves = reinterpret_cast<const DevLeaf *>(img + P->leaves_off);
         const float2 *ldata = reinterpret_cast<const float2 *>(img + P->leaf_data_off);
-        Bits x = {0ull, 0ull};
-        uint64_t o = 0;
-        if (rs.flags & (kStepALeaf | kStepBLeaf)) {
-            const int64_t item = item_begin + il;
-            x = load_bits(a.bitstrings, item / a.o_count, a.words);
-            o = (uint64_t)(a.o_begin + item % a.o_count);
-        }
-        A = (rs.flags & kStepALeaf) ? ldata + leaf_base(leaves[rs.a_off], x, o) : arena + rs.a_off;
-        B = (rs.flags & kStepBLeaf) ? ldata + leaf_base(leaves[rs.b_off], x, o) : arena + rs.b_off;
+        uint64_t o;
+        const Bits x = item_bits(a, item_begin + il, &o);
+        if (rs.flags & kStepALeaf) A0 = ldata + leaf_base(leaves[rs.a_off], x, o);
+        if (rs.flags & kStepBLeaf) B0 = ldata + leaf_base(leaves[rs.b_off], x, o);
     }
-    const uint32_t c0 = pext_runs(t, rs.free_runs, rs.n_free);
-    A += pext_runs(c0, rs.runs_a, rs.na_runs);
-    B += pext_runs(c0, rs.runs_b, rs.nb_runs);
     const uint32_t nab = rs.nk_ab, na = rs.nk_a;
     const uint32_t nk = nab + na + rs.nk_b;
     const uint32_t mask_ka = (1u << (nab + na)) - 1u, mask_ab = (1u << nab) - 1u;
@@ -938,41 +982,58 @@ __global__ void __launch_bounds__(RegTileShape<RM, RN>::kThreads, RegTileShape<R
     for (int i = 0; i < TM; i++) am[i] = rs.a_m[i];
 #pragma unroll
     for (int j = 0; j < TN; j++) bn[j] = rs.b_n[j];
-    float2 acc[TM][TN];
+    uint32_t largest = 0;
+    for (uint32_t it = 0; it < (kWhole ? per_cta : 1u); it++) {
+        TileOffsets up{0u, 0u, 0u};
+        if constexpr (kWhole) up = tile_offsets(rs, (blk + it) << kThreadBits);
+        if constexpr (!kUniform) {
+            up.c += own.c;
+            up.a += own.a;
+            up.b += own.b;
+        }
+        const float2 *A = A0 + up.a, *B = B0 + up.b;
+        const uint32_t oa = kUniform ? own.a * 8u : 0u, ob = kUniform ? own.b * 8u : 0u, oc = kUniform ? own.c * 8u : 0u;
+        float2 acc[TM][TN];
 #pragma unroll
-    for (int i = 0; i < TM; i++)
+        for (int i = 0; i < TM; i++)
 #pragma unroll
-        for (int j = 0; j < TN; j++) acc[i][j] = make_float2(0.f, 0.f);
-    constexpr int kUnroll = RegTileShape<RM, RN>::kWide ? 2 : 4;
+            for (int j = 0; j < TN; j++) acc[i][j] = make_float2(0.f, 0.f);
+        constexpr int kUnroll = RM + RN >= 5 || kUniform ? 2 : 4;
+        auto products = [&](const float2 *Ak, const float2 *Bk) {
+            float2 av[TM], bv[TN];
+#pragma unroll
+            for (int i = 0; i < TM; i++) av[i] = at_bytes(Ak + am[i], oa);
+#pragma unroll
+            for (int j = 0; j < TN; j++) bv[j] = at_bytes(Bk + bn[j], ob);
+#pragma unroll
+            for (int i = 0; i < TM; i++)
+#pragma unroll
+                for (int j = 0; j < TN; j++)
+                    if constexpr (kForm == kTilesSwapped) cmac(acc[i][j], bv[j], av[i]);
+                    else cmac(acc[i][j], av[i], bv[j]);
+        };
+        if (kWhole && nk == nab) {   // every summed mode in both operands
 #pragma unroll kUnroll
-    for (uint32_t k = 0; k < (1u << nk); k++) {
-        const uint32_t ka = k & mask_ka;
-        const uint32_t kb = (k & mask_ab) | ((k >> (nab + na)) << nab);
-        const float2 *Ak = A + (ka << rs.a_cb), *Bk = B + (kb << rs.b_cb);
-        float2 av[TM], bv[TN];
-#pragma unroll
-        for (int i = 0; i < TM; i++) av[i] = Ak[am[i]];
-#pragma unroll
-        for (int j = 0; j < TN; j++) bv[j] = Bk[bn[j]];
+            for (uint32_t k = 0; k < (1u << nk); k++) products(A + (k << rs.a_cb), B + (k << rs.b_cb));
+        } else {
+            constexpr int kUnrollK = kWhole ? 1 : kUnroll;
+#pragma unroll kUnrollK
+            for (uint32_t k = 0; k < (1u << nk); k++)
+                products(A + ((k & mask_ka) << rs.a_cb), B + (((k & mask_ab) | ((k >> (nab + na)) << nab)) << rs.b_cb));
+        }
+        float2 *C = arena + rs.c_off + up.c;
 #pragma unroll
         for (int i = 0; i < TM; i++)
 #pragma unroll
-            for (int j = 0; j < TN; j++) cmac(acc[i][j], av[i], bv[j]);
+            for (int j = 0; j < TN; j++) {
+                *reinterpret_cast<float2 *>(reinterpret_cast<char *>(C + (rs.c_m[i] + rs.c_n[j])) + oc) = acc[i][j];
+                if (kMax) largest = abs_max(largest, acc[i][j]);
+            }
     }
-    float2 *C = arena + rs.c_off + c0;
-#pragma unroll
-    for (int i = 0; i < TM; i++)
-#pragma unroll
-        for (int j = 0; j < TN; j++) C[rs.c_m[i] + rs.c_n[j]] = acc[i][j];
     if constexpr (kMax) {
-        uint32_t largest = 0;
-#pragma unroll
-        for (int i = 0; i < TM; i++)
-#pragma unroll
-            for (int j = 0; j < TN; j++) largest = abs_max(largest, acc[i][j]);
         // one merge per CTA when all of it works on one item: with one per warp the merges into
         // one word outlasted the stores of the largest tensors
-        if ((1ull << rs.nt) >= blockDim.x) {
+        if (rs.nt >= kThreadBits) {
             __shared__ uint32_t warp_max[RegTileShape<RM, RN>::kThreads / 32];
             const uint32_t w = __reduce_max_sync(0xffffffffu, largest);
             if (threadIdx.x % 32 == 0) warp_max[threadIdx.x / 32] = w;
@@ -1619,13 +1680,69 @@ cudaError_t launch_splitk_step(const LaunchArgs &a, uint32_t step, int64_t item_
     return counted(cudaGetLastError());
 }
 
+// Form of a launch over `blocks` blocks of tiles; *per_cta blocks of one item go to a CTA. With
+// too few blocks for two per CTA and up to four summed entries the flat form is the faster one by
+// up to 15 % (242 items of a 6 x 7 grid at depth 26: 36.6 us a step against 41.1): it has no second
+// index to work out; from eight summed entries on it is the slower one (128 of them: 141 us against
+// 110). The base forms pay where one operand is far smaller than the other (2^7 times: 1.21 x
+// faster) and lose where both come from L2 (4 times: 1.26 x slower, the same size and 128 summed
+// entries: 2 x).
+template <int RM, int RN>
+static TileForm tile_form(const RegTileStep &rs, uint64_t blocks, uint32_t *per_cta) {
+    *per_cta = 1u;
+    // (the 32-bit byte offsets of a thread hold operands and results of up to 2^29 entries)
+    const int rank_a = rs.a_cb + rs.nk_ab + rs.nk_a, rank_b = rs.b_cb + rs.nk_ab + rs.nk_b;
+    if (rs.nt < RegTileShape<RM, RN>::kThreadBits || std::max({rank_a, rank_b, (int)rs.rc}) > 29) return kTilesFlat;
+    const uint32_t most = std::min(kMaxTileBlocks, 1u << (rs.nt - RegTileShape<RM, RN>::kThreadBits));
+    while (*per_cta < most && blocks / (2u * *per_cta) >= kMinTileCtas) *per_cta *= 2u;
+    if (*per_cta == 1u) return rs.nk_ab + rs.nk_a + rs.nk_b < 3 ? kTilesFlat : kTilesBlocks;
+    if (RM != 2 || RN != 2 || std::abs(rank_a - rank_b) < 6) return kTilesBlocks;
+    if (rank_a < rank_b) return kTilesBase;
+    return rs.nk_a + rs.nk_b == 0 ? kTilesSwapped : kTilesBlocks;   // (modes of one operand: A's before B's)
+}
+
+static RegTileStep swapped(const RegTileStep &rs) {
+    RegTileStep r = rs;
+    std::swap(r.a_off, r.b_off);
+    std::swap(r.a_cb, r.b_cb);
+    std::swap(r.na_runs, r.nb_runs);
+    std::swap(r.runs_a, r.runs_b);
+    std::swap(r.a_m, r.b_n);
+    std::swap(r.c_m, r.c_n);
+    r.flags = rs.flags & ~(kStepALeaf | kStepBLeaf);
+    if (rs.flags & kStepALeaf) r.flags |= kStepBLeaf;
+    if (rs.flags & kStepBLeaf) r.flags |= kStepALeaf;
+    return r;
+}
+
+template <int RM, int RN, TileForm kForm>
+static void launch_regtile_f(const LaunchArgs &a, const RegTileStep &rs, int64_t item_begin, int64_t n_items,
+                             float2 *arenas, uint32_t *max_c, uint64_t blocks, uint32_t per_cta, cudaStream_t s) {
+    constexpr int kThreads = RegTileShape<RM, RN>::kThreads;
+    const unsigned grid = (unsigned)(blocks / per_cta);   // per_cta divides an item's blocks
+    if (max_c)
+        regtile_step_kernel<RM, RN, true, kForm><<<grid, kThreads, 0, s>>>(a, rs, item_begin, n_items, arenas, max_c, per_cta);
+    else
+        regtile_step_kernel<RM, RN, false, kForm><<<grid, kThreads, 0, s>>>(a, rs, item_begin, n_items, arenas, nullptr, per_cta);
+}
+
 template <int RM, int RN>
 static void launch_regtile_t(const LaunchArgs &a, const RegTileStep &rs, int64_t item_begin, int64_t n_items,
                              float2 *arenas, uint32_t *max_c, cudaStream_t s) {
     constexpr int kThreads = RegTileShape<RM, RN>::kThreads;
     const uint64_t blocks = (((uint64_t)n_items << rs.nt) + kThreads - 1) / kThreads;
-    if (max_c) regtile_step_kernel<RM, RN, true><<<(unsigned)blocks, kThreads, 0, s>>>(a, rs, item_begin, n_items, arenas, max_c);
-    else regtile_step_kernel<RM, RN, false><<<(unsigned)blocks, kThreads, 0, s>>>(a, rs, item_begin, n_items, arenas, nullptr);
+    uint32_t per_cta;
+    const TileForm form = tile_form<RM, RN>(rs, blocks, &per_cta);
+    if constexpr (RM == 2 && RN == 2) {
+        if (form == kTilesBase)
+            return launch_regtile_f<RM, RN, kTilesBase>(a, rs, item_begin, n_items, arenas, max_c, blocks, per_cta, s);
+        if (form == kTilesSwapped)
+            return launch_regtile_f<RM, RN, kTilesSwapped>(a, swapped(rs), item_begin, n_items, arenas, max_c, blocks, per_cta, s);
+    }
+    if (form == kTilesFlat)
+        launch_regtile_f<RM, RN, kTilesFlat>(a, rs, item_begin, n_items, arenas, max_c, blocks, 1u, s);
+    else
+        launch_regtile_f<RM, RN, kTilesBlocks>(a, rs, item_begin, n_items, arenas, max_c, blocks, per_cta, s);
 }
 
 cudaError_t launch_regtile_step(const LaunchArgs &a, const RegTileStep &rs, int64_t item_begin, int64_t n_items,

@@ -1525,7 +1525,10 @@ bool serialize(Plan &p, std::string *err) {
     // item) take up to three of each: an 8 x 8 tile does 16 FMAs per loaded 8-byte entry where
     // a 4 x 4 tile does 8, which halves the L1 traffic that bounds the smaller tile there. On
     // output-bound steps the wide tile's 8 warps per SM issue too few stores (2.8 TB/s on a
-    // 7-flop/B step), so they keep the 4 x 4 tile
+    // 7-flop/B step), so they keep the 4 x 4 tile. Between, from 4 flops per byte up, the side
+    // against the larger operand takes three bits: an 8 x 4 tile reads that operand half as
+    // often from L2 and keeps 16 warps per SM (32-entry sums of 6 and 10 flops per byte: 1.54 to
+    // 1.48 ms and 0.81 to 0.71 ms; at 3 flops per byte 10 % slower)
     std::vector<RegTileStep> rts;
     if (p.engine != QVX_ENGINE_FUSED) {
         rts.assign(ds.size(), RegTileStep{});
@@ -1539,11 +1542,14 @@ bool serialize(Plan &p, std::string *err) {
             step_work(p, st, &fl, &by);
             // (the persistent kernel has the tiles of up to 4 x 4)
             const size_t max_bits = p.engine == QVX_ENGINE_STEPWISE && fl >= 16.0 * by && LC.size() >= 18 ? 3 : 2;
+            size_t max_a = max_bits, max_b = max_bits;
+            if (p.engine == QVX_ENGINE_STEPWISE && max_bits == 2 && fl >= 4.0 * by && LC.size() >= 16)
+                (LB.size() >= LA.size() ? max_a : max_b) = 3;
             std::vector<int> tm, tn;   // tile bits: positions in C
             for (int j = 5; j < (int)LC.size(); j++) {
                 const bool ia = find_pos(LA, LC[j]) >= 0, ib = find_pos(LB, LC[j]) >= 0;
-                if (ia && !ib && tm.size() < max_bits) tm.push_back(j);
-                if (ib && !ia && tn.size() < max_bits) tn.push_back(j);
+                if (ia && !ib && tm.size() < max_a) tm.push_back(j);
+                if (ib && !ia && tn.size() < max_b) tn.push_back(j);
             }
             if (tm.empty() && tn.empty()) continue;
             const DevStep &d = ds[s];
