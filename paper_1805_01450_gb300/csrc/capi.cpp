@@ -188,14 +188,16 @@ qvx_status run_items(qvx_plan *plan, const uint64_t *bits, int64_t batch, int64_
             if (s != QVX_OK) return s;
             if ((e = qvx::fused_prepare(shared + (size_t)max_ipc * group)) != cudaSuccess)
                 return cuda_fail(e, "fused kernel attributes");
-            for (int ipc = 1; ipc <= 8; ipc++)
+            for (int ipc = 1; ipc <= qvx::kFusedGroups; ipc++)
                 plan->ctas_per_sm[ipc] =
                     ipc <= max_ipc ? qvx::fused_blocks_per_sm(32 * wpi * ipc, shared + ipc * group, staged) : 0;
             plan->sms = caps.sms;
             plan->launch_device = dev;
         }
-        // spread the items over every SM first, then stack up to 8 warps per CTA
-        const int ipc = (int)std::max<int64_t>(1, std::min<int64_t>(max_ipc, (n_items + plan->sms - 1) / plan->sms));
+        // spread the items over every SM first, then stack them in a CTA, as many as share the
+        // SM's passes evenly
+        const int64_t per_sm = (n_items + plan->sms - 1) / plan->sms, passes = (per_sm + max_ipc - 1) / max_ipc;
+        const int ipc = (int)((per_sm + passes - 1) / passes);
         if (plan->ctas_per_sm[ipc] < 1) return fail(QVX_EUNSUPPORTED, "fused kernel: no CTA fits on an SM");
         const int64_t ctas_needed = (n_items + ipc - 1) / ipc;
         const int grid = (int)std::min<int64_t>(ctas_needed, (int64_t)plan->sms * plan->ctas_per_sm[ipc]);

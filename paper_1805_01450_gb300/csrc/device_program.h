@@ -116,6 +116,9 @@ struct RegTileStep {
     uint32_t a_m[8], b_n[8], c_m[8], c_n[8];
 };
 
+// Fused engine: most warps of a CTA, most work items it runs at a time.
+constexpr int kFusedWarps = 32, kFusedGroups = 32;
+
 // Tensor-core form of a dense two-operand step C[b, m, n] = sum_k A[b, m, k] B[b, k, n]
 // (stepwise engine): b are the output modes held by A and B, m those held by A alone, n those
 // held by B alone, k the summed modes (all held by both). A group's compact index (its modes

@@ -178,6 +178,11 @@ __device__ __forceinline__ FinishInfo finish_info(const DevProgram *P) {
     return f;
 }
 
+// Whether a bitstring has amplitude zero whatever the slices.
+__device__ __forceinline__ bool item_is_zero(const FinishInfo &P, const Bits &x) {
+    return bits_hit(x, P.zero_mask, P.zero_mask_hi);
+}
+
 __device__ __forceinline__ uint32_t compress_bits(uint32_t v, uint32_t mask, uint32_t n) {
     uint32_t r = 0, bit = 0;
     for (uint32_t j = 0; j < n; j++)
@@ -191,8 +196,7 @@ __device__ __forceinline__ uint32_t compress_bits(uint32_t v, uint32_t mask, uin
 // scalar) at terms[slot * (s_end - s_begin) + s - s_begin].
 template <bool CG>
 __device__ void finish_item_t(const FinishInfo &P, const LaunchArgs &a, const float2 *fin, int64_t b, uint64_t o,
-                              int lane, const Bits &x) {
-    const bool zero = bits_hit(x, P.zero_mask, P.zero_mask_hi);
+                              int lane, bool zero) {
     const uint32_t n_in = P.n_in, present = P.present;
     const uint32_t inner_bits = __popc(present);
     for (uint32_t j = 0; j < (1u << P.n_open); j++) {
@@ -224,12 +228,12 @@ __device__ void finish_item_t(const FinishInfo &P, const LaunchArgs &a, const fl
 
 __device__ __forceinline__ void finish_item(const FinishInfo &P, const LaunchArgs &a, const float2 *fin, int64_t b,
                                             uint64_t o, int lane, int) {
-    finish_item_t<false>(P, a, fin, b, o, lane, load_bits(a.bitstrings, b, a.words));
+    finish_item_t<false>(P, a, fin, b, o, lane, item_is_zero(P, load_bits(a.bitstrings, b, a.words)));
 }
 
 __device__ __forceinline__ void finish_item_cg(const FinishInfo &P, const LaunchArgs &a, const float2 *fin, int64_t b,
                                                uint64_t o, int lane) {
-    finish_item_t<true>(P, a, fin, b, o, lane, load_bits(a.bitstrings, b, a.words));
+    finish_item_t<true>(P, a, fin, b, o, lane, item_is_zero(P, load_bits(a.bitstrings, b, a.words)));
 }
 
 // ------------------------------------------------------------------ fused engine
@@ -364,6 +368,7 @@ __device__ __forceinline__ LaneWork lane_work(uint32_t m, const FusedStep *steps
 }
 
 // The lane's entries of its step, with the summed-index loop unrolled by case.
+template <int WARPS>
 __device__ __forceinline__ void run_lane_work(const LaneWork &w) {
     const uint32_t n_out = 1u << (w.info & 0xffu), nk = (w.info >> 8) & 0xffu;
     const bool unary = (w.info >> 16) & 1u;
@@ -387,7 +392,7 @@ __device__ __forceinline__ void run_lane_work(const LaneWork &w) {
         }
     } else if (!unary && nk == 1) {
         uint32_t c = w.sub;
-        for (; c + 3 * w.cnt < n_out; c += 4 * w.cnt) {   // four entries: loads of all issued first
+        for (; WARPS <= 16 && c + 3 * w.cnt < n_out; c += 4 * w.cnt) {   // four entries: loads of all issued first
             uint32_t e[4];
             float2 p[4], q[4], r[4], t[4];
 #pragma unroll
@@ -432,7 +437,26 @@ __device__ __forceinline__ void run_lane_work(const LaneWork &w) {
     } else if (!unary && nk == 2) {
         lane_entries_k<2>(*w.stp, w.sub, w.cnt, n_out, w.tab, A, B, w.C);
     } else if (!unary && nk == 3) {
-        lane_entries_k<3>(*w.stp, w.sub, w.cnt, n_out, w.tab, A, B, w.C);
+        if constexpr (WARPS <= 16) {
+            lane_entries_k<3>(*w.stp, w.sub, w.cnt, n_out, w.tab, A, B, w.C);
+        } else {   // four summed entries at a time: 64 or 80 registers
+            for (uint32_t c = w.sub; c < n_out; c += w.cnt) {
+                const uint32_t e = w.tab[c], ia = e & 0xffffu, ib = e >> 16;
+                float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int h = 0; h < 8; h += 4) {
+                    float2 p[4], q[4];
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        p[k] = A[ia + w.stp->koff_a[h + k]];
+                        q[k] = B[ib + w.stp->koff_b[h + k]];
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; k++) cmac(acc, p[k], q[k]);
+                }
+                w.C[c] = acc;
+            }
+        }
     } else {
         for (uint32_t c = w.sub; c < n_out; c += w.cnt) w.C[c] = fused_entry(*w.stp, w.tab[c], A, B, unary);
     }
@@ -443,37 +467,46 @@ __device__ __forceinline__ void run_lane_work(const LaneWork &w) {
 // access is a shared-memory access; otherwise the program is read from global memory.
 // Header fields are read once into registers. Each phase's lane work is prepared one
 // phase ahead, so a phase's critical path is its operand loads, FMAs, store and barrier.
-template <bool STAGED>
-__global__ void __launch_bounds__(512) fused_program_kernel(LaunchArgs a, int warps_per_item) {
+// WARPS: most warps of a CTA. 16 get up to 128 registers a thread and two entries with eight
+// summed entries at a time; 24 and 32 (fused_shape says when) get 80 and 64 and take such entries
+// one at a time. Spilled registers cost more than the warps give: with 64 registers for 16 warps
+// 7 amplitudes of a 6 x 7 grid at depth 26 took 94 us, with 128 they take 73 (88 with generic loads).
+template <bool STAGED, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 1) fused_program_kernel(LaunchArgs a, int warps_per_item) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(8) uint64_t stage_bar;
+    __shared__ FinishInfo fin;   // (kept out of the registers: it is used once per item)
     const unsigned char *img = a.image;
     const DevProgram *P = reinterpret_cast<const DevProgram *>(img);
     const uint64_t steps_off = a.fused_steps_off, tab_off = a.fused_tab_off, map_off = a.fused_lane_map_off;
     const uint32_t n_phases = a.n_fused_phases, n_leaves = a.n_leaves;
     const uint64_t final_off = a.final_off;
-    const DevLeaf *leaves = reinterpret_cast<const DevLeaf *>(img + a.leaves_off);
-    const FusedStep *steps = reinterpret_cast<const FusedStep *>(img + steps_off);
-    const uint32_t *tabs = reinterpret_cast<const uint32_t *>(img + tab_off);
-    const uint32_t *lane_map = reinterpret_cast<const uint32_t *>(img + map_off);
-    const float2 *ldata = reinterpret_cast<const float2 *>(img + a.leaf_data_off);
-    unsigned char *cur = smem;
+    // where the program lies. With STAGED these have to be addresses in shared memory on every
+    // path: where they may be either, all operand accesses become generic loads of 64-bit addresses
+    const uint32_t s1 = STAGED ? a.smem_steps_bytes : 0u, s2 = s1 + (STAGED ? a.smem_leaf_bytes : 0u);
+    const uint32_t s3 = s2 + (STAGED ? a.smem_leaves_bytes : 0u);
+    const FusedStep *steps = reinterpret_cast<const FusedStep *>(STAGED ? smem : img + steps_off);
+    const uint32_t *tabs = reinterpret_cast<const uint32_t *>(STAGED ? smem + (tab_off - steps_off) : img + tab_off);
+    const uint32_t *lane_map = reinterpret_cast<const uint32_t *>(STAGED ? smem + (map_off - steps_off) : img + map_off);
+    const float2 *ldata = reinterpret_cast<const float2 *>(STAGED ? smem + s1 : img + a.leaf_data_off);
+    const DevLeaf *leaves = reinterpret_cast<const DevLeaf *>(STAGED ? smem + s2 : img + a.leaves_off);
+    unsigned char *cur = smem + s3;
     // the first item's bitstring is read while the program is being staged
     const int groups0 = blockDim.x / (32 * warps_per_item);
     const int64_t item0 = (int64_t)blockIdx.x * groups0 + threadIdx.x / (32 * warps_per_item);
     Bits x_next = item0 < a.batch * a.o_count ? load_bits(a.bitstrings, item0 / a.o_count, a.words) : Bits{0ull, 0ull};
     bool staged_ok = true;
     if (STAGED) {
-        const uint32_t s1 = a.smem_steps_bytes, s2 = s1 + a.smem_leaf_bytes, s3 = s2 + a.smem_leaves_bytes;
         const uint32_t bar = smem_u32(&stage_bar);
         if (threadIdx.x == 0) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(s3) : "memory");
-            if (s1) bulk_g2s(smem_u32(smem), steps, s1, bar);
-            if (a.smem_leaf_bytes) bulk_g2s(smem_u32(smem + s1), ldata, a.smem_leaf_bytes, bar);
-            if (a.smem_leaves_bytes) bulk_g2s(smem_u32(smem + s2), leaves, a.smem_leaves_bytes, bar);
+            if (s1) bulk_g2s(smem_u32(smem), img + steps_off, s1, bar);
+            if (a.smem_leaf_bytes) bulk_g2s(smem_u32(smem + s1), img + a.leaf_data_off, a.smem_leaf_bytes, bar);
+            if (a.smem_leaves_bytes) bulk_g2s(smem_u32(smem + s2), img + a.leaves_off, a.smem_leaves_bytes, bar);
+            fin = finish_info(P);
         }
         __syncthreads();
         const bool ok = mbar_wait(bar, 0, a.selftest_stage_timeout ? 0u : kWaitPolls);
@@ -484,18 +517,11 @@ __global__ void __launch_bounds__(512) fused_program_kernel(LaunchArgs a, int wa
             if (threadIdx.x == 0) atomicCAS(a.status, 0u, 4u /* QVX_ETIMEOUT */);
             mbar_wait(bar, 0, kWaitPolls);
             staged_ok = false;
-        } else {
-            steps = reinterpret_cast<const FusedStep *>(smem);
-            tabs = reinterpret_cast<const uint32_t *>(smem + (tab_off - steps_off));
-            lane_map = reinterpret_cast<const uint32_t *>(smem + (map_off - steps_off));
-            ldata = reinterpret_cast<const float2 *>(smem + s1);
-            leaves = reinterpret_cast<const DevLeaf *>(smem + s2);
-            cur = smem + s3;
         }
     } else {
+        if (threadIdx.x == 0) fin = finish_info(P);
         __syncthreads();
     }
-    const FinishInfo fin = finish_info(P);
     if (staged_ok) {
         const int lanes = 32 * warps_per_item;
         const int group = threadIdx.x / lanes;
@@ -513,6 +539,7 @@ __global__ void __launch_bounds__(512) fused_program_kernel(LaunchArgs a, int wa
             const Bits x = x_next;
             const int64_t item_next = item + (int64_t)gridDim.x * groups;
             if (item_next < n_items) x_next = load_bits(a.bitstrings, item_next / a.o_count, a.words);
+            const bool zero = item_is_zero(fin, x);
             for (uint32_t l = lane; l < n_leaves; l += lanes) lbase[l] = leaf_base(leaves[l], x, o);
             if (warps_per_item == 1) __syncwarp();
             else asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(lanes));
@@ -521,12 +548,12 @@ __global__ void __launch_bounds__(512) fused_program_kernel(LaunchArgs a, int wa
                 const uint32_t m_next =
                     ph + 1 < n_phases ? lane_map[(ph + 1) * (uint32_t)lanes + (uint32_t)lane] : 0xffffffffu;
                 const LaneWork next = lane_work<STAGED>(m_next, steps, tabs, ldata, lbase, arena);
-                if (w.active) run_lane_work(w);
+                if (w.active) run_lane_work<WARPS>(w);
                 if (warps_per_item == 1) __syncwarp();
                 else asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(lanes));
                 w = next;
             }
-            if (lane < 32) finish_item_t<false>(fin, a, arena + final_off, b, o, lane, x);
+            if (lane < 32) finish_item_t<false>(fin, a, arena + final_off, b, o, lane, zero);
             if (warps_per_item == 1) __syncwarp();
             else asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "r"(lanes));
         }
@@ -1588,6 +1615,13 @@ cudaError_t launch_grad_sum(const unsigned char *image, const ExactPair *gpart, 
     return counted(cudaGetLastError());
 }
 
+using FusedKernel = void (*)(LaunchArgs, int);
+static FusedKernel fused_kernel(bool staged, int threads) {
+    if (threads <= 32 * 16) return staged ? fused_program_kernel<true, 16> : fused_program_kernel<false, 16>;
+    if (threads <= 32 * 24) return staged ? fused_program_kernel<true, 24> : fused_program_kernel<false, 24>;
+    return staged ? fused_program_kernel<true, kFusedWarps> : fused_program_kernel<false, kFusedWarps>;
+}
+
 // The dynamic shared-memory limit is an attribute of the kernel function, shared by every
 // plan: raise it once per device to the most the device allows, never lower it.
 cudaError_t fused_prepare(size_t smem_bytes) {
@@ -1598,22 +1632,21 @@ cudaError_t fused_prepare(size_t smem_bytes) {
     if (dev >= 0 && dev < 64 && raised[dev]) return cudaSuccess;
     int optin = 0;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, fused_program_kernel<true>)) != cudaSuccess) return e;
-    const int limit = optin - (int)fa.sharedSizeBytes;
-    if ((size_t)limit < smem_bytes) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(fused_program_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(fused_program_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) != cudaSuccess)
-        return e;
+    for (int i = 0; i < 6; i++) {
+        const FusedKernel k = fused_kernel(i & 1, 32 * (16 + 8 * (i / 2)));
+        cudaFuncAttributes fa;
+        if ((e = cudaFuncGetAttributes(&fa, k)) != cudaSuccess) return e;
+        const int limit = optin - (int)fa.sharedSizeBytes;
+        if ((size_t)limit < smem_bytes) return cudaErrorInvalidValue;
+        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) != cudaSuccess) return e;
+    }
     if (dev >= 0 && dev < 64) raised[dev] = true;
     return cudaSuccess;
 }
 
 int fused_blocks_per_sm(int threads, size_t smem_bytes, bool staged) {
     int n = 0;
-    cudaError_t e = staged ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fused_program_kernel<true>, threads, smem_bytes)
-                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fused_program_kernel<false>, threads, smem_bytes);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fused_kernel(staged, threads), threads, smem_bytes);
     return e == cudaSuccess ? n : 0;
 }
 
@@ -1644,15 +1677,21 @@ bool fused_shape(const DevProgram *h, uint64_t arena_elems, int warps_per_item, 
     a->n_fused_phases = h->n_fused_phases;
     a->n_leaves = h->n_leaves;
     *shared = sh;
-    *max_ipc = (int)std::max<size_t>(1, std::min<size_t>(std::max(1, 8 / warps_per_item), (kBudget - sh) / *group));
+    // Warps that run at a time: one CTA fits an SM when the program is staged, and a phase is a
+    // chain of shared-memory latencies and a barrier (8 warps issued in 26 % of the cycles), so a
+    // CTA takes 24 warps, or 32 in groups of 8 and 16, of which 24 hold fewer. 64 amplitudes of
+    // the 6 x 6 grid at depth 25, groups of 4: 417 us with 8 warps, 302 with 16, 291 with 24, 323
+    // with 32; groups of 8: 629 / 766 / 598 / 575 us; of 16 (6 amplitudes): 140 us with 16 or 24,
+    // 117 with 32. (A group of several warps has a named barrier of its own: 1 to 15.)
+    const int by_warps = std::min((warps_per_item >= 8 ? kFusedWarps : 24) / warps_per_item, warps_per_item > 1 ? 15 : kFusedGroups);
+    *max_ipc = (int)std::max<size_t>(1, std::min<size_t>(by_warps, (kBudget - sh) / *group));
     return true;
 }
 
 cudaError_t launch_fused(const LaunchArgs &a, int warps_per_item, int items_per_cta, int grid,
                          size_t smem_bytes, cudaStream_t s) {
     const int threads = 32 * warps_per_item * items_per_cta;
-    if (a.smem_steps_bytes) fused_program_kernel<true><<<grid, threads, smem_bytes, s>>>(a, warps_per_item);
-    else fused_program_kernel<false><<<grid, threads, smem_bytes, s>>>(a, warps_per_item);
+    fused_kernel(a.smem_steps_bytes != 0, threads)<<<grid, threads, smem_bytes, s>>>(a, warps_per_item);
     return counted(cudaGetLastError());
 }
 

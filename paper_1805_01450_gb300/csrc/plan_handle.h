@@ -11,7 +11,7 @@ struct qvx_plan {
     // fused-engine launch shape, cached for the device it was computed on
     int launch_device = -1;
     int sms = 0;
-    int ctas_per_sm[9] = {0};   // by work items per CTA
+    int ctas_per_sm[qvx::kFusedGroups + 1] = {0};   // by work items per CTA
     // persistent-engine grid, cached for the device it was computed on
     int persist_device = -1, persist_grid = 0;
     // shared-memory gradient kernel: CTAs per SM (0: the global-memory kernel runs), CTAs per
