@@ -1289,53 +1289,63 @@ __global__ void __launch_bounds__(256) grad_program_kernel(GradArgs g) {
 // One output entry of the gradient program from its record: sum over the summed index of
 // X * Y, where an operand is the shared-memory arena, a restricted leaf (base in lbase), its
 // derivative, or the constant one.
+template <bool STAGED>
 __device__ __forceinline__ float2 grad_record_value(const uint4 rv, const float2 *arena, const uint32_t *lbase,
                                                     const float2 *ldata, const float2 *ddata,
                                                     const uint32_t *ktab) {
     const uint32_t meta = rv.x >> 16;
     const uint32_t xr = rv.y & 0xffffu, xo = rv.y >> 16, yr = rv.z & 0xffffu, yo = rv.z >> 16;
     const uint32_t xk = meta & 3u, yk = (meta >> 2) & 3u, nk = (meta >> 4) & 15u;
-    const float2 *X = xk == kOpArena ? arena + xr : xk == kOpLeaf ? ldata + lbase[xr] : xk == kOpDeriv ? ddata + lbase[xr] : nullptr;
-    const float2 *Y = yk == kOpArena ? arena + yr : yk == kOpLeaf ? ldata + lbase[yr] : yk == kOpDeriv ? ddata + lbase[yr] : nullptr;
+    const bool x1s = xk == kOpOne, y1s = yk == kOpOne;
+    const float2 *X, *Y;
+    if (STAGED) {   // all of it is shared memory: an index into it, so that the loads are not generic
+        const uint32_t lo = (uint32_t)(ldata - arena), dd = (uint32_t)(ddata - arena);
+        X = arena + (xo + (xk == kOpLeaf ? lo + lbase[xr] : xk == kOpDeriv ? dd + lbase[xr] : xr));
+        Y = arena + (yo + (yk == kOpLeaf ? lo + lbase[yr] : yk == kOpDeriv ? dd + lbase[yr] : yr));
+    } else {
+        X = (xk == kOpLeaf ? ldata + lbase[xr] : xk == kOpDeriv ? ddata + lbase[xr] : arena + xr) + xo;
+        Y = (yk == kOpLeaf ? ldata + lbase[yr] : yk == kOpDeriv ? ddata + lbase[yr] : arena + yr) + yo;
+    }
     const float2 one = make_float2(1.f, 0.f);
-    if (X) X += xo;
-    if (Y) Y += yo;
     float2 acc = make_float2(0.f, 0.f);
     if (nk == 2) {   // the three offset pairs first, so the six operand loads are independent
         const uint32_t k1 = ktab[rv.w], k2 = ktab[rv.w + 1], k3 = ktab[rv.w + 2];
-        const float2 x0 = X ? X[0] : one, y0 = Y ? Y[0] : one;
-        const float2 x1 = X ? X[k1 & 0xffffu] : one, y1 = Y ? Y[k1 >> 16] : one;
-        const float2 x2 = X ? X[k2 & 0xffffu] : one, y2 = Y ? Y[k2 >> 16] : one;
-        const float2 x3 = X ? X[k3 & 0xffffu] : one, y3 = Y ? Y[k3 >> 16] : one;
+        const float2 x0 = x1s ? one : X[0], y0 = y1s ? one : Y[0];
+        const float2 x1 = x1s ? one : X[k1 & 0xffffu], y1 = y1s ? one : Y[k1 >> 16];
+        const float2 x2 = x1s ? one : X[k2 & 0xffffu], y2 = y1s ? one : Y[k2 >> 16];
+        const float2 x3 = x1s ? one : X[k3 & 0xffffu], y3 = y1s ? one : Y[k3 >> 16];
         cmac(acc, x0, y0);
         cmac(acc, x1, y1);
         cmac(acc, x2, y2);
         cmac(acc, x3, y3);
         return acc;
     }
-    cmac(acc, X ? X[0] : one, Y ? Y[0] : one);
+    cmac(acc, x1s ? one : X[0], y1s ? one : Y[0]);
     if (nk == 1) {
-        cmac(acc, X ? X[rv.w & 0xffffu] : one, Y ? Y[rv.w >> 16] : one);
+        cmac(acc, x1s ? one : X[rv.w & 0xffffu], y1s ? one : Y[rv.w >> 16]);
     } else if (nk > 2) {
 #pragma unroll 4
         for (uint32_t k = 1; k < (1u << nk); k++) {
             const uint32_t kp = ktab[rv.w + k - 1];
-            cmac(acc, X ? X[kp & 0xffffu] : one, Y ? Y[kp >> 16] : one);
+            cmac(acc, x1s ? one : X[kp & 0xffffu], y1s ? one : Y[kp >> 16]);
         }
     }
     return acc;
 }
 
-constexpr int kGradPrefetch = 4;   // records per thread loaded one phase ahead
+constexpr int kGradPrefetch = 1;   // records per thread loaded ahead
 
 // The gradient program with the work item's arena in shared memory: the records of each
 // level phase are spread over the CTA's threads, one barrier per phase, and each thread
-// loads its first record of the next phase before the barrier of the current one.
+// loads its first record two phases ahead: a phase of some 200 entries is over before a record
+// comes from L2. Latency bound (3 CTAs fit an SM by their arenas). The Jacobian of 16
+// amplitudes of a 5 x 5 grid of rotations at depth 20: 782 us with four records one phase ahead,
+// 768 / 670 / 662 us with four / two / one two phases ahead.
 // STAGED: the leaf data, the derivative data and the summed-index table are first copied
 // into shared memory (after the arena and the leaf table) by bulk asynchronous copies on one
 // mbarrier with a bounded wait, so the operand reads of every phase stay on chip.
 template <bool STAGED>
-__global__ void __launch_bounds__(256) grad_smem_kernel(GradArgs g) {
+__global__ void __launch_bounds__(256, 3) grad_smem_kernel(GradArgs g) {
     extern __shared__ float4 gsm[];
     __shared__ __align__(8) uint64_t stage_bar;
     const unsigned char *img = g.image;
@@ -1381,32 +1391,42 @@ __global__ void __launch_bounds__(256) grad_smem_kernel(GradArgs g) {
         const uint64_t o = (uint64_t)(item % g.o_count);
         const Bits x = load_bits(g.bitstrings, b, g.words);
         for (uint32_t l = threadIdx.x; l < n_leaves; l += blockDim.x) lbase[l] = leaf_base(leaves[l], x, o);
-        // a thread's first kGradPrefetch records of a phase are loaded during the phase before
-        uint4 cur[kGradPrefetch];
-#pragma unroll
-        for (int j = 0; j < kGradPrefetch; j++) {
-            const uint32_t e = pe[0] + threadIdx.x + j * blockDim.x;
-            cur[j] = n_phases > 0 && e < pe[1] ? rec[e] : make_uint4(0u, 0u, 0u, 0u);
-        }
-        __syncthreads();
-        for (uint32_t ph = 0; ph < n_phases; ph++) {
-            const uint32_t e0 = pe[ph], e1 = pe[ph + 1];
-            uint4 nxt[kGradPrefetch];
+        // a thread's first kGradPrefetch records of a phase are loaded two phases before
+        uint4 cur[kGradPrefetch], nxt[kGradPrefetch];
+        auto first_records = [&](uint4 *r, uint32_t begin, uint32_t end) {
 #pragma unroll
             for (int j = 0; j < kGradPrefetch; j++) {
-                const uint32_t e = e1 + threadIdx.x + j * blockDim.x;
-                nxt[j] = ph + 1 < n_phases && e < pe[ph + 2] ? rec[e] : make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t e = begin + threadIdx.x + j * blockDim.x;
+                r[j] = e < end ? rec[e] : make_uint4(0u, 0u, 0u, 0u);
             }
+        };
+        // first records of the phase at hand and of the three after it (none past the last)
+        auto bound = [&](uint32_t ph) { return pe[ph < n_phases ? ph : n_phases]; };
+        uint32_t e0 = bound(0), e1 = bound(1), e2 = bound(2), e3 = bound(3);
+        first_records(cur, e0, e1);
+        first_records(nxt, e1, e2);
+        __syncthreads();
+        for (uint32_t ph = 0; ph < n_phases; ph++) {
+            uint4 after[kGradPrefetch];
+            first_records(after, e2, e3);
+            const uint32_t e4 = bound(ph + 4);
 #pragma unroll
             for (int j = 0; j < kGradPrefetch; j++)
                 if (e0 + threadIdx.x + j * blockDim.x < e1)
-                    arena[cur[j].x & 0xffffu] = grad_record_value(cur[j], arena, lbase, ldata, ddata, ktab);
+                    arena[cur[j].x & 0xffffu] = grad_record_value<STAGED>(cur[j], arena, lbase, ldata, ddata, ktab);
             for (uint32_t e = e0 + threadIdx.x + kGradPrefetch * blockDim.x; e < e1; e += blockDim.x) {
                 const uint4 rv = rec[e];
-                arena[rv.x & 0xffffu] = grad_record_value(rv, arena, lbase, ldata, ddata, ktab);
+                arena[rv.x & 0xffffu] = grad_record_value<STAGED>(rv, arena, lbase, ldata, ddata, ktab);
             }
 #pragma unroll
-            for (int j = 0; j < kGradPrefetch; j++) cur[j] = nxt[j];
+            for (int j = 0; j < kGradPrefetch; j++) {
+                cur[j] = nxt[j];
+                nxt[j] = after[j];
+            }
+            e0 = e1;
+            e1 = e2;
+            e2 = e3;
+            e3 = e4;
             __syncthreads();
         }
         const bool zero = bits_hit(x, P->zero_mask, P->zero_mask_hi);
