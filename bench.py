@@ -8,7 +8,7 @@ variant kept for this circuit (recorded below: the ordering and sliced variables
 planning trials, stored in paper_1805_01450_gb300/orderings/; --autotune re-runs the
 autotuner instead). A
 step is one whole amplitude: every slice term, every pairwise contraction (the dense ones
-on the tcgen05 tensor cores as three-part bf16 GEMMs, the rest as FP32 SIMT kernels) and
+on the tcgen05 tensor cores as GEMMs of split 16-bit parts, the rest as FP32 SIMT kernels) and
 the exact sum of the slice terms.
 
 Prints one JSON line. Timing: CUDA events on the launching stream around each step, W
@@ -78,14 +78,14 @@ L2_FLUSH_BYTES = 256 << 20
 # over its launches in one ncu launch list of the workload's timed plan (profiles/ holds
 # the summaries and commands). Keyed by (workload, circuit seed, kernel, device image bytes
 # of the plan): another plan, or a kernel changed since the capture, reports null.
-NCU_TRAFFIC = {("grid8x8d40", 5001, "gemm_tc_kernel", 241664): 10230352774.4,
-               ("grid8x8d40", 5001, "regtile_step_kernel", 241664): 1338227991.4}
+# The captures of the kernels before the merged contractions are gone from here.
+NCU_TRAFFIC = {}
 # FP32 SIMT peak for the "alu" bound: 152 SMs x 128 FP32 lanes x 2 flops (FMA) x 2.07 GHz
 FP32_SIMT_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
-# the tensor-core contraction spends 48 bf16 flops per complex multiply-add (4 real MACs of
-# the real block form, each as 6 products of three-part bf16 splits) against 8 algorithmic
-# flops, so its algorithmic peak is 8/48 of the bf16 rate
-TC_ALGO_PER_BF16 = 8.0 / 48.0
+# the tensor-core contraction spends 24 16-bit flops per complex multiply-add (4 real MACs of
+# the real block form, each as 3 products of two-part fp16 splits) against 8 algorithmic
+# flops, so its algorithmic peak is 8/24 of the bf16 rate (fp16 runs at the same)
+TC_ALGO_PER_BF16 = 8.0 / 24.0
 
 
 def parse(argv=None):
@@ -103,7 +103,7 @@ def parse(argv=None):
     ap.add_argument("--warps-per-item", type=int, default=None)
     ap.add_argument("--host-merge-rank", type=int, default=8, help="fixed plan variant: leaf products contracted at plan time")
     ap.add_argument("--tensor-cores", action="store_true",
-                    help="stepwise engine: dense contractions as three-part bf16 GEMMs on the tensor cores")
+                    help="stepwise engine: dense contractions as GEMMs of split 16-bit parts on the tensor cores")
     ap.add_argument("--engine", default="auto")
     ap.add_argument("--sliced", type=int, default=None, help="override the workload's sliced-variable count")
     ap.add_argument("--plan-trials", type=int, default=None, help="planning trials (workload default)")
