@@ -1749,9 +1749,11 @@ cudaError_t launch_splitk_step(const LaunchArgs &a, uint32_t step, int64_t item_
 template <int RM, int RN>
 static TileForm tile_form(const RegTileStep &rs, uint64_t blocks, uint32_t *per_cta) {
     *per_cta = 1u;
-    // (the 32-bit byte offsets of a thread hold operands and results of up to 2^29 entries)
+    // 8 x 8 tiles are bound by their multiply-adds and registers: 38.4 ms flat, 43.5 in blocks (a step
+    // of 28 flops per byte, circuit 5001 of the 8 x 8 grid without tensor cores). (The 32-bit byte
+    // offsets of a thread hold operands and results of up to 2^29 entries.)
     const int rank_a = rs.a_cb + rs.nk_ab + rs.nk_a, rank_b = rs.b_cb + rs.nk_ab + rs.nk_b;
-    if (rs.nt < RegTileShape<RM, RN>::kThreadBits || std::max({rank_a, rank_b, (int)rs.rc}) > 29) return kTilesFlat;
+    if (RM + RN == 6 || rs.nt < RegTileShape<RM, RN>::kThreadBits || std::max({rank_a, rank_b, (int)rs.rc}) > 29) return kTilesFlat;
     const uint32_t most = std::min(kMaxTileBlocks, 1u << (rs.nt - RegTileShape<RM, RN>::kThreadBits));
     while (*per_cta < most && blocks / (2u * *per_cta) >= kMinTileCtas) *per_cta *= 2u;
     if (*per_cta == 1u) return rs.nk_ab + rs.nk_a + rs.nk_b < 3 ? kTilesFlat : kTilesBlocks;
@@ -1798,10 +1800,11 @@ static void launch_regtile_t(const LaunchArgs &a, const RegTileStep &rs, int64_t
         if (form == kTilesSwapped)
             return launch_regtile_f<RM, RN, kTilesSwapped>(a, swapped(rs), item_begin, n_items, arenas, max_c, blocks, per_cta, s);
     }
-    if (form == kTilesFlat)
-        launch_regtile_f<RM, RN, kTilesFlat>(a, rs, item_begin, n_items, arenas, max_c, blocks, 1u, s);
-    else
-        launch_regtile_f<RM, RN, kTilesBlocks>(a, rs, item_begin, n_items, arenas, max_c, blocks, per_cta, s);
+    if constexpr (RM + RN < 6) {
+        if (form == kTilesBlocks)
+            return launch_regtile_f<RM, RN, kTilesBlocks>(a, rs, item_begin, n_items, arenas, max_c, blocks, per_cta, s);
+    }
+    launch_regtile_f<RM, RN, kTilesFlat>(a, rs, item_begin, n_items, arenas, max_c, blocks, 1u, s);
 }
 
 cudaError_t launch_regtile_step(const LaunchArgs &a, const RegTileStep &rs, int64_t item_begin, int64_t n_items,
