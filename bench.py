@@ -450,7 +450,9 @@ def run_reference(args, rank, world):
 def kernel_roofline(records, hbm_gbs, bf16_tflops):
     """Per-kernel totals of the timed launch log and the dominant kernel's roofline. Each
     launch's roofline time is max(bytes / HBM, flops / compute peak), the compute peak being
-    the FP32 SIMT rate, or the tensor cores' algorithmic rate for the GEMM kernel."""
+    the FP32 SIMT rate, or the tensor cores' algorithmic rate for the GEMM kernel. Bytes are
+    the contractions' own: a launch that runs two contractions counts the result of the first,
+    which stays on chip, so the fraction of HBM can exceed 1."""
     per = {}
     for r in records:
         peak = bf16_tflops * TC_ALGO_PER_BF16 if r["kernel"] == "gemm_tc_kernel" else FP32_SIMT_TFLOPS
