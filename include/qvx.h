@@ -123,8 +123,12 @@ typedef struct {
                                   GEMMs on the tcgen05 tensor cores, each FP32 operand split into
                                   two scaled fp16 parts (three products) or, for circuits whose
                                   gate entries differ much in size, three bf16 parts (six
-                                  products), FP32 accumulation, about 2^-22 relative error per
-                                  product; 0 keeps them on FP32 SIMT kernels */
+                                  products), about 2^-22 relative error per product. They are added
+                                  in the tensor cores' FP32 accumulators, which truncate: at most 64
+                                  summed entries in a row with fp16 parts (a sum comes out up to
+                                  2^-21 too small in the mean; longer ones are added in FP32), all of
+                                  them with bf16 parts. Sums that need no rounding are exact. 0 keeps
+                                  the contractions on FP32 SIMT kernels */
     int32_t plan_trials;       /* 1 ... 65536 independent planning trials (ordering, slice choice and
                                   re-ordering, each from its own seed; trial 0 from order_seed);
                                   the plan with the smallest bandwidth-weighted contraction

@@ -31,6 +31,7 @@ cudaError_t launch_gemm_step(const LaunchArgs &a, const GemmStep &g, const GemmL
     ga.mt_bits = (uint32_t)__builtin_ctz(ga.n_mt);
     ga.nt_bits = (uint32_t)__builtin_ctz(ga.n_nt);
     ga.n_tiles = 0;
+    ga.run_bits = 0;
     if (leaf) return launch_counted(launch_gemm_leaf(ga, nt_cols, s));
     return launch_counted(scale ? launch_gemm_f16(ga, nt_cols, s) : launch_gemm_bf16(ga, nt_cols, s));
 }

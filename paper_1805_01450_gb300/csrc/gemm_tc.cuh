@@ -16,10 +16,8 @@
 //   kParts = 3: x = h + m + l in bf16 (8 bits each), the six products h*h + h*m + m*h + h*l +
 //     l*h + m*m; the dropped terms are below 2^-23 of the product. It has FP32's range and
 //     serves circuits whose gate entries differ too much in size (Plan::fp16_split).
-// What limits the accuracy is not the split but the accumulation: the tensor cores truncate
-// the FP32 accumulator at every MMA, so the error grows with the number of MMAs per entry, and
-// three products instead of six halve it (64-qubit circuit, error of the slice terms against
-// FP64: 3.2e-6 with six, 2.0e-6 with three). They also halve the MMAs and take a third off the operand
+// What limits the accuracy is not the split but the accumulation (group_chunks says how that is
+// kept short). Three products instead of six also halve the MMAs and take a third off the operand
 // parts stored in and read from shared memory, which bounds the loop. Two bf16 parts with three
 // products (about 2^-16 per product) are not accurate enough: on a 64-qubit circuit the
 // amplitude moved by 1.2e-5 of its size, above the 1e-5 tolerance.
@@ -112,6 +110,14 @@ __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.a
 template <uint32_t kRegs>
 __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs)); }
 
+// Tensor-memory columns of one accumulator.
+template <int NT>
+__host__ __device__ constexpr uint32_t acc_cols() { return NT < 32 ? 32u : (uint32_t)NT; }
+// Accumulators of the B-stationary form and of sums in runs: the narrower the column tile, the shorter a tile's
+// work against its fixed barrier round trips, so narrow tiles keep more tiles in flight
+// (tensor memory holds 512 columns: 2 x 256, 4 x 128, 8 x 64, 8 x 32).
+template <int NT>
+__host__ __device__ constexpr uint32_t bs_accs() { return 512u / acc_cols<NT>() < 8u ? 512u / acc_cols<NT>() : 8u; }
 // Operand stages of the shared-memory ring. With five (all that fit at 256 columns) the steps
 // ran 7 to 17 % slower, with two 6 to 8 %: shared memory that the ring does not take is L1 cache
 // for the columns.
@@ -211,30 +217,17 @@ __device__ __forceinline__ uint32_t scale_field(uint32_t m) {
 }
 __device__ __forceinline__ float pow2_field(uint32_t f) { return __uint_as_float(f << 23); }
 
-// The tensor cores truncate the FP32 accumulator at every MMA, which on average takes a part
-// kTrunc off its value. A sum of n_chunks chunks is built of M = 2 n_chunks increments (Ar, Ai
-// parts), each followed by three truncations (three products), and after increment j the partial
-// sum is, in the mean, j / M of the result, for terms of random signs as for terms of one sign:
-// the result is 3 kTrunc (M + 1) / 2 too small. That systematic part was nine tenths of the
-// error of the slice terms (64-qubit circuits, coefficient of a fit to the FP64 values: -1.8 to
-// -4.0e-6, rest 0.7 to 1.4e-6), so the epilogue's scale takes it back. kTrunc is the value that
-// these fits give over four programs with sums of 8 to 512 entries: 3.2e-8 +- 10 %.
-constexpr float kTrunc = 3.2e-8f;
-__device__ __forceinline__ float truncation_gain(uint32_t n_chunks) {
-    return 1.f + 1.5f * kTrunc * (float)(2u * n_chunks + 1u);
-}
-
 // What the epilogue multiplies an accumulator by to take out both operands' scales: 2^t with
 // t = 254 - fa - fb, in two factors when t is outside the float exponents.
 struct Unscale {
     float f1, f2;
     bool two;
 };
-__device__ __forceinline__ Unscale unscale_of(uint32_t ma, uint32_t mb, uint32_t n_chunks) {
+__device__ __forceinline__ Unscale unscale_of(uint32_t ma, uint32_t mb) {
     const int t = 254 - (int)scale_field(ma) - (int)scale_field(mb);
     const int t1 = max(-126, min(126, t)), t2 = max(-126, min(126, t - t1));
     Unscale u;
-    u.f1 = pow2_field((uint32_t)(t1 + 127)) * truncation_gain(n_chunks);
+    u.f1 = pow2_field((uint32_t)(t1 + 127));
     u.f2 = pow2_field((uint32_t)(t2 + 127));
     u.two = t2 != 0;
     return u;
@@ -268,27 +261,42 @@ __device__ __forceinline__ void mma_f16kind(uint32_t tmem, uint64_t ad, uint64_t
         : "memory");
 }
 
-// The products of one chunk: 2 parts (Ar, Ai) x 3 (fp16) or 6 (bf16) pairs of levels, into the
-// accumulator d (overwritten by the first product when `first`).
+// The products of one chunk, 2 parts (Ar, Ai) each: of two fp16 parts the small ones (h*l, l*h)
+// and the large one (h*h) apart, of three bf16 parts all six. The accumulator d is overwritten
+// by the first product when `first`.
 template <int kParts>
-__device__ __forceinline__ void mma_chunk(uint32_t d, uint32_t sa, uint32_t ra, const uint32_t (&sb)[2][kParts], uint32_t idesc,
-                                          bool first) {
+struct ChunkDesc {
+    uint64_t a[2][kParts], b[2][kParts];
+    __device__ __forceinline__ ChunkDesc(uint32_t sa, uint32_t ra, const uint32_t (&sb)[2][kParts]) {
+#pragma unroll
+        for (uint32_t p = 0; p < 2; p++)
+#pragma unroll
+            for (uint32_t q = 0; q < (uint32_t)kParts; q++) {
+                a[p][q] = smem_desc(sa + (kParts * p + q) * ra, 128u, kPitch);
+                b[p][q] = smem_desc(sb[p][q], 128u, kPitch);
+            }
+    }
+};
+__device__ __forceinline__ void mma_small(uint32_t d, const ChunkDesc<2> &c, uint32_t idesc, bool first) {
 #pragma unroll
     for (uint32_t p = 0; p < 2; p++) {
-        uint64_t ad[kParts], bd[kParts];
+        mma_f16kind(d, c.a[p][0], c.b[p][1], idesc, !(first && p == 0u));
+        mma_f16kind(d, c.a[p][1], c.b[p][0], idesc, 1u);
+    }
+}
+__device__ __forceinline__ void mma_large(uint32_t d, const ChunkDesc<2> &c, uint32_t idesc) {
 #pragma unroll
-        for (uint32_t q = 0; q < (uint32_t)kParts; q++) {
-            ad[q] = smem_desc(sa + (kParts * p + q) * ra, 128u, kPitch);
-            bd[q] = smem_desc(sb[p][q], 128u, kPitch);
-        }
-        mma_f16kind(d, ad[0], bd[0], idesc, !(first && p == 0u));
-        mma_f16kind(d, ad[0], bd[1], idesc, 1u);
-        mma_f16kind(d, ad[1], bd[0], idesc, 1u);
-        if constexpr (kParts == 3) {
-            mma_f16kind(d, ad[0], bd[2], idesc, 1u);
-            mma_f16kind(d, ad[2], bd[0], idesc, 1u);
-            mma_f16kind(d, ad[1], bd[1], idesc, 1u);
-        }
+    for (uint32_t p = 0; p < 2; p++) mma_f16kind(d, c.a[p][0], c.b[p][0], idesc, 1u);
+}
+__device__ __forceinline__ void mma_six(uint32_t d, const ChunkDesc<3> &c, uint32_t idesc, bool first) {
+#pragma unroll
+    for (uint32_t p = 0; p < 2; p++) {
+        mma_f16kind(d, c.a[p][0], c.b[p][0], idesc, !(first && p == 0u));
+        mma_f16kind(d, c.a[p][0], c.b[p][1], idesc, 1u);
+        mma_f16kind(d, c.a[p][1], c.b[p][0], idesc, 1u);
+        mma_f16kind(d, c.a[p][0], c.b[p][2], idesc, 1u);
+        mma_f16kind(d, c.a[p][2], c.b[p][0], idesc, 1u);
+        mma_f16kind(d, c.a[p][1], c.b[p][1], idesc, 1u);
     }
 }
 
@@ -409,56 +417,59 @@ __device__ __forceinline__ void warp_arrive(uint32_t bar) {
     if ((threadIdx.x & 31u) == 0u) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// kW Re columns and kW Im columns of this warp's 32 tensor-memory lanes into registers (one
-// column per register), waited for.
-template <uint32_t kW>
-__device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, uint32_t (&r)[kW]) {
-    if constexpr (kW == 16) {
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
-            "%12, %13, %14, %15}, [%16];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(taddr));
-    } else {
-        static_assert(kW == 8, "8 or 16 columns");
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                     : "r"(taddr));
-    }
-}
-template <uint32_t kW>
-__device__ __forceinline__ void tmem_ld(uint32_t re_addr, uint32_t im_addr, uint32_t (&re)[kW], uint32_t (&im)[kW]) {
-    tmem_ld_issue<kW>(re_addr, re);
-    tmem_ld_issue<kW>(im_addr, im);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// kW accumulator columns of this warp's 32 tensor-memory lanes into registers (one column
-// per register), waited for.
+// kW accumulator columns of this warp's 32 tensor-memory lanes into registers (one column per
+// register). The load and its wait are one asm statement: the registers hold nothing before it.
 template <uint32_t kW>
 __device__ __forceinline__ void tmem_ld_pairs(uint32_t taddr, uint32_t (&r)[kW]) {
     if constexpr (kW == 32) {
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
             "%12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, "
-            "%30, %31}, [%32];"
+            "%30, %31}, [%32];\n tcgen05.wait::ld.sync.aligned;"
             : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
               "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
               "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),
               "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
               "=r"(r[30]), "=r"(r[31])
-            : "r"(taddr));
-    } else {
-        static_assert(kW == 16, "16 or 32 columns");
+            : "r"(taddr) : "memory");
+    } else if constexpr (kW == 16) {
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
-            "%12, %13, %14, %15}, [%16];"
+            "%12, %13, %14, %15}, [%16];\n tcgen05.wait::ld.sync.aligned;"
             : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
               "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(taddr));
+            : "r"(taddr) : "memory");
+    } else {
+        static_assert(kW == 8, "8, 16 or 32 columns");
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                     " tcgen05.wait::ld.sync.aligned;"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "r"(taddr) : "memory");
     }
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// The same of kW Re columns and kW Im columns, both loads under one wait.
+template <uint32_t kW>
+__device__ __forceinline__ void tmem_ld(uint32_t re_addr, uint32_t im_addr, uint32_t (&re)[kW], uint32_t (&im)[kW]) {
+    if constexpr (kW == 16) {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+            "%12, %13, %14, %15}, [%32];\n"
+            " tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
+            "%28, %29, %30, %31}, [%33];\n tcgen05.wait::ld.sync.aligned;"
+            : "=r"(re[0]), "=r"(re[1]), "=r"(re[2]), "=r"(re[3]), "=r"(re[4]), "=r"(re[5]), "=r"(re[6]), "=r"(re[7]),
+              "=r"(re[8]), "=r"(re[9]), "=r"(re[10]), "=r"(re[11]), "=r"(re[12]), "=r"(re[13]), "=r"(re[14]), "=r"(re[15]),
+              "=r"(im[0]), "=r"(im[1]), "=r"(im[2]), "=r"(im[3]), "=r"(im[4]), "=r"(im[5]), "=r"(im[6]), "=r"(im[7]),
+              "=r"(im[8]), "=r"(im[9]), "=r"(im[10]), "=r"(im[11]), "=r"(im[12]), "=r"(im[13]), "=r"(im[14]), "=r"(im[15])
+            : "r"(re_addr), "r"(im_addr) : "memory");
+    } else {
+        static_assert(kW == 8, "8 or 16 columns");
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n"
+                     " tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n"
+                     " tcgen05.wait::ld.sync.aligned;"
+                     : "=r"(re[0]), "=r"(re[1]), "=r"(re[2]), "=r"(re[3]), "=r"(re[4]), "=r"(re[5]), "=r"(re[6]), "=r"(re[7]),
+                       "=r"(im[0]), "=r"(im[1]), "=r"(im[2]), "=r"(im[3]), "=r"(im[4]), "=r"(im[5]), "=r"(im[6]), "=r"(im[7])
+                     : "r"(re_addr), "r"(im_addr) : "memory");
+    }
 }
 
 }  // namespace
@@ -473,6 +484,7 @@ struct GemmArgs {
     float2 *arenas;
     uint32_t n_chunks, n_mt, n_nt;
     uint32_t stages;               // A stages of the B-stationary form
+    uint32_t run_bits;             // log2 of the chunks of an accumulator run (kRuns)
     uint32_t mt_bits, nt_bits;     // log2 of n_mt and n_nt (every tile count is a power of two)
     uint64_t n_tiles;
 };
@@ -530,6 +542,93 @@ __device__ __forceinline__ bool wait_or_fail(uint32_t bar, uint32_t parity, vola
 // warp-wide operations, so their lanes must leave them together.
 __device__ __forceinline__ bool warp_wait_or_fail(uint32_t bar, uint32_t parity, volatile int *fail) {
     return __all_sync(0xffffffffu, wait_or_fail(bar, parity, fail));
+}
+
+// The tensor cores truncate the accumulator at every MMA, relative to the value that it has by
+// then, so a long sum comes out too small (by 3e-8 a truncation in the mean, over three times the
+// rounding of an FP32 sum of such length). Two parts of fp16 keep the truncations of full size few:
+//  - chunks go to an accumulator in groups of two or four, first the small products (h*l, l*h) of
+//    all of them, then the large ones: an MMA costs accuracy only once large products are in, 2 of
+//    a chunk's 6 instead of all;
+//  - sums of more chunks run in several accumulators, added in FP32 by the epilogue (kRuns):
+//    a tile has a pair of them, the first for its first run and the sum, the second for the others.
+// Slice terms of 64-qubit circuits, relative error against FP64: 5.9e-7, 6.5e-7 and 9.4e-7
+// (all products in order in one accumulator: 6e-6, 2.9e-6 and 5.4e-6 too small; six bf16 products,
+// without merged steps: 3.3e-6, 2.3e-6 and 4.2e-6), and sums that need no rounding are exact.
+// A constant gain in place of this is right for no particular sum.
+template <int kParts>
+__host__ __device__ constexpr uint32_t group_chunks() { return kParts == 2 ? 2u : 1u; }
+
+// Accumulator of run r of the CTA's tile number n, and how often it was used before.
+template <uint32_t NA>
+struct RunSlot {
+    uint32_t buf, uses;
+    __device__ __forceinline__ RunSlot(uint32_t n, uint32_t r, uint32_t runs) {
+        const uint32_t before = n / (NA / 2u);
+        buf = 2u * (n % (NA / 2u)) + (r ? 1u : 0u);
+        uses = r ? before * (runs - 1u) + r - 1u : before;
+    }
+};
+
+// The MMA thread's part of a group of n chunks, from the ring's next stages into accumulator d:
+// waits for the stages, issues the products, and commits the stages' release. first: the group
+// overwrites the accumulator. b_at(i, s, bs): the addresses of the B parts of the group's chunk i
+// (ring stage s) into bs.
+template <int kParts, class BAt>
+__device__ __forceinline__ bool mma_group(uint32_t d, uint32_t n, bool first, RingPos &ring, uint32_t S, uint32_t stages,
+                                          uint32_t stage_bytes, uint32_t region, uint64_t *full, uint64_t *empty, const BAt &b_at,
+                                          uint32_t idesc, volatile int *fail) {
+    RingPos at = ring;
+    for (uint32_t i = 0; i < n; i++, at.next(S)) {
+        if (!wait_or_fail(smem_u32(&full[at.s]), at.phase, fail)) return false;
+        tc_fence_after();
+        uint32_t bs[2][kParts];
+        b_at(i, at.s, bs);
+        const ChunkDesc<kParts> c(stages + at.s * stage_bytes, region, bs);
+        if constexpr (kParts == 2) mma_small(d, c, idesc, first && i == 0u);
+        else mma_six(d, c, idesc, first && i == 0u);
+    }
+    if constexpr (kParts == 2) {
+        at = ring;
+        for (uint32_t i = 0; i < n; i++, at.next(S)) {
+            uint32_t bs[2][kParts];
+            b_at(i, at.s, bs);
+            mma_large(d, ChunkDesc<kParts>(stages + at.s * stage_bytes, region, bs), idesc);
+            mma_commit(smem_u32(&empty[at.s]));
+        }
+    } else {
+        mma_commit(smem_u32(&empty[ring.s]));
+    }
+    ring = at;
+    return true;
+}
+
+// Adds kW accumulator columns to registers, and to other columns (tensor memory), in FP32.
+template <uint32_t kW>
+__device__ __forceinline__ void add_columns(uint32_t (&sum)[kW], uint32_t taddr) {
+    uint32_t v[kW];
+    tmem_ld_pairs<kW>(taddr, v);
+#pragma unroll
+    for (uint32_t i = 0; i < kW; i++) sum[i] = __float_as_uint(__uint_as_float(sum[i]) + __uint_as_float(v[i]));
+}
+template <uint32_t kW>
+__device__ __forceinline__ void tmem_add(uint32_t to, uint32_t from) {
+    uint32_t v[kW];
+    tmem_ld_pairs<kW>(to, v);
+    add_columns<kW>(v, from);
+    if constexpr (kW == 16) {
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                     "%13, %14, %15, %16};\n tcgen05.wait::st.sync.aligned;" ::"r"(to),
+                     "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+                     "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+                     : "memory");
+    } else {
+        static_assert(kW == 8, "8 or 16 columns");
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n"
+                     " tcgen05.wait::st.sync.aligned;" ::"r"(to),
+                     "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                     : "memory");
+    }
 }
 
 struct TileCoord {
@@ -613,17 +712,17 @@ struct BsCursor {
 // memory is freed, and QVX_ETIMEOUT goes to the status word.
 // kLeaf: one operand is multiplied by a leaf between its load and its split, so that a
 // contraction and the leaf contraction of its result are one pass with a longer summed index
-// (find_pairs in planner.cpp).
-template <int NT, int kParts, bool kLeaf>
+// (find_pairs in planner.cpp). kRuns: a tile's sum in several accumulator runs.
+template <int NT, int kParts, bool kLeaf, bool kRuns>
 __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArgs ga) {
     constexpr uint32_t kMmaWarp = mma_warp<NT>(), kEpiWarp = epi_warp<NT>();
     constexpr uint32_t S = n_stages<NT, kParts>();
-    constexpr uint32_t kCols = NT < 32 ? 32u : (uint32_t)NT;   // columns of one accumulator
+    constexpr uint32_t kCols = acc_cols<NT>(), NA = kRuns ? bs_accs<NT>() : 2u;   // accumulators
     constexpr uint32_t kRegA = region_bytes(kRows), kStage = stage_bytes<NT, kParts>();
     constexpr uint32_t kW = epi_cols<NT>();
     constexpr uint32_t kNc = (uint32_t)NT / 2u;   // complex columns per tile
     extern __shared__ __align__(1024) unsigned char gsm[];
-    __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], accf_bar[2], acce_bar[2], drain_bar;
+    __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], accf_bar[NA], acce_bar[NA], drain_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int fail;
     const GemmStep &g = ga.g;
@@ -634,7 +733,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
             mbar_init(smem_u32(&full_bar[s]), kMmaWarp);
             mbar_init(smem_u32(&empty_bar[s]), 1);
         }
-        for (uint32_t b = 0; b < 2; b++) {
+        for (uint32_t b = 0; b < NA; b++) {
             mbar_init(smem_u32(&accf_bar[b]), 1);
             mbar_init(smem_u32(&acce_bar[b]), kEpiThreads / 32u);
         }
@@ -644,7 +743,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
     }
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                     "r"(2u * kCols)
+                     "r"(NA * kCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -748,35 +847,33 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
         if (warp == kMmaWarp && lane == 0) {   // MMA issuer
             constexpr uint32_t idesc = mma_idesc<kParts>(NT);
             constexpr uint32_t kBlkB = b_block_bytes(NT);
+            const uint32_t group = min(group_chunks<kParts>(), ga.n_chunks), runs = ga.n_chunks >> ga.run_bits;
             RingPos ring;
             uint32_t j = 0;
             bool ok = true;
-            for (uint64_t t = blockIdx.x; t < ga.n_tiles && ok; t += gridDim.x, j++) {
-                const uint32_t buf = j & 1u;
-                if (!wait_or_fail(smem_u32(&acce_bar[buf]), ((j >> 1) & 1u) ^ 1u, &fail)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t d = tmem + buf * kCols;
-                for (uint32_t c = 0; c < ga.n_chunks; c++, ring.next(S)) {
-                    const uint32_t s = ring.s;
-                    if (!wait_or_fail(smem_u32(&full_bar[s]), ring.phase, &fail)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t sa = sbase + s * kStage, sb = sa + a_bytes<kParts>();
-                    uint32_t bs[2][kParts];
+            auto b_at = [&](uint32_t, uint32_t stage, uint32_t (&bs)[2][kParts]) {
+                const uint32_t sb = sbase + stage * kStage + a_bytes<kParts>();
 #pragma unroll
-                    for (uint32_t q = 0; q < (uint32_t)kParts; q++) {
-                        bs[0][q] = sb + (3u * q + 1u) * kBlkB;   // [Br][Bi]
-                        bs[1][q] = sb + 3u * q * kBlkB;          // [-Bi][Br]
-                    }
-                    mma_chunk<kParts>(d, sa, kRegA, bs, idesc, c == 0u);
-                    mma_commit(smem_u32(&empty_bar[s]));
+                for (uint32_t q = 0; q < (uint32_t)kParts; q++) {
+                    bs[0][q] = sb + (3u * q + 1u) * kBlkB;   // [Br][Bi]
+                    bs[1][q] = sb + 3u * q * kBlkB;          // [-Bi][Br]
                 }
-                if (ok) mma_commit(smem_u32(&accf_bar[buf]));
+            };
+            for (uint64_t t = blockIdx.x; t < ga.n_tiles && ok; t += gridDim.x, j++) {
+                for (uint32_t c = 0; c < ga.n_chunks && ok; c += group) {
+                    const uint32_t run = c >> ga.run_bits, at = kRuns ? c & ((1u << ga.run_bits) - 1u) : c;
+                    const RunSlot<NA> slot(j, run, runs);
+                    const bool starts = at == 0u, ends = kRuns ? run != 0u && at + group == 1u << ga.run_bits : c + group >= ga.n_chunks;
+                    const uint32_t buf = kRuns ? slot.buf : j % NA;
+                    if (starts) {
+                        ok = wait_or_fail(smem_u32(&acce_bar[buf]), ((kRuns ? slot.uses : j / NA) & 1u) ^ 1u, &fail);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+                    ok = mma_group<kParts>(tmem + buf * kCols, group, starts, ring, S, sbase, kStage, kRegA, full_bar, empty_bar, b_at,
+                                           idesc, &fail);
+                    if (ok && ends) mma_commit(smem_u32(&accf_bar[buf]));
+                }
             }
             if (!ok) fail = 1;
             // every MMA issued so far completes before the tensor memory is freed
@@ -794,29 +891,48 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
         const uint32_t q = warp & 3u;
         const uint32_t share = (warp - kEpiWarp) >> 2;   // the two warps of a lane quarter split its columns
         uint32_t j = 0;
+        bool ok = true;
+        // this lane's row of C in a tile
+        auto row_of = [&](const TileCoord &tc) {
+            return ga.arenas + (uint64_t)tc.il * ga.a.arena_elems + g.c_off + pext_runs(tc.beta, g.cb, g.n_cb) +
+                   pext_runs(tc.mt * kRows + 32u * q + lane, g.cm, g.n_cm);
+        };
         uint32_t coff[kW];   // offsets of a block's columns in C
 #pragma unroll
         for (uint32_t i = 0; i < kW; i++) coff[i] = pext_runs(i, g.cn, g.n_cn);
-        const uint32_t own = pext_runs(32u * q + lane, g.cm, g.n_cm);
+        const uint32_t lanes = tmem + ((q * 32u) << 16);
+        const uint32_t runs = ga.n_chunks >> ga.run_bits;
         for (uint64_t t = blockIdx.x; t < ga.n_tiles; t += gridDim.x, j++) {
             const TileCoord tc = tile_coord(t, ga);
-            const uint32_t buf = j & 1u;
-            // this lane's row of C and the tile's base, while the MMAs run
-            float2 *Crow = ga.arenas + (uint64_t)tc.il * ga.a.arena_elems + g.c_off + pext_runs(tc.beta, g.cb, g.n_cb) +
-                           pext_runs(tc.mt * kRows, g.cm, g.n_cm) + own;
+            const RunSlot<NA> last(j, runs - 1u, runs);   // the last run, added to the sum as it is stored
+            const uint32_t buf = kRuns ? last.buf : j % NA;
+            float2 *Crow = row_of(tc);   // while the MMAs run
             Unscale un{1.f, 1.f, false};
-            if (kParts == 2) un = unscale_of(side_max<kLeaf>(ga, true, tc.il), side_max<kLeaf>(ga, false, tc.il), ga.n_chunks);
+            if (kParts == 2) un = unscale_of(side_max<kLeaf>(ga, true, tc.il), side_max<kLeaf>(ga, false, tc.il));
             uint32_t largest = 0;
-            if (!warp_wait_or_fail(smem_u32(&accf_bar[buf]), (j >> 1) & 1u, &fail)) {
-                fail = 1;
-                break;
+            if constexpr (kRuns) {
+                for (uint32_t r = 1; r + 1u < runs && ok; r++) {
+                    ok = warp_wait_or_fail(smem_u32(&accf_bar[buf]), RunSlot<NA>(j, r, runs).uses & 1u, &fail);
+                    if (!ok) break;
+                    tc_fence_after();
+                    for (uint32_t j0 = share * kW; j0 < (uint32_t)NT; j0 += 2u * kW)
+                        tmem_add<kW>(lanes + (buf - 1u) * kCols + j0, lanes + buf * kCols + j0);
+                    tc_fence_before();
+                    warp_arrive(smem_u32(&acce_bar[buf]));
+                }
             }
+            if (ok) ok = warp_wait_or_fail(smem_u32(&accf_bar[buf]), (kRuns ? last.uses : j / NA) & 1u, &fail);
+            if (!ok) break;
             tc_fence_after();
-            const uint32_t taddr = tmem + ((q * 32u) << 16) + buf * kCols;
+            const uint32_t taddr = lanes + buf * kCols;
             for (uint32_t j0 = share * kW; j0 < kNc; j0 += 2u * kW) {
                 float2 *Cblk = Crow + pext_runs(tc.nt * kNc + j0, g.cn, g.n_cn);
                 uint32_t re[kW], im[kW];
                 tmem_ld<kW>(taddr + j0, taddr + kNc + j0, re, im);
+                if constexpr (kRuns) {
+                    add_columns<kW>(re, taddr - kCols + j0);
+                    add_columns<kW>(im, taddr - kCols + kNc + j0);
+                }
 #pragma unroll
                 for (uint32_t i = 0; i < kW; i++) {
                     const float2 c = kParts == 2 ? unscaled(un, re[i], im[i])
@@ -825,17 +941,19 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
                     if (ga.max_c) largest = abs_max(largest, c);
                 }
             }
-            // the accumulator's reads are done: the MMAs of the tile after next may reuse it
+            // the accumulator's reads are done: the MMAs of a later tile may reuse it
             tc_fence_before();
             warp_arrive(smem_u32(&acce_bar[buf]));
+            if (kRuns) warp_arrive(smem_u32(&acce_bar[buf - 1u]));
             if (ga.max_c) note_max_warp(ga.max_c + tc.il, largest);
         }
+        if (!ok) fail = 1;
     }
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2u * kCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NA * kCols) : "memory");
     }
     if (fail && threadIdx.x == 0) atomicCAS(ga.a.status, 0u, 4u /* QVX_ETIMEOUT */);
 }
@@ -849,13 +967,6 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
 // the old one have completed. Against the streaming form this removes B's loads, splits and
 // stores from the loop (64-qubit circuit 5001: s118, 64 summed entries, 2.56 -> 1.88 ms, 292
 // algorithmic TFLOP/s).
-// Accumulators: the narrower the column tile, the shorter a tile's
-// work against its fixed barrier round trips, so narrow tiles keep more tiles in flight
-// (tensor memory holds 512 columns: 2 x 256, 4 x 128, 8 x 64, 8 x 32).
-template <int NT>
-__host__ __device__ constexpr uint32_t bs_cols() { return NT < 32 ? 32u : (uint32_t)NT; }   // one accumulator
-template <int NT>
-__host__ __device__ constexpr uint32_t bs_accs() { return 512u / bs_cols<NT>() < 8u ? 512u / bs_cols<NT>() : 8u; }
 template <int NT, int kParts>
 __host__ __device__ constexpr uint32_t bs_b_bytes() { return 2u * kParts * region_bytes(NT); }   // one chunk of B
 // real accumulator columns an epilogue warp reads at a time
@@ -872,17 +983,18 @@ __host__ __device__ constexpr uint32_t bs_chunks() {
     return c;
 }
 template <int NT, int kParts>
-uint32_t bs_stages(uint32_t n_chunks) {
-    return std::min(kBsStages, (kBsBytes - n_chunks * (bs_b_bytes<NT, kParts>() + 12u * kKq)) / a_bytes<kParts>());
+constexpr uint32_t bs_stages(uint32_t n_chunks) {
+    const uint32_t fit = (kBsBytes - n_chunks * (bs_b_bytes<NT, kParts>() + 12u * kKq)) / a_bytes<kParts>();
+    return fit < kBsStages ? fit : kBsStages;
 }
 
-template <int NT, int kParts, bool kLeaf>   // kLeaf: one operand is multiplied by a leaf as it is split
+template <int NT, int kParts, bool kLeaf, bool kRuns>   // as gemm_tc_kernel
 __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(GemmArgs ga) {
     const uint32_t S = ga.stages;
     constexpr uint32_t NA = bs_accs<NT>();
     constexpr uint32_t PA = 256u, PB = b_threads<NT>();
     constexpr uint32_t kMmaWarp = mma_warp<NT>(), kEpiWarp = epi_warp<NT>();
-    constexpr uint32_t kCols = NT < 32 ? 32u : (uint32_t)NT;
+    constexpr uint32_t kCols = acc_cols<NT>();
     constexpr uint32_t kRegA = region_bytes(kRows), kRegB = region_bytes(NT);
     constexpr uint32_t kStage = a_bytes<kParts>(), kBChunk = bs_b_bytes<NT, kParts>();
     constexpr uint32_t kW = bs_epi_cols<NT>();
@@ -1050,6 +1162,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
         regs_dec<Regs<NT>::kBsIssue>();
         if (warp == kMmaWarp && lane == 0) {
             constexpr uint32_t idesc = mma_idesc<kParts>(NT);
+            const uint32_t group = min(kParts == 2 && !kRuns ? 4u : group_chunks<kParts>(), ga.n_chunks), runs = ga.n_chunks >> ga.run_bits;
             RingPos ring;
             uint32_t j = 0, gi = 0;
             bool ok = true;
@@ -1062,32 +1175,29 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
                     }
                     gi++;
                 }
-                const uint32_t buf = j % NA;
-                if (!wait_or_fail(smem_u32(&acce_bar[buf]), ((j / NA) & 1u) ^ 1u, &fail)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t d = tmem + buf * kCols;
-                for (uint32_t c = 0; c < ga.n_chunks; c++, ring.next(S)) {
-                    const uint32_t s = ring.s;
-                    if (!wait_or_fail(smem_u32(&full_bar[s]), ring.phase, &fail)) {
-                        ok = false;
-                        break;
+                for (uint32_t c = 0; c < ga.n_chunks && ok; c += group) {
+                    const uint32_t run = c >> ga.run_bits, at = kRuns ? c & ((1u << ga.run_bits) - 1u) : c;
+                    const RunSlot<NA> slot(j, run, runs);
+                    const bool starts = at == 0u, ends = kRuns ? run != 0u && at + group == 1u << ga.run_bits : c + group >= ga.n_chunks;
+                    const uint32_t buf = kRuns ? slot.buf : j % NA;
+                    if (starts) {
+                        ok = wait_or_fail(smem_u32(&acce_bar[buf]), ((kRuns ? slot.uses : j / NA) & 1u) ^ 1u, &fail);
+                        if (!ok) break;
+                        tc_fence_after();
                     }
-                    tc_fence_after();
-                    const uint32_t sa = sbase + s * kStage, sb = smem_u32(sB) + c * kBChunk;
-                    uint32_t bs[2][kParts];
+                    auto b_at = [&](uint32_t i, uint32_t, uint32_t (&bs)[2][kParts]) {
+                        const uint32_t sb = smem_u32(sB) + (c + i) * kBChunk;
 #pragma unroll
-                    for (uint32_t q = 0; q < (uint32_t)kParts; q++) {
-                        bs[0][q] = sb + q * kRegB;
-                        bs[1][q] = sb + (kParts + q) * kRegB;
-                    }
-                    mma_chunk<kParts>(d, sa, kRegA, bs, idesc, c == 0u);
-                    mma_commit(smem_u32(&empty_bar[s]));
+                        for (uint32_t q = 0; q < (uint32_t)kParts; q++) {
+                            bs[0][q] = sb + q * kRegB;
+                            bs[1][q] = sb + (kParts + q) * kRegB;
+                        }
+                    };
+                    ok = mma_group<kParts>(tmem + buf * kCols, group, starts, ring, S, sbase, kStage, kRegA, full_bar, empty_bar, b_at,
+                                           idesc, &fail);
+                    if (ok && ends) mma_commit(smem_u32(&accf_bar[buf]));
                 }
                 if (!ok) break;
-                mma_commit(smem_u32(&accf_bar[buf]));
                 // the column tile's last row tile in this range: its B regions may be reloaded
                 // once these MMAs have completed
                 if (t + 1u == t1 || ((t + 1u) >> ga.mt_bits) != grp) mma_commit(smem_u32(&bempty_bar));
@@ -1100,34 +1210,50 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
     } else {
         if constexpr (Regs<NT>::kBsEpi > Regs<NT>::kLaunch) regs_inc<Regs<NT>::kBsEpi>();
         else regs_dec<Regs<NT>::kBsEpi>();
-        const uint32_t q = warp & 3u;
+        const uint32_t q = warp & 3u, lanes = tmem + ((q * 32u) << 16);
+        const uint32_t runs = ga.n_chunks >> ga.run_bits;
+        constexpr uint32_t kSum = kW < 16u ? kW : 16u;   // columns added at a time
         const uint32_t share = (warp - kEpiWarp) >> 2;
         uint32_t j = 0;
+        BsCursor cur;
+        cur.c = tile_coord_bs(t0, ga);
+        bool ok = true;
+        // this lane's row of C in a tile
+        auto row_of = [&](const TileCoord &tc) {
+            return ga.arenas + (uint64_t)tc.il * ga.a.arena_elems + g.c_off + pext_runs(tc.beta, g.cb, g.n_cb) +
+                   pext_runs(tc.mt * kRows + 32u * q + lane, g.cm, g.n_cm);
+        };
         uint32_t coff[kW / 2u];   // offsets of a block's columns in C
 #pragma unroll
         for (uint32_t i = 0; i < kW / 2u; i++) coff[i] = pext_runs(i, g.cn, g.n_cn);
-        const uint32_t own = pext_runs(32u * q + lane, g.cm, g.n_cm);
-        BsCursor cur;
-        cur.c = tile_coord_bs(t0, ga);
         for (uint64_t t = t0; t < t1; t++, j++, cur.next(ga)) {
             const TileCoord &tc = cur.c;
-            const uint32_t buf = j % NA;
-            float2 *Crow = ga.arenas + (uint64_t)tc.il * ga.a.arena_elems + g.c_off + pext_runs(tc.beta, g.cb, g.n_cb) +
-                           pext_runs(tc.mt * kRows, g.cm, g.n_cm) + own;
+            const RunSlot<NA> last(j, runs - 1u, runs);
+            const uint32_t buf = kRuns ? last.buf : j % NA;
+            float2 *Crow = row_of(tc);   // while the MMAs run
             Unscale un{1.f, 1.f, false};
-            if (kParts == 2)
-                un = unscale_of(side_max<kLeaf>(ga, true, tc.il), side_max<kLeaf>(ga, false, tc.il), ga.n_chunks);
+            if (kParts == 2) un = unscale_of(side_max<kLeaf>(ga, true, tc.il), side_max<kLeaf>(ga, false, tc.il));
             uint32_t largest = 0;
-            if (!warp_wait_or_fail(smem_u32(&accf_bar[buf]), (j / NA) & 1u, &fail)) {
-                fail = 1;
-                break;
+            if constexpr (kRuns) {
+                for (uint32_t r = 1; r + 1u < runs && ok; r++) {
+                    ok = warp_wait_or_fail(smem_u32(&accf_bar[buf]), RunSlot<NA>(j, r, runs).uses & 1u, &fail);
+                    if (!ok) break;
+                    tc_fence_after();
+                    for (uint32_t j0 = share * kSum; j0 < (uint32_t)NT; j0 += 2u * kSum)
+                        tmem_add<kSum>(lanes + (buf - 1u) * kCols + j0, lanes + buf * kCols + j0);
+                    tc_fence_before();
+                    warp_arrive(smem_u32(&acce_bar[buf]));
+                }
             }
+            if (ok) ok = warp_wait_or_fail(smem_u32(&accf_bar[buf]), (kRuns ? last.uses : j / NA) & 1u, &fail);
+            if (!ok) break;
             tc_fence_after();
-            const uint32_t taddr = tmem + ((q * 32u) << 16) + buf * kCols;
+            const uint32_t taddr = lanes + buf * kCols;
             for (uint32_t j0 = share * kW; j0 < (uint32_t)NT; j0 += 2u * kW) {
                 float2 *Cblk = Crow + pext_runs(tc.nt * kNc + j0 / 2u, g.cn, g.n_cn);
                 uint32_t r[kW];
                 tmem_ld_pairs<kW>(taddr + j0, r);
+                if constexpr (kRuns) add_columns<kW>(r, taddr - kCols + j0);
 #pragma unroll
                 for (uint32_t i = 0; i < kW / 2u; i++) {
                     const float2 c = kParts == 2 ? unscaled(un, r[2u * i], r[2u * i + 1u])
@@ -1138,8 +1264,10 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
             }
             tc_fence_before();
             warp_arrive(smem_u32(&acce_bar[buf]));
+            if (kRuns) warp_arrive(smem_u32(&acce_bar[buf - 1u]));
             if (ga.max_c) note_max_warp(ga.max_c + tc.il, largest);
         }
+        if (!ok) fail = 1;
     }
     tc_fence_before();
     __syncthreads();
@@ -1156,7 +1284,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_bs_kernel(Gemm
 // its 512 tensor-memory columns, so that no allocation ever waits for another CTA's
 // columns), queried once per device and kernel (under a lock: host threads may launch on
 // several streams at once).
-template <int NT, int kParts, bool kBs, bool kLeaf>
+template <int NT, int kParts, bool kBs, bool kLeaf, bool kRuns>
 static cudaError_t gemm_grid(uint64_t n_tiles, uint64_t *grid) {
     static int per_sm[64] = {0}, sms[64] = {0};
     static std::mutex mu;
@@ -1166,10 +1294,10 @@ static cudaError_t gemm_grid(uint64_t n_tiles, uint64_t *grid) {
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (!per_sm[dev]) {
-        const void *fn = kBs ? reinterpret_cast<const void *>(gemm_tc_bs_kernel<NT, kParts, kLeaf>)
-                             : reinterpret_cast<const void *>(gemm_tc_kernel<NT, kParts, kLeaf>);
+        const void *fn = kBs ? reinterpret_cast<const void *>(gemm_tc_bs_kernel<NT, kParts, kLeaf, kRuns>)
+                             : reinterpret_cast<const void *>(gemm_tc_kernel<NT, kParts, kLeaf, kRuns>);
         const size_t smem = kBs ? (size_t)kBsBytes : smem_bytes<NT, kParts>(1024);
-        const int threads = kBs ? (int)block_threads<NT>() : (int)(int)block_threads<NT>();
+        const int threads = (int)block_threads<NT>();
         if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
             return e;
         cudaFuncAttributes fa;
@@ -1179,7 +1307,7 @@ static cudaError_t gemm_grid(uint64_t n_tiles, uint64_t *grid) {
         int n = 0;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const int cols = kBs ? (int)(bs_accs<NT>() * bs_cols<NT>()) : 2 * (NT < 32 ? 32 : NT);
+        const int cols = (int)((kBs || kRuns ? bs_accs<NT>() : 2u) * acc_cols<NT>());
         per_sm[dev] = n < 1 ? -1 : std::min(n, 512 / cols);
     }
     if (per_sm[dev] < 1) return cudaErrorInvalidConfiguration;
@@ -1187,7 +1315,7 @@ static cudaError_t gemm_grid(uint64_t n_tiles, uint64_t *grid) {
     return cudaSuccess;
 }
 
-template <int NT, int kParts, bool kLeaf>
+template <int NT, int kParts, bool kLeaf, bool kRuns>
 static cudaError_t launch_gemm_nt(GemmArgs ga, cudaStream_t s) {
     ga.n_tiles = ((uint64_t)ga.n_items << ga.g.nb) * ga.n_mt * ga.n_nt;
     if (ga.n_tiles == 0) return cudaErrorInvalidConfiguration;
@@ -1198,7 +1326,7 @@ static cudaError_t launch_gemm_nt(GemmArgs ga, cudaStream_t s) {
     // tile's MMAs, cost more than the reuse saved; tile coordinates above the row tiles within
     // 32 bits)
     if (ga.n_chunks <= bs_chunks<NT, kParts>() && ga.n_mt >= 4u && (uint64_t)ga.n_items * ga.n_nt < (1ull << 32)) {
-        if ((e = gemm_grid<NT, kParts, true, kLeaf>(ga.n_tiles, &grid)) != cudaSuccess) return e;
+        if ((e = gemm_grid<NT, kParts, true, kLeaf, kRuns>(ga.n_tiles, &grid)) != cudaSuccess) return e;
         ga.stages = bs_stages<NT, kParts>(ga.n_chunks);
         // Shared memory asked for leaves the rest of the SM's 256 KB as L1 cache. At 256 columns
         // and up to 32 summed entries the step is bound by C's stores, and the smallest cache
@@ -1208,26 +1336,42 @@ static cudaError_t launch_gemm_nt(GemmArgs ga, cudaStream_t s) {
         // stages from 64 summed entries (s118 of 5001 1.88 ms, 2.02 with five stages).
         size_t bytes = kBsBytes;
         if (NT < 256 || ga.n_chunks > 2u) {
-            if (NT >= 256) ga.stages = 3u;
+            if (NT >= 256) ga.stages = kParts == 2 ? 4u : 3u;
             bytes = ga.stages * a_bytes<kParts>() + ga.n_chunks * (bs_b_bytes<NT, kParts>() + 12u * kKq);
         }
-        gemm_tc_bs_kernel<NT, kParts, kLeaf><<<(unsigned)grid, block_threads<NT>(), bytes, s>>>(ga);
+        gemm_tc_bs_kernel<NT, kParts, kLeaf, kRuns><<<(unsigned)grid, block_threads<NT>(), bytes, s>>>(ga);
         return cudaGetLastError();
     }
     // dynamic shared memory: the operand stage ring and the summed index tables, sized for the largest summed index (1024 entries)
-    if ((e = gemm_grid<NT, kParts, false, kLeaf>(ga.n_tiles, &grid)) != cudaSuccess) return e;
-    gemm_tc_kernel<NT, kParts, kLeaf><<<(unsigned)grid, (int)block_threads<NT>(), smem_bytes<NT, kParts>(1024), s>>>(ga);
+    if ((e = gemm_grid<NT, kParts, false, kLeaf, kRuns>(ga.n_tiles, &grid)) != cudaSuccess) return e;
+    gemm_tc_kernel<NT, kParts, kLeaf, kRuns><<<(unsigned)grid, (int)block_threads<NT>(), smem_bytes<NT, kParts>(1024), s>>>(ga);
     return cudaGetLastError();
 }
 
 template <int kParts, bool kLeaf>
 static cudaError_t launch_gemm_split(const GemmArgs &ga, uint32_t nt_cols, cudaStream_t s) {
+    if constexpr (kParts == 2) {
+        // Four chunks are one group where the ring has four stages (B-stationary form). Runs of two
+        // chunks for the others of four, of four chunks for longer sums, where two cost 8 to 20 % more
+        // (512 summed entries: 2.18 and 2.01 ms; 2.04 in one accumulator) for half the truncations.
+        static_assert(bs_chunks<256, 2>() >= 4u && bs_stages<256, 2>(4u) >= 4u && bs_stages<128, 2>(4u) >= 4u, "a group of four");
+        const bool bs = ga.n_mt >= 4u && (uint64_t)ga.n_items * ga.n_nt < (1ull << 32);
+        GemmArgs gr = ga;
+        gr.run_bits = ga.n_chunks >= 8u ? 2u : 1u;
+        if (ga.n_chunks >= (bs ? 8u : 4u)) switch (nt_cols) {
+            case 16: return launch_gemm_nt<16, kParts, kLeaf, true>(gr, s);
+            case 32: return launch_gemm_nt<32, kParts, kLeaf, true>(gr, s);
+            case 64: return launch_gemm_nt<64, kParts, kLeaf, true>(gr, s);
+            case 128: return launch_gemm_nt<128, kParts, kLeaf, true>(gr, s);
+            default: return launch_gemm_nt<256, kParts, kLeaf, true>(gr, s);
+        }
+    }
     switch (nt_cols) {
-        case 16: return launch_gemm_nt<16, kParts, kLeaf>(ga, s);
-        case 32: return launch_gemm_nt<32, kParts, kLeaf>(ga, s);
-        case 64: return launch_gemm_nt<64, kParts, kLeaf>(ga, s);
-        case 128: return launch_gemm_nt<128, kParts, kLeaf>(ga, s);
-        default: return launch_gemm_nt<256, kParts, kLeaf>(ga, s);
+        case 16: return launch_gemm_nt<16, kParts, kLeaf, false>(ga, s);
+        case 32: return launch_gemm_nt<32, kParts, kLeaf, false>(ga, s);
+        case 64: return launch_gemm_nt<64, kParts, kLeaf, false>(ga, s);
+        case 128: return launch_gemm_nt<128, kParts, kLeaf, false>(ga, s);
+        default: return launch_gemm_nt<256, kParts, kLeaf, false>(ga, s);
     }
 }
 

@@ -24,7 +24,6 @@ namespace qvx {
 namespace {
 
 constexpr uint32_t kNt = 256u;                    // real columns of a tile (128 complex)
-constexpr uint32_t kCols = kNt / 2u;
 constexpr uint32_t kRBThreads = 128u;             // B producers: two units each
 constexpr uint32_t kRMmaWarp = (256u + kRBThreads) / 32u;
 constexpr uint32_t kREpiWarp = kRMmaWarp + 4u;
@@ -204,6 +203,7 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_tc_reduce_kernel(ReduceArgs
         regs_dec<kRRegsIssue>();
         if (warp == kRMmaWarp && lane == 0) {
             constexpr uint32_t idesc = mma_idesc<2>(kNt);
+            const uint32_t group = min(group_chunks<2>(), ra.n_chunks);
             RingPos ring;
             uint32_t j = 0, gi = 0;
             bool ok = true;
@@ -223,17 +223,15 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_tc_reduce_kernel(ReduceArgs
                     const uint32_t d = tmem + buf * kNt;
                     // jo = jb * n_jm + jm: the B of this tile's jb
                     const uint32_t b0 = ((t & (n_jb * n_jm - 1u)) >> (r.jo - r.jb)) * ra.n_chunks;
-                    for (uint32_t c = 0; c < ra.n_chunks; c++, ring.next(S)) {
-                        const uint32_t s = ring.s;
-                        if (!wait_or_fail(smem_u32(&full_bar[s]), ring.phase, &fail)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint32_t sa = sbase + s * kRStage, sb = smem_u32(sB) + (b0 + c) * kRChunkB;
-                        const uint32_t bs[2][2] = {{sb, sb + kRegionB}, {sb + 2u * kRegionB, sb + 3u * kRegionB}};
-                        mma_chunk<2>(d, sa, kRegionA, bs, idesc, c == 0u);
-                        mma_commit(smem_u32(&empty_bar[s]));
+                    for (uint32_t c = 0; c < ra.n_chunks && ok; c += group) {
+                        auto b_at = [&](uint32_t i, uint32_t, uint32_t (&bs)[2][2]) {
+                            const uint32_t sb = smem_u32(sB) + (b0 + c + i) * kRChunkB;
+                            bs[0][0] = sb;
+                            bs[0][1] = sb + kRegionB;
+                            bs[1][0] = sb + 2u * kRegionB;
+                            bs[1][1] = sb + 3u * kRegionB;
+                        };
+                        ok = mma_group<2>(d, group, c == 0u, ring, S, sbase, kRStage, kRegionA, full_bar, empty_bar, b_at, idesc, &fail);
                     }
                     if (ok) mma_commit(smem_u32(&accf_bar[buf]));
                 }
@@ -333,7 +331,7 @@ __global__ void __launch_bounds__(kRThreads, 1) gemm_tc_reduce_kernel(ReduceArgs
                 }
                 if (!ok) break;
                 const Unscale un = unscale_of(operand_max(ra.sc.max_a, ra.sc.leaf_max_a, il),
-                                              operand_max(ra.sc.max_b, ra.sc.leaf_max_b, il), ra.n_chunks);
+                                              operand_max(ra.sc.max_b, ra.sc.leaf_max_b, il));
                 float2 *emo = ebase + mv(mo, r.mo_e);
 #pragma unroll
                 for (uint32_t b = 0; b < 4u; b++)
