@@ -121,9 +121,11 @@ typedef struct {
                                   summed entries, 128 output entries of one operand's own and 8 of
                                   the other's, 5 or more flops per algorithmic byte) as complex
                                   GEMMs on the tcgen05 tensor cores, each FP32 operand split into
-                                  two scaled fp16 parts (three products) or, for circuits whose
-                                  gate entries differ much in size, three bf16 parts (six
-                                  products), about 2^-22 relative error per product. They are added
+                                  two scaled fp16 parts (three products; entries below 2^-16 of
+                                  their tensor's largest have fewer bits, to 2^-40 of it) or, for
+                                  circuits with a gate whose nonzero entries are not of one
+                                  magnitude and for gradient plans with angles, three bf16 parts
+                                  (six products), about 2^-22 relative error per product. They are added
                                   in the tensor cores' FP32 accumulators, which truncate: at most 64
                                   summed entries in a row with fp16 parts (a sum comes out up to
                                   2^-21 too small in the mean; longer ones are added in FP32), all of

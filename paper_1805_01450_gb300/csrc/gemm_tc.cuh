@@ -15,7 +15,7 @@
 //     writes it (note_max).
 //   kParts = 3: x = h + m + l in bf16 (8 bits each), the six products h*h + h*m + m*h + h*l +
 //     l*h + m*m; the dropped terms are below 2^-23 of the product. It has FP32's range and
-//     serves circuits whose gate entries differ too much in size (Plan::fp16_split).
+//     serves circuits with gates whose own entries differ in size (Plan::fp16_split).
 // What limits the accuracy is not the split but the accumulation (group_chunks says how that is
 // kept short). Three products instead of six also halve the MMAs and take a third off the operand
 // parts stored in and read from shared memory, which bounds the loop. Two bf16 parts with three

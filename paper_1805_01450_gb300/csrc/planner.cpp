@@ -2107,21 +2107,31 @@ qvx_status make_plan(const qvx_circuit *c, const int32_t *order, int32_t n_order
 
 namespace {
 
-// Whether the entries of every gate are zero or of magnitude 2^-4 ... 2: the tensors' entries
-// then stay within the range that two fp16 parts hold after scaling (gates with very unequal
-// entries, U1 matrices or rotations by tiny angles, would lose the small ones).
-bool gates_alike(const qvx_circuit *c) {
+// Whether every gate's entries are zero or of one magnitude (2^-4 ... 2). Then all terms of the
+// sums that a tensor's entries are have the same magnitude, and an entry is far below the
+// tensor's largest only where terms cancel. Two fp16 parts suit such tensors: with the largest
+// entry scaled to 2^15 they hold entries to 2^-40 of it. A gate of unequal entries (a U1 matrix,
+// a rotation) multiplies its ratio into a tensor's range, gate by gate without a bound, and so do
+// angles that a gradient call may still change: such circuits keep three bf16 parts, which have
+// FP32's range.
+bool gates_alike(const qvx_circuit *c, bool angles_change) {
     if (!c || c->n_gates < 0 || (c->n_gates > 0 && !c->gates)) return false;
     for (int64_t i = 0; i < c->n_gates; i++) {
         cplx m[2][2];
-        if (c->gates[i].kind == QVX_GATE_CZ) continue;
-        if (c->gates[i].kind == QVX_GATE_T) continue;
-        if (!gate_matrix(c->gates[i], m)) return false;
+        const qvx_gate &g = c->gates[i];
+        if (g.kind == QVX_GATE_CZ || g.kind == QVX_GATE_T) continue;
+        if (angles_change && g.kind == QVX_GATE_RXY && g.param_index >= 0) return false;
+        if (!gate_matrix(g, m)) return false;
+        double least = 0, most = 0;
         for (int r = 0; r < 2; r++)
             for (int k = 0; k < 2; k++) {
                 const double v = std::abs(m[r][k]);
-                if (!(v < 1e-16 || (v >= 1.0 / 16.0 && v <= 2.0))) return false;
+                if (!(v <= 2.0)) return false;   // (or not a number)
+                if (v == 0.0) continue;
+                least = most == 0.0 ? v : std::min(least, v);
+                most = std::max(most, v);
             }
+        if (most > 0.0 && (least < 1.0 / 16.0 || least < most * (1.0 - 1e-6))) return false;
     }
     return true;
 }
@@ -2130,7 +2140,7 @@ qvx_status plan_once(const qvx_circuit *c, const int32_t *order, int32_t n_order
                      const int32_t *slices, int32_t n_slices, const qvx_plan_opts &opts,
                      Plan *p, std::string *err) {
     p->opts = opts;
-    p->fp16_split = gates_alike(c);
+    p->fp16_split = gates_alike(c, opts.gradient != 0);
     if (!build_model(c, &p->model, err, opts.gradient != 0)) return QVX_EINVAL;
     if (opts.n_open_qubits < 0 || opts.n_open_qubits > 16) { *err = "opts: n_open_qubits must be in [0, 16]"; return QVX_EINVAL; }
     if (opts.n_open_qubits > 0 && opts.gradient) { *err = "open qubits are not supported with gradients"; return QVX_EUNSUPPORTED; }
