@@ -180,7 +180,8 @@ struct DevProgram {
     uint32_t magic;
     uint32_t n_steps, n_leaves, pad0;
     uint64_t n_leaf_entries;       // complex64 entries of all stored leaves
-    uint64_t arena_elems;          // complex64 entries of one work item's arena
+    uint64_t arena_elems;          // complex64 entries of all the steps' results; a launch's arena may end
+                                   // below those that merged steps do not store (LaunchArgs)
     uint64_t final_off;            // arena offset of the final tensor (over the inner slice modes)
     uint32_t n_inner;              // inner (open) sliced variables
     uint32_t final_present;        // inner bits that are modes of the final tensor, low to high

@@ -85,7 +85,8 @@ struct Plan {
     std::vector<PStep> steps;
     std::vector<std::pair<int, int>> phases;    // [first, last) step ranges of independent steps
     int final_tensor = -1;
-    int64_t arena_elems = 0;
+    int64_t arena_elems = 0;                   // of a work item's arena
+    int64_t program_elems = 0;                 // with the results that merged steps do not store (allocate_arena)
     int max_rank = 0;
     double flops_per_item = 0, bytes_per_item = 0;
     cplx prog_scalar = 1.0;                     // model scalar times the program's own factors
