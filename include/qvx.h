@@ -155,7 +155,8 @@ typedef struct {
     int32_t n_tiled_steps;           /* contractions with a register-tiled form (global-arena engines) */
     int32_t n_phases;                /* levels of mutually independent contractions */
     int32_t n_open_qubits;           /* amplitudes per bitstring = 2^n_open_qubits */
-    int32_t n_gemm_steps;            /* contractions run on the tensor cores (opts.tensor_cores) */
+    int32_t n_gemm_steps;            /* contractions run on the tensor cores (opts.tensor_cores), those
+                                        of merged steps among them */
     int32_t grad_smem_bytes;         /* shared memory per work item of the gradient kernel's on-chip
                                         form (0: absent; larger than the device allows: global memory) */
     int32_t grad_recomputed;         /* gradient plans: forward contractions recomputed in the

@@ -476,7 +476,12 @@ qvx_status qvx_plan_get_info(const qvx_plan *plan, qvx_plan_info *info) {
     info->n_phases = (int32_t)p.phases.size();
     info->n_open_qubits = (int32_t)p.open_qubits.size();
     info->n_gemm_steps = 0;
-    for (const qvx::GemmStep &g : p.gemm) info->n_gemm_steps += g.nk > 0 ? 1 : 0;
+    for (size_t s = 0; s < p.gemm.size(); s++) {   // as launched: both steps of a pair, the reduced one of a merged step
+        const bool pair = !p.pairs.empty() && (p.pairs[s].consumer >= 0 || p.pairs[s].absorbed);
+        const bool merged = !p.reduces.empty() && p.reduces[s].merged;
+        const bool reduces = !p.reduces.empty() && p.reduces[s].producer >= 0;
+        info->n_gemm_steps += pair || merged || (p.gemm[s].nk > 0 && !reduces) ? 1 : 0;
+    }
     info->grad_recomputed = p.grad_recomputed;
     info->est_bytes_per_amplitude = qvx::plan_estimate(p);
     info->grad_smem_bytes = p.opts.gradient
