@@ -353,9 +353,12 @@ class Plan:
             if validate:
                 self._check_host_bits(bitstrings)
             if bitstrings and stream.value == (_current_stream() or None):
-                # pageable words are staged by the driver before the call returns: no need to
-                # wait for the stream as well
-                words = torch.tensor(bitstring_words(bitstrings, self.words), dtype=torch.int64)
+                # from page-locked memory without waiting for the stream: torch gives the block to
+                # nobody else before the copy is through. A capture would record the copy and read
+                # the block again at every replay
+                if torch.cuda.is_current_stream_capturing():
+                    raise QvxError(QVX_ECUDA, "bitstrings cannot be uploaded during stream capture")
+                words = torch.tensor(bitstring_words(bitstrings, self.words), dtype=torch.int64, pin_memory=True)
                 return words.to("cuda", non_blocking=True), -1
             return self._bits(bitstrings), -1
         bits = self._bits(bitstrings)
