@@ -793,7 +793,14 @@ int64_t take_ticket(int device, BitsTicket *out, cudaError_t *e) {
         if (g_tickets[i].device == device) { at = i; break; }
         if (g_tickets[i].device < 0) at = i;
     }
-    if (at == g_tickets.size()) g_tickets.push_back(BitsTicket{});
+    if (at == g_tickets.size()) {
+        try {
+            g_tickets.push_back(BitsTicket{});
+        } catch (const std::bad_alloc &) {   // no exception leaves the C interface
+            *e = cudaErrorMemoryAllocation;
+            return -1;
+        }
+    }
     BitsTicket &t = g_tickets[at];
     if (t.device != device) {
         t = BitsTicket{};
