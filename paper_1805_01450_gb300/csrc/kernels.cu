@@ -958,14 +958,12 @@ __global__ void __launch_bounds__(256, 3) persistent_program_kernel(LaunchArgs a
 // by load latency and instructions, at 45 % of the issue slots. What was taken from that, on the
 // 1,024 amplitudes of a 7 x 7 grid at depth 30 (9.93 ms at first, 8.46 now):
 //  - the item, its leaves and the tile index's high bits are found once per CTA, and a CTA walks
-//    up to 8 blocks of tiles: 9.2 ms (with one block per CTA 10.4);
+//    up to 8 blocks of tiles where that pays (tile_form);
 //  - 4 x 4 tiles of a small and a large operand address these by a block-uniform base and a
 //    32-bit offset per thread, which leaves registers for loads: a 32-entry sum goes from 1.80
-//    to 1.56 ms. Smaller tiles lose 10 % by it and keep their own pointers;
-//  - in that form, with 64 registers, the compiler loads a tile's B entries together and its A
-//    entries one by one, so B has to be the operand that comes from DRAM: they are swapped where
-//    A is the larger (a 16-entry sum over a 2^25-entry A: 1.85 to 0.94 ms). At 72 and 80
-//    registers it does so for none (2.28 ms for 1.56);
+//    to 1.56 ms. Smaller tiles lose 10 % by it and keep their own pointers. With 64 registers the
+//    compiler loads a tile's B entries together and its A entries one by one, so B has to be the
+//    larger operand; at 72 and 80 registers it does so for none (2.28 ms for 1.56);
 //  - 8 x 4 tiles from 4 flops per byte up (RegTileStep's rule): 8.73 to 8.58 ms.
 constexpr uint32_t kMaxTileBlocks = 8;          // blocks of tiles per CTA (16: 3 % slower)
 constexpr uint64_t kMinTileCtas = 2048;         // while this many CTAs remain (3.4 waves of 4 per SM)
@@ -997,9 +995,8 @@ __device__ __forceinline__ float2 at_bytes(const float2 *base, uint32_t bytes) {
 enum TileForm {
     kTilesFlat,      // one tile per thread, any item and tile per thread
     kTilesBlocks,    // several blocks of tiles of one item
-    kTilesBase,      // the same; block-uniform bases and a 32-bit offset per thread
-    kTilesSwapped    // the same; A and B are the step's second and first operand. A product's
-};                   // two terms are added in the step's own order, so the bits are the same
+    kTilesBase       // the same; block-uniform bases and a 32-bit offset per thread
+};
 // kMax: the output's largest entries are wanted (max_c).
 template <int RM, int RN, bool kMax, TileForm kForm>
 __global__ void __launch_bounds__(RegTileShape<RM, RN>::kThreads, RegTileShape<RM, RN>::kMinBlocks)
@@ -1007,7 +1004,7 @@ __global__ void __launch_bounds__(RegTileShape<RM, RN>::kThreads, RegTileShape<R
                         uint32_t *max_c, uint32_t per_cta) {
     constexpr int TM = 1 << RM, TN = 1 << RN;
     constexpr int kThreadBits = RegTileShape<RM, RN>::kThreadBits;
-    constexpr bool kWhole = kForm != kTilesFlat, kUniform = kForm == kTilesBase || kForm == kTilesSwapped;
+    constexpr bool kWhole = kForm != kTilesFlat, kUniform = kForm == kTilesBase;
     int64_t il;
     uint32_t blk = 0;              // kWhole: first block of tiles of this CTA
     TileOffsets own;
@@ -1068,9 +1065,7 @@ __global__ void __launch_bounds__(RegTileShape<RM, RN>::kThreads, RegTileShape<R
 #pragma unroll
             for (int i = 0; i < TM; i++)
 #pragma unroll
-                for (int j = 0; j < TN; j++)
-                    if constexpr (kForm == kTilesSwapped) cmac(acc[i][j], bv[j], av[i]);
-                    else cmac(acc[i][j], av[i], bv[j]);
+                for (int j = 0; j < TN; j++) cmac(acc[i][j], av[i], bv[j]);
         };
         if (kWhole && nk == nab) {   // every summed mode in both operands
 #pragma unroll kUnroll
@@ -1772,41 +1767,45 @@ cudaError_t launch_splitk_step(const LaunchArgs &a, uint32_t step, int64_t item_
     return counted(cudaGetLastError());
 }
 
-// Form of a launch over `blocks` blocks of tiles; *per_cta blocks of one item go to a CTA. With
-// too few blocks for two per CTA and up to four summed entries the flat form is the faster one by
-// up to 15 % (242 items of a 6 x 7 grid at depth 26: 36.6 us a step against 41.1): it has no second
-// index to work out; from eight summed entries on it is the slower one (128 of them: 141 us against
-// 110). The base forms pay where one operand is far smaller than the other (2^7 times: 1.21 x
-// faster) and lose where both come from L2 (4 times: 1.26 x slower, the same size and 128 summed
-// entries: 2 x).
+// Form of a launch over `blocks` blocks of tiles; *per_cta blocks of one item go to a CTA. max: the
+// output's largest entries are wanted. Timed on 260 steps of 6 x 6 to 8 x 8 circuits (2^8 to 2^24
+// tiles an item, 0 to 8 summed modes), the other form against the one taken:
+//  - with too few blocks for two per CTA: 1.15 x slower up to four summed entries (242 items of a
+//    6 x 7 grid at depth 26: 36.6 us a step against 41.1), flat from eight on 1.28 x slower;
+//  - 4 x 4 tiles: with a second operand 2^6 times larger than the first, flat 1.1 to 1.9 x slower
+//    than a block-uniform base, plain pointers 1.1 to 1.2 x; with a larger first operand flat is
+//    the faster one by up to 8 %, otherwise blocks are by up to 16 %;
+//  - 8 x 4 tiles: flat is 2 to 7 % faster while an operand stays in L2, blocks 16 % with both from
+//    memory (2^20 and 2^23 entries, 14 items);
+//  - smaller tiles: from eight summed entries on flat is faster by up to 20 % (more CTAs per SM fit its
+//    registers, and the operand read only once comes in order); with four, where the operands
+//    outweigh the result or a thread holds eight entries, by 2 to 18 %; with one or two it is 3 to 24 %
+//    slower, except a thread's eight entries out of an operand as large as the result (2 to 11 % faster).
+//    Blocks merge the largest entry of eight blocks at once, which turns the last two cases for
+//    2 x 4 tiles (1.06 and 1.13 x slower).
 template <int RM, int RN>
-static TileForm tile_form(const RegTileStep &rs, uint64_t blocks, uint32_t *per_cta) {
+static TileForm tile_form(const RegTileStep &rs, uint64_t blocks, bool max, uint32_t *per_cta) {
     *per_cta = 1u;
     // 8 x 8 tiles are bound by their multiply-adds and registers: 38.4 ms flat, 43.5 in blocks (a step
     // of 28 flops per byte, circuit 5001 of the 8 x 8 grid without tensor cores). (The 32-bit byte
     // offsets of a thread hold operands and results of up to 2^29 entries.)
-    const int rank_a = rs.a_cb + rs.nk_ab + rs.nk_a, rank_b = rs.b_cb + rs.nk_ab + rs.nk_b;
-    if (RM + RN == 6 || rs.nt < RegTileShape<RM, RN>::kThreadBits || std::max({rank_a, rank_b, (int)rs.rc}) > 29) return kTilesFlat;
+    const int nk = rs.nk_ab + rs.nk_a + rs.nk_b;
+    const int rank_a = rs.a_cb + rs.nk_ab + rs.nk_a, rank_b = rs.b_cb + rs.nk_ab + rs.nk_b, larger = std::max(rank_a, rank_b);
+    if (RM + RN == 6 || rs.nt < RegTileShape<RM, RN>::kThreadBits || std::max(larger, (int)rs.rc) > 29) return kTilesFlat;
     const uint32_t most = std::min(kMaxTileBlocks, 1u << (rs.nt - RegTileShape<RM, RN>::kThreadBits));
-    while (*per_cta < most && blocks / (2u * *per_cta) >= kMinTileCtas) *per_cta *= 2u;
-    if (*per_cta == 1u) return rs.nk_ab + rs.nk_a + rs.nk_b < 3 ? kTilesFlat : kTilesBlocks;
-    if (RM != 2 || RN != 2 || std::abs(rank_a - rank_b) < 6) return kTilesBlocks;
-    if (rank_a < rank_b) return kTilesBase;
-    return rs.nk_a + rs.nk_b == 0 ? kTilesSwapped : kTilesBlocks;   // (modes of one operand: A's before B's)
-}
-
-static RegTileStep swapped(const RegTileStep &rs) {
-    RegTileStep r = rs;
-    std::swap(r.a_off, r.b_off);
-    std::swap(r.a_cb, r.b_cb);
-    std::swap(r.na_runs, r.nb_runs);
-    std::swap(r.runs_a, r.runs_b);
-    std::swap(r.a_m, r.b_n);
-    std::swap(r.c_m, r.c_n);
-    r.flags = rs.flags & ~(kStepALeaf | kStepBLeaf);
-    if (rs.flags & kStepALeaf) r.flags |= kStepBLeaf;
-    if (rs.flags & kStepBLeaf) r.flags |= kStepALeaf;
-    return r;
+    uint32_t n = 1u;
+    while (n < most && blocks / (2u * n) >= kMinTileCtas) n *= 2u;
+    if (n == 1u) return nk < 3 ? kTilesFlat : kTilesBlocks;
+    const bool merges = max && RM == 1 && RN == 2;
+    bool flat;
+    if (RM == 2 && RN == 2) flat = rank_a - rank_b >= 6;
+    else if (RM + RN == 5) flat = std::min(rank_a, rank_b) < 18;
+    else if (nk >= 3) flat = true;
+    else if (nk == 2) flat = (RM + RN == 3 && !merges) || rs.rc < larger;
+    else flat = nk == 1 && RM + RN == 3 && rs.rc <= larger && !merges;
+    if (flat) return kTilesFlat;
+    *per_cta = n;
+    return RM == 2 && RN == 2 && rank_b - rank_a >= 6 ? kTilesBase : kTilesBlocks;
 }
 
 template <int RM, int RN, TileForm kForm>
@@ -1826,12 +1825,10 @@ static void launch_regtile_t(const LaunchArgs &a, const RegTileStep &rs, int64_t
     constexpr int kThreads = RegTileShape<RM, RN>::kThreads;
     const uint64_t blocks = (((uint64_t)n_items << rs.nt) + kThreads - 1) / kThreads;
     uint32_t per_cta;
-    const TileForm form = tile_form<RM, RN>(rs, blocks, &per_cta);
+    const TileForm form = tile_form<RM, RN>(rs, blocks, max_c != nullptr, &per_cta);
     if constexpr (RM == 2 && RN == 2) {
         if (form == kTilesBase)
             return launch_regtile_f<RM, RN, kTilesBase>(a, rs, item_begin, n_items, arenas, max_c, blocks, per_cta, s);
-        if (form == kTilesSwapped)
-            return launch_regtile_f<RM, RN, kTilesSwapped>(a, swapped(rs), item_begin, n_items, arenas, max_c, blocks, per_cta, s);
     }
     if constexpr (RM + RN < 6) {
         if (form == kTilesBlocks)
