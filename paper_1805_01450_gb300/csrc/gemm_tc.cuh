@@ -118,17 +118,18 @@ __host__ __device__ constexpr uint32_t acc_cols() { return NT < 32 ? 32u : (uint
 // (tensor memory holds 512 columns: 2 x 256, 4 x 128, 8 x 64, 8 x 32).
 template <int NT>
 __host__ __device__ constexpr uint32_t bs_accs() { return 512u / acc_cols<NT>() < 8u ? 512u / acc_cols<NT>() : 8u; }
-// Operand stages of the shared-memory ring. With five (all that fit at 256 columns) the steps
-// ran 7 to 17 % slower, with two 6 to 8 %: shared memory that the ring does not take is L1 cache
-// for the columns.
-template <int NT, int kParts>
-__host__ __device__ constexpr uint32_t n_stages() { return 3u; }
+// Operand stages of the shared-memory ring: three, or four for a group of four chunks. With five
+// (all that fit at 256 columns) the steps ran 7 to 17 % slower, with two 6 to 8 %: shared memory
+// that the ring does not take is L1 cache for the columns.
+constexpr uint32_t kStages = 4u;
+template <int kParts>
+__host__ __device__ constexpr uint32_t n_stages(uint32_t n_chunks) { return kParts == 2 && n_chunks == 4u ? 4u : 3u; }
 // complex columns an epilogue warp reads at a time (the same number of Re and Im columns)
 template <int NT>
 __host__ __device__ constexpr uint32_t epi_cols() { return NT >= 64 ? 16u : 8u; }
 template <int NT, int kParts>
-__host__ __device__ constexpr size_t smem_bytes(uint32_t K) {   // three offset tables (A, B, the leaf)
-    return (size_t)n_stages<NT, kParts>() * stage_bytes<NT, kParts>() + 12u * (size_t)K;
+__host__ __device__ constexpr size_t smem_bytes(uint32_t stages, uint32_t K) {   // three offset tables (A, B, the leaf)
+    return (size_t)stages * stage_bytes<NT, kParts>() + 12u * (size_t)K;
 }
 
 __device__ __forceinline__ uint32_t core_offset(uint32_t r, uint32_t g) {
@@ -716,13 +717,13 @@ struct BsCursor {
 template <int NT, int kParts, bool kLeaf, bool kRuns>
 __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArgs ga) {
     constexpr uint32_t kMmaWarp = mma_warp<NT>(), kEpiWarp = epi_warp<NT>();
-    constexpr uint32_t S = n_stages<NT, kParts>();
+    const uint32_t S = n_stages<kParts>(ga.n_chunks);
     constexpr uint32_t kCols = acc_cols<NT>(), NA = kRuns ? bs_accs<NT>() : 2u;   // accumulators
     constexpr uint32_t kRegA = region_bytes(kRows), kStage = stage_bytes<NT, kParts>();
     constexpr uint32_t kW = epi_cols<NT>();
     constexpr uint32_t kNc = (uint32_t)NT / 2u;   // complex columns per tile
     extern __shared__ __align__(1024) unsigned char gsm[];
-    __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], accf_bar[NA], acce_bar[NA], drain_bar;
+    __shared__ __align__(8) uint64_t full_bar[kStages], empty_bar[kStages], accf_bar[NA], acce_bar[NA], drain_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int fail;
     const GemmStep &g = ga.g;
@@ -847,7 +848,7 @@ __global__ void __launch_bounds__(block_threads<NT>(), 1) gemm_tc_kernel(GemmArg
         if (warp == kMmaWarp && lane == 0) {   // MMA issuer
             constexpr uint32_t idesc = mma_idesc<kParts>(NT);
             constexpr uint32_t kBlkB = b_block_bytes(NT);
-            const uint32_t group = min(group_chunks<kParts>(), ga.n_chunks), runs = ga.n_chunks >> ga.run_bits;
+            const uint32_t group = min(kParts == 2 && !kRuns ? 4u : group_chunks<kParts>(), ga.n_chunks), runs = ga.n_chunks >> ga.run_bits;
             RingPos ring;
             uint32_t j = 0;
             bool ok = true;
@@ -1296,7 +1297,7 @@ static cudaError_t gemm_grid(uint64_t n_tiles, uint64_t *grid) {
     if (!per_sm[dev]) {
         const void *fn = kBs ? reinterpret_cast<const void *>(gemm_tc_bs_kernel<NT, kParts, kLeaf, kRuns>)
                              : reinterpret_cast<const void *>(gemm_tc_kernel<NT, kParts, kLeaf, kRuns>);
-        const size_t smem = kBs ? (size_t)kBsBytes : smem_bytes<NT, kParts>(1024);
+        const size_t smem = kBs ? (size_t)kBsBytes : smem_bytes<NT, kParts>(n_stages<kParts>(4u), 1024);
         const int threads = (int)block_threads<NT>();
         if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
             return e;
@@ -1342,23 +1343,23 @@ static cudaError_t launch_gemm_nt(GemmArgs ga, cudaStream_t s) {
         gemm_tc_bs_kernel<NT, kParts, kLeaf, kRuns><<<(unsigned)grid, block_threads<NT>(), bytes, s>>>(ga);
         return cudaGetLastError();
     }
-    // dynamic shared memory: the operand stage ring and the summed index tables, sized for the largest summed index (1024 entries)
+    // dynamic shared memory: the operand stage ring and the summed index tables, sized for the largest
+    // summed index (1024 entries)
     if ((e = gemm_grid<NT, kParts, false, kLeaf, kRuns>(ga.n_tiles, &grid)) != cudaSuccess) return e;
-    gemm_tc_kernel<NT, kParts, kLeaf, kRuns><<<(unsigned)grid, (int)block_threads<NT>(), smem_bytes<NT, kParts>(1024), s>>>(ga);
+    gemm_tc_kernel<NT, kParts, kLeaf, kRuns><<<(unsigned)grid, (int)block_threads<NT>(), smem_bytes<NT, kParts>(n_stages<kParts>(ga.n_chunks), 1024), s>>>(ga);
     return cudaGetLastError();
 }
 
 template <int kParts, bool kLeaf>
 static cudaError_t launch_gemm_split(const GemmArgs &ga, uint32_t nt_cols, cudaStream_t s) {
     if constexpr (kParts == 2) {
-        // Four chunks are one group where the ring has four stages (B-stationary form). Runs of two
-        // chunks for the others of four, of four chunks for longer sums, where two cost 8 to 20 % more
-        // (512 summed entries: 2.18 and 2.01 ms; 2.04 in one accumulator) for half the truncations.
-        static_assert(bs_chunks<256, 2>() >= 4u && bs_stages<256, 2>(4u) >= 4u && bs_stages<128, 2>(4u) >= 4u, "a group of four");
-        const bool bs = ga.n_mt >= 4u && (uint64_t)ga.n_items * ga.n_nt < (1ull << 32);
+        // Up to four chunks are one group. Longer sums take runs of two chunks up to 128 summed entries, of
+        // four beyond, where two cost 8 to 20 % more (512 entries: 2.18 and 2.01 ms; 2.04 in one
+        // accumulator) for half the truncations.
+        static_assert(bs_stages<256, 2>(4u) >= 4u && bs_stages<128, 2>(4u) >= 4u, "a group of four");
         GemmArgs gr = ga;
-        gr.run_bits = ga.n_chunks >= 8u ? 2u : 1u;
-        if (ga.n_chunks >= (bs ? 8u : 4u)) switch (nt_cols) {
+        gr.run_bits = ga.n_chunks > 8u ? 2u : 1u;
+        if (ga.n_chunks >= 8u) switch (nt_cols) {
             case 16: return launch_gemm_nt<16, kParts, kLeaf, true>(gr, s);
             case 32: return launch_gemm_nt<32, kParts, kLeaf, true>(gr, s);
             case 64: return launch_gemm_nt<64, kParts, kLeaf, true>(gr, s);

@@ -34,7 +34,7 @@ def launched(image, parts):
         nm, nn, nk = (int(g[f]) for f in ("nm", "nn", "nk"))
         nt, chunks = 256 if nn >= 7 else 2 << nn, max(1, (1 << nk) // 16)
         bs = (1 << nm) // 128 >= 4 and chunks <= RESIDENT[parts][nt]
-        how = "one" if parts == 3 or chunks <= 2 else "four" if chunks == 4 and (1 << nm) // 128 >= 4 else "runs"
+        how = "one" if parts == 3 or chunks <= 2 else "four" if chunks == 4 else "runs"
         out.add((kind, nt, "stationary" if bs else "streaming", how))
     return out
 
@@ -44,18 +44,18 @@ CASES = [   # (rows, cols, depth, seed, sliced, inner), launches that the case i
     ((5, 7, 40, 25, 10, 4), [("cols", 256, S, "one"), ("cols", 256, S, "runs"), ("plain", 128, S, "one")]),
     ((6, 6, 36, 33, 8, 2), [("plain", 16, S, "one"), ("plain", 64, B, "one"), ("rows", 16, B, "one"), ("rows", 32, B, "one")]),
     ((5, 7, 40, 35, 10, 4), [("cols", 128, S, "runs"), ("plain", 32, B, "one"), ("rows", 128, S, "one"), ("rows", 16, S, "one")]),
-    ((6, 6, 40, 16, 10, 4), [("cols", 32, B, "four"), ("plain", 256, B, "one"), ("plain", 256, B, "four"), ("plain", 256, S, "runs")]),
+    ((6, 6, 40, 16, 10, 4), [("cols", 32, B, "four"), ("plain", 256, B, "one"), ("plain", 256, B, "four"), ("plain", 256, S, "four")]),
     ((6, 6, 36, 37, 10, 4), [("cols", 32, B, "one"), ("cols", 64, S, "one"), ("plain", 64, S, "one")]),
-    ((6, 6, 40, 28, 10, 4), [("cols", 64, S, "runs"), ("plain", 256, S, "one"), ("rows", 32, S, "one")]),
+    ((6, 6, 40, 28, 10, 4), [("cols", 64, S, "four"), ("plain", 256, S, "one"), ("rows", 32, S, "one")]),
     ((6, 6, 36, 25, 10, 4), [("cols", 128, S, "one"), ("plain", 64, S, "runs")]),
     ((6, 6, 36, 2, 8, 2), [("cols", 16, S, "one"), ("rows", 64, S, "one")]),
-    ((5, 6, 40, 15, 8, 2), [("cols", 16, S, "runs"), ("rows", 64, B, "one")]),
+    ((5, 6, 40, 15, 8, 2), [("cols", 16, S, "four"), ("rows", 64, B, "one")]),
     ((5, 7, 40, 14, 8, 2), [("cols", 16, B, "one"), ("rows", 256, S, "one")]),
     ((6, 6, 40, 18, 8, 2), [("cols", 64, B, "one"), ("rows", 256, S, "runs")]),
-    ((6, 6, 40, 12, 8, 2), [("cols", 256, B, "four"), ("rows", 64, S, "runs")]),
+    ((6, 6, 40, 12, 8, 2), [("cols", 256, B, "four"), ("rows", 64, S, "four")]),
     ((5, 6, 40, 9, 8, 2), [("plain", 16, B, "one")]),
-    ((6, 6, 36, 15, 8, 2), [("rows", 16, S, "runs")]),
-    ((5, 6, 40, 8, 8, 2), [("rows", 32, S, "runs")]),
+    ((6, 6, 36, 15, 8, 2), [("rows", 16, S, "four")]),
+    ((5, 6, 40, 8, 8, 2), [("rows", 32, S, "four")]),
     ((5, 7, 40, 18, 10, 4), [("rows", 128, B, "one")]),
     ((5, 7, 40, 5, 8, 2), [("cols", 32, S, "runs")]),
     ((5, 7, 40, 11, 10, 4), [("plain", 128, B, "one")]),
@@ -66,9 +66,13 @@ CASES = [   # (rows, cols, depth, seed, sliced, inner), launches that the case i
     ((5, 6, 40, 20, 8, 2), [("rows", 16, B, "four")]),
     ((6, 6, 36, 9, 8, 2), [("plain", 128, S, "runs")]),
     ((6, 6, 40, 37, 8, 2), [("cols", 64, B, "runs")]),
-    ((6, 6, 40, 10, 10, 4), [("plain", 16, S, "runs")]),
+    ((6, 6, 40, 10, 10, 4), [("plain", 16, S, "four")]),
     ((5, 6, 40, 35, 10, 4), [("plain", 128, B, "four")]),
     ((6, 6, 40, 38, 8, 2), [("cols", 32, B, "runs")]),
+    ((6, 7, 40, 8, 10, 4), [("plain", 256, S, "runs"), ("cols", 128, B, "runs")]),
+    ((5, 7, 40, 5, 10, 4), [("cols", 64, S, "runs")]),
+    ((5, 7, 40, 10, 8, 2), [("cols", 16, S, "runs")]),
+    ((5, 7, 40, 9, 10, 4), [("rows", 32, S, "runs")]),
 ]
 THREE_PARTS = set()   # launches of the three-part runs below
 

@@ -47,12 +47,11 @@ def test_sums_without_rounding_are_exact(seed):
     assert np.array_equal(mantissa * 256, np.round(mantissa * 256))
 
 
-def truncations(chunks, row_tiles):
+def truncations(chunks):
     """Truncations of a sum in the mean, each weighed with the part of the sum that is in by then."""
-    if chunks <= 2 or (chunks == 4 and row_tiles >= 4):   # one group: two large products a chunk
+    if chunks <= 4:                        # one group: two large products a chunk
         return chunks + 0.5
-    run = 4 if chunks >= 8 else 2
-    return {2: 2.5, 4: 8.5}[run]                          # groups of two: also the second's small products
+    return 2.5 if chunks == 8 else 8.5     # runs of one group of two, of two groups of two
 
 
 # sums of 16 to 256 entries on the streaming and the B-stationary form, alone and with a leaf
@@ -67,7 +66,7 @@ def test_long_sums_vs_oracle(seed, inner, longest):
     taken = {int(pr[f]) for pr in pairs for f in ("producer", "consumer")}
     forms += [g for i, g in enumerate(Program(image).gemms) if int(g["nk"]) > 0 and i not in taken]
     assert max(int(g["nk"]) for g in forms) >= longest
-    bound = sum(truncations(max(1, (1 << int(g["nk"])) // 16), 1 << (int(g["nm"]) - 7)) for g in forms) * 2.0 ** -24
+    bound = sum(truncations(max(1, (1 << int(g["nk"])) // 16)) for g in forms) * 2.0 ** -24
     x = cg.random_bitstrings(42, 1, seed + 7)[0]
     terms = p.slice_terms([x]).cpu().numpy()[0].astype(np.complex128)
     ids = np.argsort(-np.abs(terms))[:8]
