@@ -82,10 +82,11 @@ L2_FLUSH_BYTES = 256 << 20
 NCU_TRAFFIC = {}
 # FP32 SIMT peak for the "alu" bound: 152 SMs x 128 FP32 lanes x 2 flops (FMA) x 2.07 GHz
 FP32_SIMT_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
-# the tensor-core contraction spends 24 16-bit flops per complex multiply-add (4 real MACs of
-# the real block form, each as 3 products of two-part fp16 splits) against 8 algorithmic
-# flops, so its algorithmic peak is 8/24 of the bf16 rate (fp16 runs at the same)
-TC_ALGO_PER_BF16 = 8.0 / 24.0
+# the tensor-core contraction spends 24 or 48 16-bit flops per complex multiply-add (4 real MACs
+# of the real block form, each as 3 products of two-part fp16 or 6 of three-part bf16 splits)
+# against 8 algorithmic flops, so its algorithmic peak is 8/24 or 8/48 of the bf16 rate (fp16
+# runs at the same)
+TC_ALGO_PER_BF16 = {2: 8.0 / 24.0, 3: 8.0 / 48.0}
 
 
 def parse(argv=None):
@@ -447,29 +448,30 @@ def run_reference(args, rank, world):
     print(json.dumps(out), flush=True)
 
 
-def kernel_roofline(records, hbm_gbs, bf16_tflops):
+def kernel_roofline(records, hbm_gbs, bf16_tflops, parts):
     """Per-kernel totals of the timed launch log and the dominant kernel's roofline. Each
     launch's roofline time is max(bytes / HBM, flops / compute peak), the compute peak being
-    the FP32 SIMT rate, or the tensor cores' algorithmic rate for the GEMM kernel. Bytes are
-    the contractions' own: a launch that runs two contractions counts the result of the first,
-    which stays on chip, so the fraction of HBM can exceed 1."""
+    the FP32 SIMT rate, or the tensor cores' algorithmic rate for the GEMM kernel (operands in
+    `parts` parts). Bytes are those a launch has to move: of two contractions that run as one the
+    tensor between them, which stays on the chip, is left out."""
     per = {}
     for r in records:
-        peak = bf16_tflops * TC_ALGO_PER_BF16 if r["kernel"] == "gemm_tc_kernel" else FP32_SIMT_TFLOPS
-        t_mem = r["bytes"] / (hbm_gbs * 1e9)
+        peak = bf16_tflops * TC_ALGO_PER_BF16[parts] if r["kernel"] == "gemm_tc_kernel" else FP32_SIMT_TFLOPS
+        t_mem = r["moved"] / (hbm_gbs * 1e9)
         t_cmp = r["flops"] / (peak * 1e12)
-        d = per.setdefault(r["kernel"], {"launches": 0, "ms": 0.0, "bytes": 0.0, "flops": 0.0, "t_mem": 0.0,
+        d = per.setdefault(r["kernel"], {"launches": 0, "ms": 0.0, "bytes": 0.0, "moved": 0.0, "flops": 0.0, "t_mem": 0.0,
                                          "t_cmp": 0.0, "t_roof": 0.0, "peak_tflops": peak})
         d["launches"] += 1
         d["ms"] += r["ms"]
         d["bytes"] += r["bytes"]
+        d["moved"] += r["moved"]
         d["flops"] += r["flops"]
         d["t_mem"] += t_mem
         d["t_cmp"] += t_cmp
         d["t_roof"] += max(t_mem, t_cmp)
     total = sum(d["ms"] for d in per.values()) or 1.0
     summary = {k: {"launches": d["launches"], "ms": d["ms"], "share": d["ms"] / total,
-                   "gbs": d["bytes"] / (d["ms"] / 1e3) / 1e9 if d["ms"] else None,
+                   "gbs": d["moved"] / (d["ms"] / 1e3) / 1e9 if d["ms"] else None,
                    "tflops": d["flops"] / (d["ms"] / 1e3) / 1e12 if d["ms"] else None,
                    "roofline_time_frac": d["t_roof"] / (d["ms"] / 1e3) if d["ms"] else None}
                for k, d in per.items()}
@@ -477,13 +479,14 @@ def kernel_roofline(records, hbm_gbs, bf16_tflops):
     d = per[name]
     sec = d["ms"] / 1e3
     if d["t_mem"] >= d["t_cmp"]:
-        bound, achieved, peak, unit = "hbm", d["bytes"] / sec / 1e9, hbm_gbs, "GB/s"
+        bound, achieved, peak, unit = "hbm", d["moved"] / sec / 1e9, hbm_gbs, "GB/s"
     else:
         bound = "tensor" if name == "gemm_tc_kernel" else "alu"
         achieved, peak, unit = d["flops"] / sec / 1e12, d["peak_tflops"], "TFLOP/s"
     roof = {"bound": bound, "achieved": achieved, "peak": peak, "unit": unit, "frac": achieved / peak,
             "kernel": name, "launches": d["launches"],
             "algorithmic_bytes_per_launch": d["bytes"] / d["launches"],
+            "moved_bytes_per_launch": d["moved"] / d["launches"],
             "algorithmic_flops_per_launch": d["flops"] / d["launches"],
             "mean_launch_ms": d["ms"] / d["launches"],
             "roofline_time_frac": d["t_roof"] / sec}
@@ -662,7 +665,7 @@ def main():
     algo_bytes = (info["grad_bytes_per_amplitude"] if grad else info["bytes_per_amplitude"]) * B
     hbm, bf16, peak_kind = measured_peaks()
     if records:
-        roof, kernels = kernel_roofline(records, hbm, bf16)
+        roof, kernels = kernel_roofline(records, hbm, bf16, plan.step_traffic(0)[1] or 3)
     else:   # gradient and slice-sharded runs: the whole step against the HBM roofline
         if grad:
             kname = "grad_smem_kernel" if 0 < info["grad_smem_bytes"] <= 232448 else "grad_program_kernel"

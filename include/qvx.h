@@ -340,11 +340,17 @@ typedef struct {
     double bytes;          /* algorithmic bytes of the launch: each operand read and each
                               output written once (complex64; 32-byte exact partials), summed
                               over the contractions it runs, also where a tensor between two of
-                              them stays on the chip */
+                              them stays on the chip (qvx_step_traffic leaves it out) */
     float ms;              /* device time between CUDA events recorded on the call's stream
                               just before and just after the launch */
     int32_t pad;
 } qvx_launch_record;
+
+/* Bytes that the launch recorded for program step `step` moves per work item at least: as the
+ * record's, but of two contractions that run as one without the tensor between them.
+ * parts (may be NULL): the 16-bit parts of a tensor-core operand in this plan, 2 or 3 (3 or 6
+ * products per multiply-add); 0 without tensor cores. */
+qvx_status qvx_step_traffic(const qvx_plan *plan, int32_t step, double *bytes, int32_t *parts);
 
 /* qvx_amplitude_slices with a CUDA event recorded on `stream` just before and just after
  * every kernel launch, for measuring each kernel against its roofline. The launches are

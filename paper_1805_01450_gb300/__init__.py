@@ -77,7 +77,8 @@ EXPORTED = ("qvx_plan_opts_default", "qvx_graph_export", "qvx_plan_create", "qvx
             "qvx_amplitude", "qvx_amplitude_slices", "qvx_slice_terms", "qvx_workspace_status",
             "qvx_last_error", "qvx_amplitude_noalloc", "qvx_amplitude_grad", "qvx_amplitude_host",
             "qvx_selftest_wait_timeout", "qvx_kernel_launches", "qvx_noalloc_status", "qvx_amplitude_profiled",
-            "qvx_profile_read", "qvx_kernel_name", "qvx_selftest_fused_timeout", "qvx_bits_check", "qvx_bits_result")
+            "qvx_profile_read", "qvx_kernel_name", "qvx_selftest_fused_timeout", "qvx_bits_check", "qvx_bits_result",
+            "qvx_step_traffic")
 
 
 def lib():
@@ -117,6 +118,7 @@ def lib():
         "qvx_selftest_fused_timeout": (ctypes.c_int, [P, P, i64, P, P, ctypes.c_size_t, P]),
         "qvx_bits_check": (ctypes.c_int, [P, P, i64, P, ctypes.POINTER(i64)]),
         "qvx_bits_result": (ctypes.c_int, [i64]),
+        "qvx_step_traffic": (ctypes.c_int, [P, i32, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(i32)]),
     }
     for name, (res, args) in sig.items():
         f = getattr(L, name)
@@ -495,7 +497,8 @@ class Plan:
 
     def read_profile(self):
         """The launch log of amplitude_profiled calls since the last read, in issue order: a
-        list of dicts (kernel name, step, items, algorithmic flops and bytes, ms); empties it."""
+        list of dicts (kernel name, step, items, algorithmic flops and bytes, bytes without the
+        tensors that merged steps keep on the chip, ms); empties it."""
         L = lib()
         n = ctypes.c_int64()
         _check(L.qvx_profile_read(self._h, None, 0, ctypes.byref(n)))   # the count; the log stays
@@ -503,7 +506,15 @@ class Plan:
         recs = (LaunchRecord * cap)()
         _check(L.qvx_profile_read(self._h, recs, cap, ctypes.byref(n)))
         return [dict(kernel=L.qvx_kernel_name(r.kernel).decode(), step=r.step, items=r.items, flops=r.flops,
-                     bytes=r.bytes, ms=r.ms) for r in recs[:min(n.value, cap)]]
+                     bytes=r.bytes, moved=self.step_traffic(r.step)[0] * r.items if r.step >= 0 else r.bytes, ms=r.ms)
+                for r in recs[:min(n.value, cap)]]
+
+    def step_traffic(self, step):
+        """(bytes that the launch of a program step moves per work item at least, 16-bit parts of a
+        tensor-core operand or 0)."""
+        b, parts = ctypes.c_double(), ctypes.c_int32()
+        _check(lib().qvx_step_traffic(self._h, step, ctypes.byref(b), ctypes.byref(parts)))
+        return b.value, parts.value
 
     def check_status(self, workspace, stream=None):
         """Synchronises and raises if a kernel set the workspace's device status word."""

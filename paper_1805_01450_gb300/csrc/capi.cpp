@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -606,6 +607,25 @@ qvx_status qvx_profile_read(qvx_plan *plan, qvx_launch_record *records, int64_t 
         if ((int64_t)i < cap) records[i] = log[i];
     }
     if (n_records) *n_records = (int64_t)log.size();
+    return QVX_OK;
+}
+
+qvx_status qvx_step_traffic(const qvx_plan *plan, int32_t step, double *bytes, int32_t *parts) {
+    if (!plan || !bytes) return fail(QVX_EINVAL, "null argument");
+    const qvx::Plan &p = plan->p;
+    if (step < 0 || (size_t)step >= p.steps.size()) return fail(QVX_EINVAL, "no such step");
+    double fl, first = 0, second = 0;
+    qvx::step_cost(p, (size_t)step, &fl, &first);
+    int inner = -1;   // the tensor that stays on the chip
+    if (!p.pairs.empty() && p.pairs[step].consumer >= 0) {
+        qvx::step_cost(p, (size_t)p.pairs[step].consumer, &fl, &second);
+        inner = p.steps[step].c;
+    } else if (!p.reduces.empty() && p.reduces[step].producer >= 0) {
+        qvx::step_cost(p, (size_t)p.reduces[step].producer, &fl, &second);
+        inner = p.steps[p.reduces[step].producer].c;
+    }
+    *bytes = first + second - (inner < 0 ? 0.0 : 16.0 * std::ldexp(1.0, (int)p.tensors[inner].modes.size()));
+    if (parts) *parts = p.gemm.empty() ? 0 : (p.fp16_split ? 2 : 3);
     return QVX_OK;
 }
 
