@@ -64,11 +64,11 @@ __host__ __device__ constexpr uint32_t region_bytes(uint32_t rows) { return rows
 // real columns of a tile are all its Re columns, then all its Im columns, so part 0 of the
 // right factor is the two blocks [Br][Bi] and part 1 the two blocks [-Bi][Br]: a descriptor
 // that starts one block earlier, and Br is stored once. With Re and Im interleaved column by
-// column a level took four blocks: 48 instead of 36 KB of stores per chunk of a 256-column
-// tile, whose loop is bound by shared-memory traffic. Together with one barrier arrival per
-// warp (warp_arrive) the streaming steps of a 64-qubit circuit went from 2.90 to 2.56 ms (64
-// summed entries, 190 -> 215 algorithmic TFLOP/s) and from 1.52 to 1.21 ms (32 summed, 128
-// columns).
+// column a level took four blocks: with three parts 48 instead of 36 KB of stores per chunk of a
+// 256-column tile, whose loop is bound by shared-memory traffic. Together with one barrier arrival
+// per warp (warp_arrive) the streaming steps of a 64-qubit circuit, with three parts, went from 2.90
+// to 2.56 ms (64 summed entries, 190 -> 215 algorithmic TFLOP/s) and from 1.52 to 1.21 ms (32
+// summed, 128 columns).
 __host__ __device__ constexpr uint32_t b_block_bytes(uint32_t nt) { return region_bytes(nt / 2u); }
 template <int kParts>
 __host__ __device__ constexpr uint32_t b_chunk_bytes(uint32_t nt) { return 3u * kParts * b_block_bytes(nt); }

@@ -483,8 +483,9 @@ __device__ __forceinline__ void run_lane_work(const LaneWork &w) {
 // phase ahead, so a phase's critical path is its operand loads, FMAs, store and barrier.
 // WARPS: most warps of a CTA. 16 get up to 128 registers a thread and two entries with eight
 // summed entries at a time; 24 and 32 (fused_shape says when) get 80 and 64 and take such entries
-// one at a time. Spilled registers cost more than the warps give: with 64 registers for 16 warps
-// 7 amplitudes of a 6 x 7 grid at depth 26 took 94 us, with 128 they take 73 (88 with generic loads).
+// one at a time; the 32-warp kernels still spill 68 and 120 bytes. Spilled registers cost more than
+// the warps give: with 64 registers for 16 warps 7 amplitudes of a 6 x 7 grid at depth 26 took 94 us,
+// with 128 they take 73 (88 with generic loads).
 template <bool STAGED, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, 1) fused_program_kernel(LaunchArgs a, int warps_per_item) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -813,8 +814,8 @@ __device__ __forceinline__ void tile_entries(const RegTileStep &rs, const float2
 // maps of the tile index are tabulated there for its low and next eight bits (output, A and B
 // offset), so a tile costs two table reads instead of some fifteen run moves. What bounds the
 // kernel is instruction issue. 16 amplitudes of a 49-qubit circuit (8 sliced variables, 4096
-// work items): 8.84 ms with one thread per entry, 2.57 ms; three CTAs per SM (80 registers) ran
-// 4 % faster than four (64, spilled).
+// work items): 8.84 ms with one thread per entry, 2.57 ms; three CTAs per SM (80 registers, 140
+// bytes spilled) ran 4 % faster than four (64, more spilled).
 constexpr uint32_t kStepBits = 1024;
 struct PersistentSmem {
     RegTileStep rt;
@@ -1728,9 +1729,11 @@ bool fused_shape(const DevProgram *h, uint64_t arena_elems, int warps_per_item, 
     // Warps that run at a time: one CTA fits an SM when the program is staged, and a phase is a
     // chain of shared-memory latencies and a barrier (8 warps issued in 26 % of the cycles), so a
     // CTA takes 24 warps, or 32 in groups of 8 and 16, of which 24 hold fewer. 64 amplitudes of
-    // the 6 x 6 grid at depth 25, groups of 4: 417 us with 8 warps, 302 with 16, 291 with 24, 323
-    // with 32; groups of 8: 629 / 766 / 598 / 575 us; of 16 (6 amplitudes): 140 us with 16 or 24,
-    // 117 with 32. (A group of several warps has a named barrier of its own: 1 to 15.)
+    // the 6 x 6 grid at depth 25, groups of 4: 299 us with 8 warps, 192 with 16, 154 with 24, 156
+    // with 32; 50 in groups of 8: 384 / 244 / 193 / 177 us; in groups of 16: 402 with 16 or 24, 302
+    // with 32. (With fewer open slices a group of 16 gains less: 3 amplitudes of 512 work items each
+    // 88 us with one at a time in two CTAs, 96 with two in one; 50 amplitudes 1251 and 1186. A group
+    // of several warps has a named barrier of its own: 1 to 15.)
     const int by_warps = std::min((warps_per_item >= 8 ? kFusedWarps : 24) / warps_per_item, warps_per_item > 1 ? 15 : kFusedGroups);
     *max_ipc = (int)std::max<size_t>(1, std::min<size_t>(by_warps, (kBudget - sh) / *group));
     return true;
@@ -1770,8 +1773,9 @@ cudaError_t launch_splitk_step(const LaunchArgs &a, uint32_t step, int64_t item_
 // Form of a launch over `blocks` blocks of tiles; *per_cta blocks of one item go to a CTA. max: the
 // output's largest entries are wanted. Timed on 260 steps of 6 x 6 to 8 x 8 circuits (2^8 to 2^24
 // tiles an item, 0 to 8 summed modes), the other form against the one taken:
-//  - with too few blocks for two per CTA: 1.15 x slower up to four summed entries (242 items of a
-//    6 x 7 grid at depth 26: 36.6 us a step against 41.1), flat from eight on 1.28 x slower;
+//  - with too few blocks for two per CTA: blocks up to 1.15 x slower (242 items of a 6 x 7 grid at
+//    depth 26: 36.6 us a step against 41.1), flat 1.05 to 1.36 x on 4 x 4 tiles from eight summed
+//    entries on;
 //  - 4 x 4 tiles: with a second operand 2^6 times larger than the first, flat 1.1 to 1.9 x slower
 //    than a block-uniform base, plain pointers 1.1 to 1.2 x; with a larger first operand flat is
 //    the faster one by up to 8 %, otherwise blocks are by up to 16 %;
@@ -1795,7 +1799,7 @@ static TileForm tile_form(const RegTileStep &rs, uint64_t blocks, bool max, uint
     const uint32_t most = std::min(kMaxTileBlocks, 1u << (rs.nt - RegTileShape<RM, RN>::kThreadBits));
     uint32_t n = 1u;
     while (n < most && blocks / (2u * n) >= kMinTileCtas) n *= 2u;
-    if (n == 1u) return nk < 3 ? kTilesFlat : kTilesBlocks;
+    if (n == 1u) return RM == 2 && RN == 2 && nk >= 3 ? kTilesBlocks : kTilesFlat;
     const bool merges = max && RM == 1 && RN == 2;
     bool flat;
     if (RM == 2 && RN == 2) flat = rank_a - rank_b >= 6;

@@ -74,3 +74,24 @@ def test_long_sums_vs_oracle(seed, inner, longest):
     err = np.linalg.norm(terms[ids] - ref) / np.linalg.norm(ref)
     # every step's truncation in one direction, and 2^-20 for the roundings of the program's FP32 sums
     assert err < bound + 2.0 ** -20
+
+
+# gates whose small entry is a sixteenth or less of the large one: seven of them put entries of a
+# tensor 2^-28 below its largest. The error counts against the terms themselves
+@pytest.mark.parametrize("small", (1 / 16, 1 / 30, 1 / 200))
+@pytest.mark.parametrize("r,c_,d,seed,k,inner", [(6, 6, 40, 7066, 8, 2), (5, 7, 40, 25, 10, 4)])
+def test_unequal_gates_relative_to_the_terms(r, c_, d, seed, k, inner, small):
+    c = cg.grid_circuit(r, c_, d, seed)
+    roots = [i for i, g in enumerate(c.gates) if g.kind in (cg.SQRT_X, cg.SQRT_Y)]
+    large = (1.0 - small * small) ** 0.5
+    for i in roots[len(roots) // 4::max(1, len(roots) // 12)][:7]:
+        c.gates[i] = cg.Gate(cg.U1, c.gates[i].q0, u=(large, 0.0, -small, 0.0, small, 0.0, large, 0.0), cycle=c.gates[i].cycle)
+    base = q.Plan(cg.grid_circuit(r, c_, d, seed), n_slices=k, inner_slices=inner, engine="stepwise", tensor_cores=True,
+                  order_restarts=2)
+    p = q.Plan(c, order=base.order, slices=base.slices, inner_slices=inner, engine="stepwise", tensor_cores=True)
+    assert p.info["n_gemm_steps"] >= 1 and p.step_traffic(0)[1] == 3
+    x = cg.random_bitstrings(r * c_, 1, seed + 1)[0]
+    terms = p.slice_terms([x]).cpu().numpy()[0].astype(np.complex128)
+    ids = np.argsort(-np.abs(terms))[:6]
+    ref = VE.slice_terms(c, x, p.order, p.slices, slice_ids=ids)
+    assert np.linalg.norm(terms[ids] - ref) < 1e-5 * np.linalg.norm(ref)
