@@ -229,6 +229,11 @@ qvx_status qvx_amplitude(qvx_plan *plan, const uint64_t *bitstrings_dev, int64_t
 qvx_status qvx_amplitude_host(qvx_plan *plan, const uint64_t *bitstrings_host, int64_t batch, double *amps_host,
                               void *workspace_dev, size_t workspace_bytes, void *stream);
 
+/* Writes n words of host memory to device memory in stream order: the words may be freed or
+ * overwritten as soon as the call returns, and nothing waits for the stream (each 256 words are a
+ * kernel's parameters). Not during stream capture (QVX_ECUDA). */
+qvx_status qvx_words_upload(const uint64_t *words_host, int64_t n, uint64_t *words_dev, void *stream);
+
 /* Checks device bitstrings without waiting for the work already in the stream: qvx_bits_check
  * enqueues one small kernel that looks for bits at or above n_qubits and returns a ticket;
  * qvx_bits_result waits for that kernel only (not for anything enqueued after it), gives the

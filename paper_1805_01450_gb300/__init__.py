@@ -78,7 +78,7 @@ EXPORTED = ("qvx_plan_opts_default", "qvx_graph_export", "qvx_plan_create", "qvx
             "qvx_last_error", "qvx_amplitude_noalloc", "qvx_amplitude_grad", "qvx_amplitude_host",
             "qvx_selftest_wait_timeout", "qvx_kernel_launches", "qvx_noalloc_status", "qvx_amplitude_profiled",
             "qvx_profile_read", "qvx_kernel_name", "qvx_selftest_fused_timeout", "qvx_bits_check", "qvx_bits_result",
-            "qvx_step_traffic")
+            "qvx_step_traffic", "qvx_words_upload")
 
 
 def lib():
@@ -118,6 +118,7 @@ def lib():
         "qvx_selftest_fused_timeout": (ctypes.c_int, [P, P, i64, P, P, ctypes.c_size_t, P]),
         "qvx_bits_check": (ctypes.c_int, [P, P, i64, P, ctypes.POINTER(i64)]),
         "qvx_bits_result": (ctypes.c_int, [i64]),
+        "qvx_words_upload": (ctypes.c_int, [P, i64, P, P]),
         "qvx_step_traffic": (ctypes.c_int, [P, i32, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(i32)]),
     }
     for name, (res, args) in sig.items():
@@ -355,13 +356,17 @@ class Plan:
             if validate:
                 self._check_host_bits(bitstrings)
             if bitstrings and stream.value == (_current_stream() or None):
-                # from page-locked memory without waiting for the stream: torch gives the block to
-                # nobody else before the copy is through. A capture would record the copy and read
-                # the block again at every replay
+                # without waiting for the stream: a few words go as kernel parameters, more from
+                # page-locked memory, whose block torch gives to nobody else before the copy is
+                # through. A capture would record the copy and read the block again at every replay
+                words = bitstring_words(bitstrings, self.words)
+                if len(words) <= 256:
+                    bits = torch.empty(len(words), dtype=torch.int64, device="cuda")
+                    _check(lib().qvx_words_upload((ctypes.c_int64 * len(words))(*words), len(words), bits.data_ptr(), stream))
+                    return bits, -1
                 if torch.cuda.is_current_stream_capturing():
                     raise QvxError(QVX_ECUDA, "bitstrings cannot be uploaded during stream capture")
-                words = torch.tensor(bitstring_words(bitstrings, self.words), dtype=torch.int64, pin_memory=True)
-                return words.to("cuda", non_blocking=True), -1
+                return torch.tensor(words, dtype=torch.int64, pin_memory=True).to("cuda", non_blocking=True), -1
             return self._bits(bitstrings), -1
         bits = self._bits(bitstrings)
         if validate:

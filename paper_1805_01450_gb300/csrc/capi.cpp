@@ -845,6 +845,20 @@ void give_ticket(int64_t i) {
 
 extern "C" {
 
+qvx_status qvx_words_upload(const uint64_t *words_host, int64_t n, uint64_t *words_dev, void *stream) {
+    if (n < 0 || (n > 0 && (!words_host || !words_dev))) return fail(QVX_EINVAL, "bad argument");
+    if (n == 0) return QVX_OK;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(st, &cap)) != cudaSuccess) return cuda_fail(e, "capture query");
+    if (cap != cudaStreamCaptureStatusNone) return fail(QVX_ECUDA, "bitstrings cannot be uploaded during stream capture");
+    for (int64_t i = 0; i < n; i += qvx::kWordsAtOnce)
+        if ((e = qvx::launch_words(words_host + i, (int)std::min<int64_t>(qvx::kWordsAtOnce, n - i), words_dev + i, st)) != cudaSuccess)
+            return cuda_fail(e, "word upload");
+    return QVX_OK;
+}
+
 qvx_status qvx_bits_check(const qvx_plan *plan, const uint64_t *bitstrings_dev, int64_t batch, void *stream, int64_t *ticket) {
     if (!plan || !ticket || batch < 0 || (batch > 0 && !bitstrings_dev)) return fail(QVX_EINVAL, "bad argument");
     *ticket = -1;

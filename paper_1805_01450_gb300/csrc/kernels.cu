@@ -1548,6 +1548,15 @@ __global__ void check_bits_kernel(const uint64_t *bitstrings, int64_t n, uint32_
     if (bad) *reinterpret_cast<volatile unsigned *>(flag) = 1u;
 }
 
+// Words that a launch carries as its parameters: they are copied when it is enqueued, so the
+// caller's memory is free at once, and no copy waits for the stream.
+struct WordBlock {
+    uint64_t w[kWordsAtOnce];
+};
+__global__ void words_kernel(WordBlock b, int n, uint64_t *out) {
+    if ((int)threadIdx.x < n) out[threadIdx.x] = b.w[threadIdx.x];
+}
+
 // Self-test of the bounded waits: a grid barrier for two CTAs run by one, and an mbarrier
 // whose phase never completes. Each wait must give up after `polls` polls; the kernel
 // records which did in out[0] (barrier) and out[1] (mbarrier) and sets the status word.
@@ -1592,6 +1601,14 @@ cudaError_t launch_check_bits(const uint64_t *bitstrings, int64_t batch, uint32_
     const int64_t n = batch * words;
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 64));
     check_bits_kernel<<<blocks, 256, 0, s>>>(bitstrings, n, words, valid_lo, valid_hi, flag);
+    return counted(cudaGetLastError());
+}
+
+cudaError_t launch_words(const uint64_t *words, int n, uint64_t *out, cudaStream_t s) {
+    WordBlock b;
+    std::copy(words, words + n, b.w);
+    std::fill(b.w + n, b.w + kWordsAtOnce, 0ull);
+    words_kernel<<<1, kWordsAtOnce, 0, s>>>(b, n, out);
     return counted(cudaGetLastError());
 }
 

@@ -147,6 +147,9 @@ cudaError_t launch_reduce_step(const LaunchArgs &a, const ReduceStep &r, const G
 // valid_hi (word 1).
 cudaError_t launch_check_bits(const uint64_t *bitstrings, int64_t batch, uint32_t words, uint64_t valid_lo,
                               uint64_t valid_hi, unsigned *flag, cudaStream_t s);
+// Up to kWordsAtOnce words from the host to device memory, as parameters of a kernel.
+constexpr int kWordsAtOnce = 256;
+cudaError_t launch_words(const uint64_t *words, int n, uint64_t *out, cudaStream_t s);
 // Self-test of the bounded waits (grid barrier and mbarrier that can never complete).
 cudaError_t launch_wait_selftest(unsigned *words, unsigned *status, uint32_t polls, unsigned *out, cudaStream_t s);
 

@@ -16,10 +16,11 @@ def _cuda():
         pytest.skip("no CUDA device")
 
 
-@pytest.mark.parametrize("rows,cols", [(3, 3), (8, 9)])
-def test_copies_without_a_wait_are_page_locked(monkeypatch, rows, cols):
+# up to 256 words go as kernel parameters
+@pytest.mark.parametrize("rows,cols,batch", [(3, 3, 5), (8, 9, 5), (8, 9, 128), (8, 9, 129), (3, 3, 256), (3, 3, 257)])
+def test_copies_without_a_wait_are_page_locked(monkeypatch, rows, cols, batch):
     p = q.Plan(cg.grid_circuit(rows, cols, 4, 1))
-    xs = cg.random_bitstrings(rows * cols, 5, 2)
+    xs = cg.random_bitstrings(rows * cols, batch, 2)
     want = p.amplitude(torch.tensor(q.bitstring_words(xs, p.words), dtype=torch.int64, device="cuda"))
     unwaited, plain = [], torch.Tensor.to
 
@@ -32,21 +33,32 @@ def test_copies_without_a_wait_are_page_locked(monkeypatch, rows, cols):
     got = [p.amplitude(xs) for _ in range(50)]   # many in flight, each with its own words
     other = [p.amplitude([x ^ 1 for x in xs]) for _ in range(50)]
     monkeypatch.undo()
-    assert unwaited and all(unwaited)
+    assert all(unwaited) and bool(unwaited) == (batch * p.words > 256)
     assert all(torch.equal(g, want) for g in got)
     assert all(torch.equal(o, other[0]) for o in other) and not torch.equal(other[0], want)
 
 
-def test_no_upload_during_capture():
+def test_uploaded_words():
+    for n in (1, 255, 256, 257, 1000):
+        words = torch.randint(-(1 << 62), 1 << 62, (n,), dtype=torch.int64)
+        out = torch.full((n + 1,), 7, dtype=torch.int64, device="cuda")
+        host = words.clone()
+        assert q.lib().qvx_words_upload(host.data_ptr(), n, out.data_ptr(), torch.cuda.current_stream().cuda_stream) == q.QVX_OK
+        host.zero_()   # free to the caller at once
+        assert torch.equal(out[:n].cpu(), words) and int(out[n]) == 7
+
+
+@pytest.mark.parametrize("count", [2, 300])
+def test_no_upload_during_capture(count):
     p = q.Plan(cg.grid_circuit(3, 3, 4, 1))
     bits = torch.tensor([1, 2], dtype=torch.int64, device="cuda")
     want = p.amplitude(bits)
-    ws = p.workspace(2)
+    ws = p.workspace(count)
     for validate in (True, False):
         g = torch.cuda.CUDAGraph()
         with pytest.raises(q.QvxError):
             with torch.cuda.graph(g):
-                p.amplitude([1, 2], workspace=ws, validate=validate)
+                p.amplitude([1, 2] * (count // 2), workspace=ws, validate=validate)
     replay, out = p.graphed(bits)
     replay()
     torch.cuda.synchronize()
